@@ -234,7 +234,23 @@ extern "C" int sub_create(const sub_params* p, void* stream, sub_ctx** out) {
     rc = dalloc(c, w.p, w.b);
     if (rc) return fail(rc);
   }
-  c->rep.nbins = n < kAccReplicaBins ? n : kAccReplicaBins;
+  {
+    // the tree's node sums take the end of the replica buffer (0.4 of its 256 bytes per bin),
+    // so a context's memory does not depend on them
+    Tree& tr = c->tree;
+    int nodes = 0;
+    for (int l = 0; l < kTreeLevels; ++l) {
+      tr.n[l] = (int)(n >> (5 * (l + 1)));
+      tr.off[l] = nodes;
+      nodes = (nodes + tr.n[l] + 3) & ~3;  // a level starts on 16 bytes
+    }
+    const size_t bytes = (size_t)kAccReplicas * (n < kAccReplicaBins ? n : kAccReplicaBins) * 16;
+    const size_t sums = (size_t)nodes * (sizeof(double) + sizeof(float));
+    c->rep.nbins = (long long)((bytes - sums) / ((size_t)kAccReplicas * 16));
+    double* gsum = (double*)(c->rep.w + (size_t)kAccReplicas * c->rep.nbins * 2);
+    tr.gsum = gsum;
+    tr.h = (float*)(gsum + nodes);
+  }
   if (p->estimator != SUB_MEAN) {
     rc = dalloc(c, (void**)&c->skey, (size_t)ncell * 8);
     if (!rc) rc = dalloc(c, (void**)&c->srank, (size_t)ncell * 2);
@@ -252,6 +268,10 @@ extern "C" int sub_create(const sub_params* p, void* stream, sub_ctx** out) {
   // FP32 normal range over any band whose S_instr spans less than 2^60.
   if (e == cudaSuccess) e = cudaMemsetAsync(&c->rs->max_p_bits, 0, 8, c->stream);
   if (e == cudaSuccess) launch_max_bits(c->S, n, &c->rs->max_p_bits, c->stream);
+  // and the largest gq, for the units of the tree's nodes (any scratch word of the state)
+  if (e == cudaSuccess) e = cudaMemsetAsync(&c->rs->relchg_bits, 0, 8, c->stream);
+  if (e == cudaSuccess) launch_max_bits(c->gq, n, &c->rs->relchg_bits, c->stream);
+  if (e == cudaSuccess) launch_tree_sums(c->gq, c->tree, const_cast<double*>(c->tree.gsum), c->stream);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(c->h_rs, c->rs, sizeof(RunState), cudaMemcpyDeviceToHost, c->stream);
@@ -263,6 +283,13 @@ extern "C" int sub_create(const sub_params* p, void* stream, sub_ctx** out) {
     std::memcpy(&smax, &b, 8);
     int ex = smax > 0.0 ? std::ilogb(smax) : 0;
     c->plan.key_scale = std::ldexp(1.0, 59 - ex);
+    double gmax;
+    b = c->h_rs->relchg_bits;
+    std::memcpy(&gmax, &b, 8);
+    // an infinite scale sends every sweep bin by bin
+    const bool fin = std::isfinite(gmax) && gmax > 0.0 && std::ilogb(gmax) < 1000;
+    c->tree.g = fin ? std::ilogb(gmax) + 1 : 0;
+    c->tree.scale = fin ? std::ldexp(1.0, c->tree.g) : (double)INFINITY;
   }
   *out = c;
   return SUB_OK;
@@ -472,6 +499,7 @@ static Tables tables_of(const sub_ctx* c) {
   t.gq = c->gq;
   t.Gf = c->Gf;
   t.invSf = c->invSf;
+  t.tree = c->tree;
   return t;
 }
 
@@ -536,6 +564,26 @@ static cudaError_t enqueue_pre(sub_ctx* c, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// Estimator inputs: the run's spectrum, or a plain array.
+static SpecIn spectrum_of(const sub_ctx* c) {
+  SpecIn in;
+  in.acc = c->acc;
+  in.S = c->S;
+  in.x = nullptr;
+  in.gq = c->gq;
+  in.nb = c->grid.nb;
+  in.g = c->tree.g;
+  in.tree = &c->rs->tree;
+  return in;
+}
+static SpecIn array_of(const sub_ctx* c, const double* x) {
+  SpecIn in = spectrum_of(c);
+  in.acc = nullptr;
+  in.x = x;
+  in.tree = nullptr;
+  return in;
+}
+
 // One estimate of S_gal from `in` into c->Sg (and inv_f when with_inv).  With track, only
 // the chunks whose inputs changed since the previous iteration are recomputed.
 // Chunks around a changed chunk whose S_gal changes: the median and the mean read one chunk
@@ -554,6 +602,9 @@ static void enqueue_estimate(sub_ctx* c, cudaStream_t st, SpecIn in, int rtol_on
   o.invSf = c->invSf;
   o.rtol_on = rtol_on;
   o.rs = c->rs;
+  o.Gf = c->Gf;
+  o.tree = c->tree;
+  if (!with_inv) o.tree.h = nullptr;
   switch (c->p.estimator) {
     case SUB_MEAN: {
       { KTimer t(c, st, SUB_K_PREFIX); launch_chunk_prefix(in, n, pl, c->pre_lo, c->pre_hi, c->sig, c->uflow, c->P, d, 0, st); }
@@ -570,10 +621,8 @@ static void enqueue_estimate(sub_ctx* c, cudaStream_t st, SpecIn in, int rtol_on
       om.out = c->M;
       om.inv_f = nullptr;
       om.rtol_on = 0;
-      SpecIn mi;
-      mi.acc = nullptr;
-      mi.S = nullptr;
-      mi.x = c->M;
+      om.tree.h = nullptr;
+      const SpecIn mi = array_of(c, c->M);
       { KTimer t(c, st, SUB_K_SORT); launch_chunk_sort(in, n, pl, c->skey, c->srank, d, st); }
       { KTimer t(c, st, SUB_K_MEDIAN); launch_running_median(c->skey, c->srank, n, pl, om, d, st); }
       { KTimer t(c, st, SUB_K_PREFIX); launch_chunk_prefix(mi, n, pl, c->pre_lo, c->pre_hi, c->sig, c->uflow, nullptr, d, 1, st); }
@@ -586,11 +635,7 @@ static void enqueue_estimate(sub_ctx* c, cudaStream_t st, SpecIn in, int rtol_on
 static cudaError_t enqueue_body(sub_ctx* c, cudaStream_t st, unsigned long long handle, int use_cond) {
   const int rtol_on = c->p.conv_rtol > 0.0 ? 1 : 0;
   RunState* rs = c->rs;
-  SpecIn in;
-  in.acc = c->acc;
-  in.S = c->S;
-  in.x = nullptr;
-  enqueue_estimate(c, st, in, rtol_on, true, true);
+  enqueue_estimate(c, st, spectrum_of(c), rtol_on, true, true);
   double th2 = c->p.rho_th * c->p.rho_th;
   {
     KTimer t(c, st, SUB_K_SNR);
@@ -856,11 +901,7 @@ extern "C" int sub_estimate(sub_ctx* c, const double* P, double* out, int64_t n,
   double* in_buf = c->estimate_in;
   CU(cudaMemcpyAsync(in_buf, P, (size_t)n * 8, k_in, st), c);
   CU(cudaMemsetAsync(c->rs, 0, sizeof(RunState), st), c);
-  SpecIn in;
-  in.acc = nullptr;
-  in.S = nullptr;
-  in.x = in_buf;
-  enqueue_estimate(c, st, in, 0, false, false);
+  enqueue_estimate(c, st, array_of(c, in_buf), 0, false, false);
   CU(cudaGetLastError(), c);
   CU(cudaMemcpyAsync(out, c->Sg, (size_t)n * 8, k_out, st), c);
   CU(cudaStreamSynchronize(st), c);
@@ -934,7 +975,7 @@ extern "C" int sub_get_power(sub_ctx* c, double* P, int64_t n, int where) {
   if (n != c->grid.nb || !P) { set_err(c, "n must equal n_bins"); return SUB_EINVAL; }
   if (where != SUB_HOST && where != SUB_DEVICE) { set_err(c, "bad where"); return SUB_EINVAL; }
   if (!c->ran) { set_err(c, "no run yet"); return SUB_ESTATE; }
-  launch_power_out(c->acc, c->S, n, c->estimate_in, c->stream);
+  launch_power_out(spectrum_of(c), n, c->estimate_in, c->stream);
   CU(cudaGetLastError(), c);
   CU(cudaMemcpyAsync(P, c->estimate_in, (size_t)n * 8,
                      where == SUB_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, c->stream), c);

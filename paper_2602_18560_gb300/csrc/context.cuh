@@ -40,6 +40,7 @@ struct sub_ctx {
   // spectrum and smoothing buffers
   unsigned long long* acc = nullptr;  // 4 words per bin
   AccReplicas rep = {nullptr, 0};     // private copies of the first bins (catalog pass)
+  gbsub::Tree tree = {};              // node sums of the long sweeps (behind the copies)
   double *P = nullptr, *M = nullptr, *Sg = nullptr;
   double* estimate_in = nullptr;  // input copy of sub_estimate
   double* cg = nullptr;           // coarse graining: [S | f | counts | edges] of cg_cap bins

@@ -20,6 +20,8 @@
 // bits of the doubles, window sums are integer, and the SNR test is screened in FP32 with
 // a proven error margin (exact FP64 recomputation inside the margin).
 
+#include <cstring>
+
 #include <cuda_runtime.h>
 #include <cuda_device_runtime_api.h>
 
@@ -120,33 +122,158 @@ __device__ __forceinline__ void sub_parts(unsigned long long* acc, long long j, 
   if (c2) atomicAdd(a + 2, (u64)(0ull - c2));
 }
 
-// Estimator input of bin j: P_j = S_j Q_j 2^-96, or x[j].
-__device__ __forceinline__ double spec_value(const SpecIn& in, long long j) {
-  if (in.acc) {
+// ---------------------------------------------------------------- the tree of bins
+// Words of a node: three of them, as a bin's, in the padding words of the node's first bins
+// (level 1 in bins 0-2, level 2 in 3-5, level 3 in 6-8: a complete node has at least 32 bins).
+// They need no memory and no clearing of their own.
+__device__ __forceinline__ size_t node_word(int level, long long i, int w) {
+  return 4 * (size_t)((i << (5 * level)) + 3 * (level - 1) + w) + 3;
+}
+
+// What the nodes above bin j add to its Q (units of 2^-64 S_instr): the sum N of their words,
+// c in units of 2^(32 - g), times gq_j.  The top 64 bits of N times gq's mantissa, truncated:
+// within 2^-62 of the exact product, or one unit.
+__device__ __noinline__ U128 tree_units(const unsigned long long* __restrict__ acc, long long j,
+                                        long long nb, double gq, int g) {
+  U128 N{0ull, 0ull};
+#pragma unroll
+  for (int l = 1; l <= kTreeLevels; ++l) {
+    const long long i = j >> (5 * l);
+    if (((i + 1) << (5 * l)) <= nb) {  // an incomplete node takes nothing, and has no words
+      const unsigned long long* a = acc + node_word(l, i, 0);
+      N = u128_add(N, q_combine3(a[0], a[4], a[8]));
+    }
+  }
+  U128 r{0ull, 0ull};
+  if (u128_is_zero(N)) return r;
+  const int lz = N.hi ? __clzll((i64)N.hi) : 64 + __clzll((i64)N.lo);
+  // top in [2^63, 2^64), N = top 2^(64 - lz) up to the bits dropped
+  const u64 top = lz >= 64 ? N.lo << (lz - 64)
+                           : (lz ? (N.hi << lz) | (N.lo >> (64 - lz)) : N.hi);
+  const u64 bg = (u64)__double_as_longlong(gq);
+  const int eg = (int)(bg >> 52) & 0x7FF;
+  if (eg == 0) return r;
+  const u64 mg = ((bg & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << 11;
+  const u64 p = __umul64hi(top, mg);  // N gq 2^-g = p 2^sh
+  const int sh = 64 + (64 - lz) + (eg - 1086) - g;
+  if (sh >= 64) {
+    r.hi = p << (sh - 64);
+  } else if (sh > 0) {
+    r.lo = p << sh;
+    r.hi = p >> (64 - sh);
+  } else if (sh > -64) {
+    r.lo = p >> (-sh);
+  }
+  return r;
+}
+
+// Estimator input of bin j: P_j = S_j Q_j 2^-64 (kSpec), or x[j].  tree: sources were
+// deposited into the tree.  The kernels that read it are built for each kind of input: an
+// estimate of a plain array keeps none of the spectrum's registers.
+template <bool kSpec>
+__device__ __forceinline__ double spec_value(const SpecIn& in, long long j, bool tree) {
+  if (kSpec) {
     const ulonglong2* a = reinterpret_cast<const ulonglong2*>(in.acc + 4 * j);
     ulonglong2 w01 = a[0];
     u64 w2 = in.acc[4 * j + 2];
     U128 Q = q_combine3(w01.x, w01.y, w2);
+    if (tree) Q = u128_add(Q, tree_units(in.acc, j, in.nb, in.gq[j], in.g));
     return __dmul_rn(in.S[j], u128_to_dbl_scaled(Q, 64));
   }
   return in.x[j];
 }
 
-__global__ void k_power_out(const unsigned long long* __restrict__ acc, const double* __restrict__ S,
-                            long long n, double* __restrict__ P) {
+__global__ void k_power_out(SpecIn in, long long n, double* __restrict__ P) {
   long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (j >= n) return;
-  SpecIn in;
-  in.acc = acc;
-  in.S = S;
-  in.x = nullptr;
-  P[j] = spec_value(in, j);
+  P[j] = spec_value<true>(in, j, *in.tree != 0);
 }
 
-void launch_power_out(const unsigned long long* acc, const double* S, long long n, double* P,
-                      cudaStream_t st) {
+void launch_power_out(SpecIn in, long long n, double* P, cudaStream_t st) {
   int th = 256;
-  k_power_out<<<(unsigned)((n + th - 1) / th), th, 0, st>>>(acc, S, n, P);
+  k_power_out<<<(unsigned)((n + th - 1) / th), th, 0, st>>>(in, n, P);
+}
+
+// One level of Tree::gsum: a warp per node adds 32 consecutive values of the level below.
+__global__ void k_tree_sums(const double* __restrict__ in, int n, double* __restrict__ out) {
+  const int i = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
+  if (i >= n) return;
+  double v = in[(size_t)i * 32 + (threadIdx.x & 31)];
+  for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+  if ((threadIdx.x & 31) == 0) out[i] = v;
+}
+
+void launch_tree_sums(const double* gq, const Tree& tr, double* gsum, cudaStream_t st) {
+  const double* in = gq;
+  for (int l = 0; l < kTreeLevels; ++l) {
+    double* out = gsum + tr.off[l];
+    if (tr.n[l] > 0) k_tree_sums<<<(tr.n[l] + 7) / 8, 256, 0, st>>>(in, tr.n[l], out);
+    in = out;
+  }
+}
+
+// The parts of a long sweep: bins [b0, b1) and [b2, b3) one by one, and the nodes
+// [lo[l], mid0[l]) and [mid1[l], hi[l]) of each level between them (all relative to the band).
+// k0 .. k1 are the sweep's bins inside the band and ka, kb its first and last: a node holds
+// whole cells only, so never those two.
+struct TreeSpan {
+  int b0, b1, b2, b3;
+  int lo[kTreeLevels], mid0[kTreeLevels], mid1[kTreeLevels], hi[kTreeLevels];
+  int nbins, nnodes;
+};
+__device__ __forceinline__ TreeSpan tree_span(long long ka, long long kb, long long k0,
+                                              long long k1) {
+  TreeSpan t;
+  const int a = (int)(k0 > ka ? k0 : ka + 1), b = (int)(k1 < kb ? k1 : kb - 1) + 1;  // whole cells
+  int lo = (a + 31) >> 5, hi = b >> 5;
+  t.b0 = (int)k0;
+  t.b1 = lo << 5;
+  t.b2 = hi << 5;
+  t.b3 = (int)k1 + 1;
+  t.nbins = (t.b1 - t.b0) + (t.b3 - t.b2);
+  t.nnodes = 0;
+#pragma unroll
+  for (int l = 0; l < kTreeLevels; ++l) {
+    const int up_lo = (lo + 31) >> 5, up_hi = hi >> 5;
+    const bool up = l + 1 < kTreeLevels && up_lo < up_hi;
+    t.lo[l] = lo;
+    t.hi[l] = hi;
+    t.mid0[l] = up ? up_lo << 5 : hi;
+    t.mid1[l] = up ? up_hi << 5 : hi;
+    t.nnodes += (t.mid0[l] - t.lo[l]) + (t.hi[l] - t.mid1[l]);
+    lo = up ? up_lo : 0;
+    hi = up ? up_hi : 0;
+  }
+  return t;
+}
+// Bin x of the span's bins taken one by one (0 <= x < nbins).
+__device__ __forceinline__ int tree_bin(const TreeSpan& t, int x) {
+  const int n0 = t.b1 - t.b0;
+  return x < n0 ? t.b0 + x : t.b2 + (x - n0);
+}
+// Node x of the span's nodes (0 <= x < nnodes): its level (1 ..) and index.
+__device__ __forceinline__ void tree_node(const TreeSpan& t, int x, int* level, int* i) {
+  *level = 1;
+  *i = 0;
+#pragma unroll
+  for (int l = 0; l < kTreeLevels; ++l) {
+    const int n0 = t.mid0[l] - t.lo[l], n1 = t.hi[l] - t.mid1[l];
+    if (x >= 0 && x < n0 + n1) {
+      *level = l + 1;
+      *i = x < n0 ? t.lo[l] + x : t.mid1[l] + (x - n0);
+    }
+    x -= n0 + n1;
+  }
+}
+
+// q of a node for a sweep of length 1 / inv: c = A^2 inv in units of 2^-g (exact: a power of
+// two).  The sweep goes through the tree only when that is inside the fixed-point range (then
+// every bin's power is too, gq < 2^g); otherwise it is walked bin by bin.
+__device__ __forceinline__ bool tree_takes(const Tree& tr, double a2, double inv, long long k0,
+                                           long long k1, double* q) {
+  if (k1 - k0 < kTreeBins) return false;
+  *q = __dmul_rn(__dmul_rn(a2, inv), tr.scale);
+  return (u64)__double_as_longlong(*q) < kQLimitBits;
 }
 
 // ============================================================================ prepass
@@ -217,8 +344,8 @@ __device__ __forceinline__ double sweep_deposit(const Sweep& sw, const Grid& g, 
 // common path.
 // A single-bin sweep is deposited as q_single(A, gq) exactly as the common path deposits it, so
 // that every single-bin source is removed the same way whichever path deposited it.
-__device__ __noinline__ double prepass_slow(double A, double fs, double fds, const Grid g,
-                                            const Tables tb, unsigned long long* acc,
+__device__ __forceinline__ double prepass_slow(double A, double fs, double fds, const Grid& g,
+                                            const Tables& tb, unsigned long long* acc,
                                             unsigned* err) {
   Sweep sw = make_sweep(fs, fds, g.T, g.T2);
   if (sw.ka == sw.kb) {
@@ -240,7 +367,7 @@ __device__ __noinline__ double prepass_slow(double A, double fs, double fds, con
 }
 
 // Bins the FP64 path of a source would walk (0 for a single-bin sweep).
-__device__ __noinline__ long long slow_span(double fs, double fds, const Grid g) {
+__device__ __forceinline__ long long slow_span(double fs, double fds, const Grid& g) {
   Sweep sw = make_sweep(fs, fds, g.T, g.T2);
   if (sw.ka == sw.kb) return 0;
   long long k0, k1;
@@ -248,24 +375,52 @@ __device__ __noinline__ long long slow_span(double fs, double fds, const Grid g)
   return k1 >= k0 ? k1 - k0 + 1 : 0;
 }
 
-// The FP64 path of one long sweep, by a whole warp: the lanes share its bins; the sum of the
+// The FP64 path of one long sweep, by a whole warp: the lanes share its bins, or, beyond
+// kTreeBins of them, the bins at its ends and the nodes of the tree between; the sum of the
 // contributions comes back in every lane.
-__device__ __noinline__ double prepass_slow_warp(double A, double fs, double fds, const Grid g,
-                                                 const Tables tb, unsigned long long* acc,
-                                                 unsigned* err) {
+__device__ __forceinline__ double prepass_slow_warp(double A, double fs, double fds, const Grid& g,
+                                                 const Tables& tb, unsigned long long* acc,
+                                                 RunState* rs) {
   const int lane = threadIdx.x & 31;
   Sweep sw = make_sweep(fs, fds, g.T, g.T2);
   long long k0, k1;
   sweep_bins(sw, g, &k0, &k1);
-  double r = sweep_deposit(sw, g, tb, __dmul_rn(A, A), k0, k1, lane, 32, acc, err);
+  const double a2 = __dmul_rn(A, A), inv = sweep_inv_len(sw);
+  double r = 0.0, q;
+  if (!tree_takes(tb.tree, a2, inv, k0, k1, &q)) {
+    r = sweep_deposit(sw, g, tb, a2, k0, k1, lane, 32, acc, &rs->err);
+  } else if (q > 0.0) {
+    const TreeSpan t = tree_span(sw.ka - g.k_lo, sw.kb - g.k_lo, k0 - g.k_lo, k1 - g.k_lo);
+    for (int x = lane; x < t.nbins; x += 32) {
+      const int j = tree_bin(t, x);
+      const double w = sweep_weight_inv(sw, g.k_lo + j, inv);
+      if (w > 0.0) {
+        const double qj = __dmul_rn(__dmul_rn(a2, w), tb.gq[j]);
+        deposit_q(acc, j, qj, &rs->err);
+        r = __dadd_rn(r, qj);
+      }
+    }
+    u64 c0, c1, c2;
+    q_parts(q, &c0, &c1, &c2);
+    const double c = __dmul_rn(a2, inv);
+    for (int x = lane; x < t.nnodes; x += 32) {
+      int l, i;
+      tree_node(t, x, &l, &i);
+      if (c0) atomicAdd(acc + node_word(l, i, 0), c0);
+      if (c1) atomicAdd(acc + node_word(l, i, 1), c1);
+      if (c2) atomicAdd(acc + node_word(l, i, 2), c2);
+      r = __dadd_rn(r, __dmul_rn(c, tb.tree.gsum[tb.tree.off[l - 1] + i]));
+    }
+    if (lane == 0) rs->tree = 1;
+  }
   for (int o = 16; o > 0; o >>= 1) r = __dadd_rn(r, __shfl_xor_sync(0xFFFFFFFFu, r, o));
   return r;
 }
 
-// Record of a kept candidate (rare; out of line).
-__device__ __noinline__ void emit_candidate(Cands cd, long long c, long long s, double A,
-                                            double fs, double fds, const Grid g,
-                                            unsigned long long* nwide) {
+// Record of a kept candidate.
+__device__ __forceinline__ void emit_candidate(const Cands& cd, long long c, long long s, double A,
+                                            double fs, double fds, const Grid& g,
+                                            RunState* rs) {
   Sweep sw = make_sweep(fs, fds, g.T, g.T2);
   const double a2 = __dmul_rn(A, A);
   cd.src[c] = s;
@@ -278,33 +433,35 @@ __device__ __noinline__ void emit_candidate(Cands cd, long long c, long long s, 
   cd.lo[c] = sw.lo;
   cd.hi[c] = sw.hi;
   cd.res[c] = 0;
-  if (sw.kb - sw.ka + 1 > kSnrLaneBins) cd.wide[atomicAdd(nwide, 1ull)] = c;
+  if (sw.kb - sw.ka + 1 > kSnrLaneBins) cd.wide[atomicAdd(&rs->nwide, 1ull)] = c;
+  if (sw.kb - sw.ka + 1 > kTreeBins) rs->tree_live = 1;
 }
 
-// The decision for one source once r (its rho_0^2 / 4 in units of 2^-96) is known: count
-// it among the paper's candidates, and keep it when it can still be resolved.
-__device__ __forceinline__ void prepass_decide(double r, u64 tk_bits, u64 tl_bits, bool valid,
-                                               long long s, double A, double fs, double fds,
-                                               const Grid& g, Cands& cd, RunState* rs,
-                                               unsigned long long& nkappa) {
+// Keep the live lanes' sources as candidates (the warp together).
+__device__ __forceinline__ void prepass_keep(bool live, long long s, double A, double fs,
+                                             double fds, const Grid& g, const Cands& cd,
+                                             RunState* rs) {
   const int lane = threadIdx.x & 31;
-  u64 rb = (u64)__double_as_longlong(r);
-  bool live = false;
-  if (valid) {
-    if (rb >= tk_bits) ++nkappa;
-    live = (rb > tl_bits) && (rb >= tk_bits);
+  const unsigned m = __ballot_sync(0xFFFFFFFFu, live);
+  if (!m) return;
+  unsigned long long b0 = 0;
+  const int leader = __ffs(m) - 1;
+  if (lane == leader) b0 = atomicAdd(&rs->nlive, (unsigned long long)__popc(m));
+  b0 = __shfl_sync(0xFFFFFFFFu, b0, leader);
+  if (live) {
+    const long long c = (long long)b0 + __popc(m & ((1u << lane) - 1u));
+    emit_candidate(cd, c, s, A, fs, fds, g, rs);
   }
-  unsigned m = __ballot_sync(0xFFFFFFFFu, live);
-  if (m) {
-    unsigned long long b0 = 0;
-    int leader = __ffs(m) - 1;
-    if (lane == leader) b0 = atomicAdd(&rs->nlive, (unsigned long long)__popc(m));
-    b0 = __shfl_sync(0xFFFFFFFFu, b0, leader);
-    if (live) {
-      long long c = (long long)b0 + __popc(m & ((1u << lane) - 1u));
-      emit_candidate(cd, c, s, A, fs, fds, g, &rs->nwide);
-    }
-  }
+}
+
+// The decision for one source once r (its rho_0^2 / 4 in units of 2^-96) is known: counted
+// among the paper's candidates (nkappa), and true when it can still be resolved.
+__device__ __forceinline__ bool prepass_decide(double r, u64 tk_bits, u64 tl_bits,
+                                               unsigned& nkappa) {
+  const u64 rb = (u64)__double_as_longlong(r);
+  if (rb < tk_bits) return false;
+  ++nkappa;
+  return rb > tl_bits;
 }
 
 // ---------------------------------------------------------------- TMA staging
@@ -367,7 +524,7 @@ constexpr int kPreTile = 512;                                 // sources per sta
 constexpr int kPreStages = 4;                                 // tiles in flight per CTA
 constexpr int kPreWarpSrc = kPreTile / kPreConsumers;         // sources per consumer warp
 constexpr int kPrePer = kPreWarpSrc / 32;                     // sources per lane per tile
-constexpr int kSlowWarpCap = 64;                              // queue of a warp (drained at 32)
+constexpr int kSlowWarpCap = 32 + kPreWarpSrc;                // queue of a warp (drained at 32)
 constexpr size_t kPrepassSmem = (size_t)kPreStages * kPreTile * 3 * sizeof(double);
 
 // Sweeps longer than this many bins are walked by a whole warp (loud high-frequency sources
@@ -427,22 +584,37 @@ __device__ __forceinline__ bool single_bin(double fs, double fds, const Grid& g,
   return (x >= m) && (x < __fsub_rn(1.0f, m));
 }
 
-// The FP64 path of up to 32 queued sources q[0 .. cnt) of one warp (lane i takes entry i;
-// sweeps longer than kSlowLaneBins by the whole warp).
+// Arguments of the catalog pass, one block so that the out-of-line parts take one pointer.
+struct PrepassArgs {
+  const CatalogRef* cat;
+  Grid g;
+  Tables tb;
+  u64 tk_bits, tl_bits;  // thresholds on r >= 0, as the bits of non-negative doubles
+  unsigned long long* acc;
+  AccReplicas rep;
+  Cands cd;
+  RunState* rs;
+  int test_flags;
+};
+
+// What a warp sets aside in its queue: a source of the FP64 path, or (tagged) one that the
+// common path deposited and that is to be kept as a candidate.  Both are rare, and the queue's
+// drain is out of line and called once per tile, so that none of its registers are held in the
+// common path.
+constexpr long long kQueueKeep = 1LL << 62;
+
+// Up to 32 queued entries q[0 .. cnt) of one warp (lane i takes entry i; sweeps longer than
+// kSlowLaneBins by the whole warp); returns this lane's count of the paper's candidates.
 template <bool kGen>
-__device__ __forceinline__ void prepass_drain_warp(const CatalogRef* __restrict__ cat,
-                                                   const double* __restrict__ A,
-                                                   const double* __restrict__ f,
-                                                   const double* __restrict__ fdot,
-                                                   const Grid& g, const Tables& tb, u64 tk_bits,
-                                                   u64 tl_bits, unsigned long long* __restrict__ acc,
-                                                   Cands& cd, RunState* rs, const long long* q,
-                                                   int cnt, unsigned long long& nkappa) {
+__device__ __noinline__ unsigned prepass_drain_warp(const PrepassArgs& pa, const CatalogRef* cat,
+                                                    const long long* q, int cnt) {
   const int lane = threadIdx.x & 31;
+  unsigned nkappa = 0;
   const bool valid = lane < cnt;
-  long long s = valid ? q[lane] : 0;
-  double a = 0.0, fs = 0.0, fds = 0.0, r = 0.0;
-  bool wide = false;
+  const long long entry = valid ? q[lane] : 0;
+  const long long s = entry & ~kQueueKeep;
+  double a = 0.0, fs = 0.0, fds = 0.0;
+  bool wide = false, live = (entry & kQueueKeep) != 0;
   if (valid) {
     if (kGen) {
       const double3 gsrc = gen_source_at(cat, s);
@@ -450,81 +622,87 @@ __device__ __forceinline__ void prepass_drain_warp(const CatalogRef* __restrict_
       fs = gsrc.y;
       fds = gsrc.z;
     } else {
-      a = A[s];
-      fs = f[s];
-      fds = fdot[s];
+      a = cat->A[s];
+      fs = cat->f[s];
+      fds = cat->fdot[s];
     }
-    wide = slow_span(fs, fds, g) > kSlowLaneBins;
-    if (!wide) r = prepass_slow(a, fs, fds, g, tb, acc, &rs->err);
+    if (!live) {
+      wide = slow_span(fs, fds, pa.g) > kSlowLaneBins;
+      if (!wide)
+        live = prepass_decide(prepass_slow(a, fs, fds, pa.g, pa.tb, pa.acc, &pa.rs->err),
+                              pa.tk_bits, pa.tl_bits, nkappa);
+    }
   }
-  prepass_decide(r, tk_bits, tl_bits, valid && !wide, s, a, fs, fds, g, cd, rs, nkappa);
   unsigned pending = __ballot_sync(0xFFFFFFFFu, wide);
   while (pending) {
     const int src = __ffs(pending) - 1;
     pending &= pending - 1;
-    const long long sw_s = __shfl_sync(0xFFFFFFFFu, s, src);
     const double sw_a = __shfl_sync(0xFFFFFFFFu, a, src);
     const double sw_f = __shfl_sync(0xFFFFFFFFu, fs, src);
     const double sw_fd = __shfl_sync(0xFFFFFFFFu, fds, src);
-    const double rw = prepass_slow_warp(sw_a, sw_f, sw_fd, g, tb, acc, &rs->err);
-    prepass_decide(rw, tk_bits, tl_bits, lane == 0, sw_s, sw_a, sw_f, sw_fd, g, cd, rs,
-                   nkappa);
+    const double rw = prepass_slow_warp(sw_a, sw_f, sw_fd, pa.g, pa.tb, pa.acc, pa.rs);
+    if (lane == src) live = prepass_decide(rw, pa.tk_bits, pa.tl_bits, nkappa);
+  }
+  prepass_keep(live, s, a, fs, fds, pa.g, pa.cd, pa.rs);
+  return nkappa;
+}
+
+// Drain the warp's queue while it holds 32 entries or more.
+template <bool kGen>
+__device__ __forceinline__ void prepass_drain_full(const PrepassArgs& pa, const CatalogRef* cat,
+                                                   const long long* q, int& qn,
+                                                   unsigned& nkappa) {
+  while (qn >= 32) {
+    // the last 32 entries: nothing moves down
+    __syncwarp();
+    nkappa += prepass_drain_warp<kGen>(pa, cat, q + qn - 32, 32);
+    qn -= 32;
+    __syncwarp();
   }
 }
 
 // One source of the catalog pass (s < N; every lane of the warp calls it together): the
-// common case deposited here, a source the FP64 path must take appended to the warp's queue
-// q (qn entries, the same in every lane), which is drained 32 at a time.
-template <bool kGen>
+// common case deposited here; a source of the FP64 path, or one to keep as a candidate,
+// appended to the warp's queue q (qn entries, the same in every lane).
 __device__ __forceinline__ void prepass_source(
-    long long s, long long N, double a, double fs, double fds, const CatalogRef* __restrict__ cat,
-    const double* __restrict__ A, const double* __restrict__ f, const double* __restrict__ fdot,
-    const Grid& g, const Tables& tb, u64 tk_bits, u64 tl_bits, unsigned long long* __restrict__ acc,
-    const AccReplicas& rep, Cands& cd, RunState* rs, long long* q, int& qn,
-    unsigned long long& nkappa) {
+    long long s, long long N, double a, double fs, double fds, const PrepassArgs& pa, long long* q,
+    int& qn, unsigned& nkappa) {
+  const Grid& g = pa.g;
   const int lane = threadIdx.x & 31;
-  bool valid = false, slow = false;
-  double r = 0.0;
+  long long entry = s;
+  bool set_aside = false;
   if (s < N) {
     // finite inputs, and A^2 finite (|A| < 2^512): else the source is refused below
     const bool fin = finite3(a, fs, fds) && (((u64)__double_as_longlong(a) >> 52) & 0x7FF) < 1535;
     long long k0 = 0;
     const bool single = fin && single_bin(fs, fds, g, &k0);
     if (single) {
-      valid = true;
       const long long j = k0 - g.k_lo;
+      u64 qb = 0;
       if (j >= 0 && j < g.nb) {
-        u64 c0, c1, c2, qb;
-        if (q_single(a, tb.gq[j], &c0, &c1, &c2, &qb)) {
-          if (j < rep.nbins)
-            add_parts_rep(rep, acc, j, (int)(s & (kAccReplicas - 1)), c0, c1, c2);
+        u64 c0, c1, c2;
+        if (q_single(a, pa.tb.gq[j], &c0, &c1, &c2, &qb)) {
+          if (j < pa.rep.nbins)
+            add_parts_rep(pa.rep, pa.acc, j, (int)(s & (kAccReplicas - 1)), c0, c1, c2);
           else
-            add_parts(acc, j, c0, c1, c2);
-          r = __longlong_as_double((long long)qb);
+            add_parts(pa.acc, j, c0, c1, c2);
         } else {
-          atomicOr(&rs->err, ERR_RANGE);
+          qb = 0;
+          atomicOr(&pa.rs->err, ERR_RANGE);
         }
       }
+      set_aside = prepass_decide(__longlong_as_double((long long)qb), pa.tk_bits, pa.tl_bits,
+                                 nkappa);
+      entry |= kQueueKeep;
     } else if (fin) {
-      slow = true;
+      set_aside = true;
     } else {
-      atomicOr(&rs->err, ERR_INPUT);  // the source is skipped; the run reports it
+      atomicOr(&pa.rs->err, ERR_INPUT);  // the source is skipped; the run reports it
     }
   }
-  // append the warp's slow sources to its queue
-  const unsigned sm = __ballot_sync(0xFFFFFFFFu, slow);
-  if (slow) q[qn + __popc(sm & ((1u << lane) - 1u))] = s;
+  const unsigned sm = __ballot_sync(0xFFFFFFFFu, set_aside);
+  if (set_aside) q[qn + __popc(sm & ((1u << lane) - 1u))] = entry;
   qn += __popc(sm);
-  prepass_decide(r, tk_bits, tl_bits, valid, s, a, fs, fds, g, cd, rs, nkappa);
-  if (qn >= 32) {
-    __syncwarp();
-    prepass_drain_warp<kGen>(cat, A, f, fdot, g, tb, tk_bits, tl_bits, acc, cd, rs, q, 32,
-                             nkappa);
-    __syncwarp();
-    if (lane < qn - 32) q[lane] = q[32 + lane];
-    qn -= 32;
-    __syncwarp();
-  }
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
@@ -555,10 +733,9 @@ __device__ __forceinline__ bool mbar_wait_abort(uint64_t* bar, unsigned parity,
   return false;
 }
 
-__global__ void __launch_bounds__(kPrepassThreads, 3) k_prepass(
-    const CatalogRef* cat, Grid g, Tables tb, double thr_kappa, double thr_live,
-    unsigned long long* __restrict__ acc, AccReplicas rep, Cands cd, RunState* rs,
-    int test_flags) {
+__global__ void __launch_bounds__(kPrepassThreads, 3)
+    k_prepass(const __grid_constant__ PrepassArgs pa) {
+  RunState* const rs = pa.rs;
   extern __shared__ __align__(128) double pre_tiles[];  // [stage][A | f | fdot][kPreTile]
   __shared__ __align__(8) uint64_t full[kPreStages], empty[kPreStages];
   __shared__ long long stage_tile[kPreStages];  // tile held by each stage
@@ -569,7 +746,7 @@ __global__ void __launch_bounds__(kPrepassThreads, 3) k_prepass(
   __shared__ CatalogRef scat;
   const int tid = threadIdx.x;
   if (tid == 0) {
-    scat = *cat;
+    scat = *pa.cat;
     for (int k = 0; k < kPreStages; ++k) {
       mbar_init(&full[k], 1);
       mbar_init(&empty[k], kPreConsumers);
@@ -578,7 +755,6 @@ __global__ void __launch_bounds__(kPrepassThreads, 3) k_prepass(
     abort_flag = 0;
   }
   __syncthreads();
-  cat = &scat;
   const double* __restrict__ A = scat.A;
   const double* __restrict__ f = scat.f;
   const double* __restrict__ fdot = scat.fdot;
@@ -612,7 +788,7 @@ __global__ void __launch_bounds__(kPrepassThreads, 3) k_prepass(
       }
       const long long t = (long long)atomicAdd(&rs->next_tile, 1ull);
       stage_tile[stage] = t;
-      if (t < nfull && !(test_flags & 1)) {
+      if (t < nfull && !(pa.test_flags & 1)) {
         copying |= 1u << stage;
         copy_par = (copy_par & ~(1u << stage)) | ((use & 1u) << stage);
         double* d = pre_tiles + (size_t)stage * 3 * kPreTile;
@@ -637,10 +813,7 @@ __global__ void __launch_bounds__(kPrepassThreads, 3) k_prepass(
   }
 
   // -------------------------------------------------- consumers
-  // thresholds on r >= 0 compared as the integer bits of non-negative doubles
-  const u64 tk_bits = (u64)__double_as_longlong(thr_kappa);
-  const u64 tl_bits = (u64)__double_as_longlong(thr_live);
-  unsigned long long nkappa = 0;
+  unsigned nkappa = 0;  // a lane's share of the catalog
   long long* myq = slow_q[warp];
   int qn = 0;  // entries of the warp's queue (the same in every lane)
   for (long long i = 0;; ++i) {
@@ -684,15 +857,14 @@ __global__ void __launch_bounds__(kPrepassThreads, 3) k_prepass(
     if (lane == 0) mbar_arrive(&empty[stage]);
 #pragma unroll
     for (int k = 0; k < kPrePer; ++k)
-      prepass_source<false>(t * kPreTile + base + 32 * k, N, av[k], fv[k], dv[k], cat, A, f,
-                            fdot, g, tb, tk_bits, tl_bits, acc, rep, cd, rs, myq, qn, nkappa);
+      prepass_source(t * kPreTile + base + 32 * k, N, av[k], fv[k], dv[k], pa, myq, qn, nkappa);
+    prepass_drain_full<false>(pa, &scat, myq, qn, nkappa);
   }
   __syncwarp();
   if (qn > 0)
-    prepass_drain_warp<false>(cat, A, f, fdot, g, tb, tk_bits, tl_bits, acc, cd, rs, myq, qn,
-                              nkappa);
+    nkappa += prepass_drain_warp<false>(pa, &scat, myq, qn);
   for (int o = 16; o > 0; o >>= 1) nkappa += __shfl_xor_sync(0xFFFFFFFFu, nkappa, o);
-  if (lane == 0 && nkappa) atomicAdd(&rs->ncand, nkappa);
+  if (lane == 0 && nkappa) atomicAdd(&rs->ncand, (unsigned long long)nkappa);
 }
 
 // The catalog pass over a generated catalog: every source computed from (seed, index) where
@@ -703,20 +875,17 @@ __global__ void __launch_bounds__(kPrepassThreads, 3) k_prepass(
 constexpr int kGenThreads = 256;
 constexpr int kGenPer = 8;  // sources per lane per run
 
-__global__ void __launch_bounds__(kGenThreads, 4) k_prepass_gen(
-    const CatalogRef* cat, Grid g, Tables tb, double thr_kappa, double thr_live,
-    unsigned long long* __restrict__ acc, AccReplicas rep, Cands cd, RunState* rs) {
+__global__ void __launch_bounds__(kGenThreads, 4)
+    k_prepass_gen(const __grid_constant__ PrepassArgs pa) {
+  RunState* const rs = pa.rs;
   __shared__ CatalogRef scat;
   __shared__ long long slow_q[kGenThreads / 32][kSlowWarpCap];
-  if (threadIdx.x == 0) scat = *cat;
+  if (threadIdx.x == 0) scat = *pa.cat;
   __syncthreads();
   if (scat.staged != kCatGenerated) return;
-  cat = &scat;
   const long long N = scat.n;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const u64 tk_bits = (u64)__double_as_longlong(thr_kappa);
-  const u64 tl_bits = (u64)__double_as_longlong(thr_live);
-  unsigned long long nkappa = 0;
+  unsigned nkappa = 0;  // a lane's share of the catalog
   long long* myq = slow_q[warp];
   int qn = 0;
   constexpr long long kRun = 32LL * kGenPer;
@@ -729,17 +898,16 @@ __global__ void __launch_bounds__(kGenThreads, 4) k_prepass_gen(
     for (int k = 0; k < kGenPer; ++k) {
       const long long s = base + 32 * k + lane;
       double3 src = make_double3(0.0, 0.0, 0.0);
-      if (s < N) src = gen_source_at(cat, s);
-      prepass_source<true>(s, N, src.x, src.y, src.z, cat, nullptr, nullptr, nullptr, g, tb,
-                           tk_bits, tl_bits, acc, rep, cd, rs, myq, qn, nkappa);
+      if (s < N) src = gen_source_at(&scat, s);
+      prepass_source(s, N, src.x, src.y, src.z, pa, myq, qn, nkappa);
+      prepass_drain_full<true>(pa, &scat, myq, qn, nkappa);
     }
   }
   __syncwarp();
   if (qn > 0)
-    prepass_drain_warp<true>(cat, nullptr, nullptr, nullptr, g, tb, tk_bits, tl_bits, acc, cd,
-                             rs, myq, qn, nkappa);
+    nkappa += prepass_drain_warp<true>(pa, &scat, myq, qn);
   for (int o = 16; o > 0; o >>= 1) nkappa += __shfl_xor_sync(0xFFFFFFFFu, nkappa, o);
-  if (lane == 0 && nkappa) atomicAdd(&rs->ncand, nkappa);
+  if (lane == 0 && nkappa) atomicAdd(&rs->ncand, (unsigned long long)nkappa);
 }
 
 void launch_prepass(const CatalogRef* cat, long long cap, const Grid& g, const Tables& tb,
@@ -748,14 +916,24 @@ void launch_prepass(const CatalogRef* cat, long long cap, const Grid& g, const T
   long long tiles = (cap + kPreTile - 1) / kPreTile;
   long long lim = (long long)nsm * 3;  // resident CTAs (launch bounds, shared memory)
   int bl = (int)(tiles < lim ? (tiles < 1 ? 1 : tiles) : lim);
-  k_prepass<<<bl, kPrepassThreads, kPrepassSmem, st>>>(cat, g, tb, thr_kappa, thr_live, acc,
-                                                       rep, cd, rs, test_flags);
+  PrepassArgs pa;
+  pa.cat = cat;
+  pa.g = g;
+  pa.tb = tb;
+  memcpy(&pa.tk_bits, &thr_kappa, sizeof(double));
+  memcpy(&pa.tl_bits, &thr_live, sizeof(double));
+  pa.acc = acc;
+  pa.rep = rep;
+  pa.cd = cd;
+  pa.rs = rs;
+  pa.test_flags = test_flags;
+  k_prepass<<<bl, kPrepassThreads, kPrepassSmem, st>>>(pa);
   // the generated-catalog pass: resident CTAs, at most one per run of sources
   const long long runs = (cap + 32LL * kGenPer - 1) / (32LL * kGenPer);
   const long long glim = (long long)nsm * 4 * (kGenThreads / 32);
   const long long gwarps = runs < glim ? (runs < 1 ? 1 : runs) : glim;
   k_prepass_gen<<<(unsigned)((gwarps + kGenThreads / 32 - 1) / (kGenThreads / 32)), kGenThreads, 0,
-                  st>>>(cat, g, tb, thr_kappa, thr_live, acc, rep, cd, rs);
+                  st>>>(pa);
   if (rep.nbins > 0)
     k_fold_replicas<<<(unsigned)((rep.nbins + 255) / 256), 256, 0, st>>>(acc, rep);
 }
@@ -893,7 +1071,9 @@ void launch_max_bits(const double* x, long long n, unsigned long long* max_bits,
 
 // S_gal epilogue: store, fold the relative change of S_n for conv_rtol, and the FP32
 // factor 1 / (1 + S_gal / S_instr) that the SNR screen multiplies rho_0^2 by.
-__device__ __forceinline__ double sg_store(const SgOut& o, long long j, double v) {
+// inv (may be null) receives that factor.
+__device__ __forceinline__ double sg_store(const SgOut& o, long long j, double v,
+                                           float* inv = nullptr) {
   double rel = 0.0;
   if (o.rtol_on) {
     double a = __dadd_rn(o.S[j], v), b = __dadd_rn(o.S[j], o.out[j]);
@@ -902,9 +1082,97 @@ __device__ __forceinline__ double sg_store(const SgOut& o, long long j, double v
   o.out[j] = v;
   if (o.inv_f) {
     float ratio = __fmul_rn(dbl_to_f32_scaled(v, 150), o.invSf[j]);
-    o.inv_f[j] = __frcp_rn(__fadd_rn(1.0f, ratio));
+    const float f = __frcp_rn(__fadd_rn(1.0f, ratio));
+    o.inv_f[j] = f;
+    if (inv) *inv = f;
   }
   return rel;
+}
+
+// ---------------------------------------------------------------- node sums of the SNR
+// h of a node is the sum over its bins of Gf / (1 + S_gal / S_instr) in FP32, so that the
+// screen of a long sweep reads nodes instead of bins.  The kernel that writes S_gal writes
+// level 1 of the bins it wrote; its last CTA to finish (a ticket, no CTA waits) adds up the
+// levels above.  Only in runs that keep a candidate with such a sweep (tree_live).
+__device__ __forceinline__ float warp_sum_f32(float v) {
+  for (int o = 16; o > 0; o >>= 1) v = __fadd_rn(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+  return v;
+}
+// Level 1 nodes [a, b) from the bins' factors in memory (the whole CTA).
+__device__ __forceinline__ void tree_h_nodes(const SgOut& o, int a, int b) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  for (int i = a + warp; i < b; i += nwarp) {
+    const long long j = (long long)i * 32 + lane;
+    const float v = warp_sum_f32(__fmul_rn(o.Gf[j], o.inv_f[j]));
+    if (lane == 0) o.tree.h[i] = v;
+  }
+}
+// True in every thread of the last CTA of the grid to get here; what the others wrote before
+// is then visible to it.
+__device__ __forceinline__ bool last_cta(unsigned* ticket) {
+  __shared__ int last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned t = atomicAdd(ticket, 1u);
+    last = t == gridDim.x - 1;
+    if (last) {
+      *ticket = 0u;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  return last != 0;
+}
+// Sum of 32 values pairwise, v holding them four at a time.
+__device__ __forceinline__ float sum32(const float4 (&v)[8]) {
+  float s[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    s[k] = __fadd_rn(__fadd_rn(v[k].x, v[k].y), __fadd_rn(v[k].z, v[k].w));
+#pragma unroll
+  for (int w = 4; w > 0; w >>= 1)
+#pragma unroll
+    for (int k = 0; k < w; ++k) s[k] = __fadd_rn(s[k], s[k + w]);
+  return s[0];
+}
+// Levels 2 and up from level 1 (the whole CTA): a thread per node adds its 32 values, all of
+// them loaded at once.  (A warp per node left the one CTA waiting on a load per node: 20 us
+// for a band of 1.25e6 bins, against 4.)
+__device__ __noinline__ void tree_h_levels(const Tree& tr) {
+  for (int l = 1; l < kTreeLevels; ++l) {
+    const float4* in = reinterpret_cast<const float4*>(tr.h + tr.off[l - 1]);
+    float* out = tr.h + tr.off[l];
+    for (int i = threadIdx.x; i < tr.n[l]; i += blockDim.x) {
+      float4 v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = __ldcg(in + (size_t)i * 8 + k);
+      out[i] = sum32(v);
+    }
+    __threadfence();
+    __syncthreads();
+  }
+}
+// The level 1 nodes that straddle two median tiles (the bins (u Kc + h) for u < nch), from the
+// factors in memory, a thread per node.
+__device__ __noinline__ void tree_h_straddle(const float* Gf, const float* inv_f, float* h1, int n1,
+                                             int Kc, int h, int nch) {
+  for (int u = threadIdx.x; u < nch; u += blockDim.x) {
+    const long long i = ((long long)u * Kc + h) >> 5;
+    if (i >= n1) continue;
+    const float4* G = reinterpret_cast<const float4*>(Gf + i * 32);
+    const float4* F = reinterpret_cast<const float4*>(inv_f + i * 32);
+    float4 v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const float4 a = G[k], f = __ldcg(F + k);
+      v[k] = make_float4(__fmul_rn(a.x, f.x), __fmul_rn(a.y, f.y), __fmul_rn(a.z, f.z),
+                         __fmul_rn(a.w, f.w));
+    }
+    h1[i] = sum32(v);
+  }
+  __threadfence();
+  __syncthreads();
 }
 
 // Sum over the CTA of every thread's count c (0 <= c <= cmax, cmax the same in every thread),
@@ -1125,8 +1393,9 @@ __device__ bool resort_few_changes(const K (&knew)[E], const K (&kold)[E], const
   return true;
 }
 
-template <int E, typename K>
-__global__ void __launch_bounds__(1024) k_chunk_sort(SpecIn in, long long n, SmoothPlan pl,
+// two elements per thread: 32 registers, so that a whole SM's threads stay resident
+template <int E, typename K, bool kSpec>
+__global__ void __launch_bounds__(1024, E == 2 ? 2 : 1) k_chunk_sort(SpecIn in, long long n, SmoothPlan pl,
                                                      K* __restrict__ skey,
                                                      uint16_t* __restrict__ srank, Dirty d) {
   extern __shared__ __align__(16) unsigned char sort_raw[];
@@ -1134,7 +1403,7 @@ __global__ void __launch_bounds__(1024) k_chunk_sort(SpecIn in, long long n, Smo
   uint16_t* sm_idx = (uint16_t*)(sm_keys + pl.kpad);
   const int T = blockDim.x, tid = threadIdx.x;
   const int kpad = pl.kpad;  // = T * E
-  const ListHead head = list_head(d, kListR0, pl.nch);
+  const ListHead head = list_head(d, kListR0, pl.nch, in.tree);
   const int nitem = head.count;
   // after the first iteration of a tracked run every chunk holds the sorted state of its
   // previous values
@@ -1158,7 +1427,7 @@ __global__ void __launch_bounds__(1024) k_chunk_sort(SpecIn in, long long n, Smo
     for (int a = 0; a < E; ++a) {
       const int i = tid * E + a;
       K kv = (K)~(K)0;
-      if (i < len) kv = sort_key<K>(spec_value(in, base + i), pl.key_scale);
+      if (i < len) kv = sort_key<K>(spec_value<kSpec>(in, base + i, head.tree != 0), pl.key_scale);
       k[a] = kv;
       x[a] = i;
     }
@@ -1321,20 +1590,20 @@ static size_t sort_smem(const SmoothPlan& pl) {
                      (size_t)kResortMax * 2 * (kb + 2);
   return full > few ? full : few;
 }
-template <typename K, typename F>
+template <typename K, bool kSpec, typename F>
 static void with_sort_kernel_k(const SmoothPlan& pl, F fn) {
   switch (sort_per_thread(pl)) {
-    case 2: fn(k_chunk_sort<2, K>); break;
-    case 4: fn(k_chunk_sort<4, K>); break;
-    default: fn(k_chunk_sort<8, K>); break;
+    case 2: fn(k_chunk_sort<2, K, kSpec>); break;
+    case 4: fn(k_chunk_sort<4, K, kSpec>); break;
+    default: fn(k_chunk_sort<8, K, kSpec>); break;
   }
 }
-template <typename F>
+template <bool kSpec, typename F>
 static void with_sort_kernel(const SmoothPlan& pl, F fn) {
   if (pl.fp32_keys)
-    with_sort_kernel_k<uint32_t>(pl, fn);
+    with_sort_kernel_k<uint32_t, kSpec>(pl, fn);
   else
-    with_sort_kernel_k<u64>(pl, fn);
+    with_sort_kernel_k<u64, kSpec>(pl, fn);
 }
 
 void launch_chunk_sort(SpecIn in, long long n, const SmoothPlan& pl, unsigned long long* skey,
@@ -1342,9 +1611,13 @@ void launch_chunk_sort(SpecIn in, long long n, const SmoothPlan& pl, unsigned lo
   const size_t smem = sort_smem(pl);
   const int th = sort_threads(pl);
   const int bl = persistent_grid(pl, pl.nch, pl.res_sort);
-  with_sort_kernel(pl, [&](auto kern) {
+  auto launch = [&](auto kern) {
     launch_sort_as(kern, bl, th, smem, st, in, n, pl, skey, srank, d);
-  });
+  };
+  if (in.acc)
+    with_sort_kernel<true>(pl, launch);
+  else
+    with_sort_kernel<false>(pl, launch);
 }
 
 // ============================================================================ running median
@@ -1672,11 +1945,12 @@ __device__ __forceinline__ double median_tile(const K* __restrict__ skey,
 template <typename K>
 __global__ void __launch_bounds__(512, 2) k_median_wm(
     const K* __restrict__ skey, const uint16_t* __restrict__ srank,
-    long long n, SmoothPlan pl, SgOut o, Dirty d) {
+    long long n, SmoothPlan pl, const __grid_constant__ SgOut o, Dirty d) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   __shared__ int zeros[16];
   double relmax = 0.0;
-  const ListHead head = list_head(d, kListTile, pl.nch + 1);
+  const ListHead head =
+      list_head(d, kListTile, pl.nch + 1, o.tree.h ? &o.rs->tree_live : nullptr);
   const int nitem = head.count;
   int u_next = head.first;
   for (int it = blockIdx.x; it < nitem; it += gridDim.x) {
@@ -1686,6 +1960,18 @@ __global__ void __launch_bounds__(512, 2) k_median_wm(
     double r = median_tile<K>(skey, srank, n, pl, o, u, sm_raw, zeros);
     relmax = r > relmax ? r : relmax;
     __syncthreads();  // before the next tile overwrites shared memory
+    if (head.tree) {
+      // nodes whose bins all lie in this tile's outputs [(u-1) Kc + h, u Kc + h)
+      const long long a = (long long)(u - 1) * pl.Kc + pl.W / 2, b = a + pl.Kc;
+      const long long n1 = o.tree.n[0], na = a > 0 ? (a + 31) >> 5 : 0;
+      tree_h_nodes(o, (int)na, (int)min(b >> 5, n1));
+    }
+  }
+  if (head.tree && last_cta(&o.rs->ticket)) {
+    // the nodes that straddle two tiles, then the levels above
+    if ((pl.W / 2) & 31)
+      tree_h_straddle(o.Gf, o.inv_f, o.tree.h, o.tree.n[0], pl.Kc, pl.W / 2, pl.nch);
+    tree_h_levels(o.tree);
   }
   if (o.rtol_on) warp_max_atomic((u64)__double_as_longlong(relmax), &o.rs->relchg_bits);
 }
@@ -1732,12 +2018,13 @@ __device__ __forceinline__ int sigma_from_max(u64 maxbits) {
 }
 
 // Prefix sums of chunk b.
+template <bool kSpec>
 __device__ __forceinline__ void chunk_prefix(const SpecIn& in, long long n, const SmoothPlan& pl,
                                              unsigned long long* __restrict__ pre_lo,
                                              unsigned long long* __restrict__ pre_hi,
                                              int* __restrict__ sig, unsigned* __restrict__ uflow,
                                              double* __restrict__ x_out, int b, U128* warp_tot,
-                                             u64* warp_max, int& any_uf) {
+                                             u64* warp_max, int& any_uf, bool tree) {
   const long long base = (long long)b * pl.Kc;
   const int len = (int)((n - base) < pl.Kc ? (n - base) : pl.Kc);
   const int per = (pl.Kc + blockDim.x - 1) / blockDim.x;
@@ -1752,7 +2039,7 @@ __device__ __forceinline__ void chunk_prefix(const SpecIn& in, long long n, cons
       int p = p0 + i;
       double x = 0.0;
       if (p < len) {
-        x = spec_value(in, base + p);
+        x = spec_value<kSpec>(in, base + p, tree);
         if (x_out) x_out[base + p] = x;
       }
       v[i] = x;
@@ -1842,6 +2129,7 @@ __device__ __forceinline__ void chunk_prefix(const SpecIn& in, long long n, cons
   }
 }
 
+template <bool kSpec>
 __global__ void k_chunk_prefix(SpecIn in, long long n, SmoothPlan pl,
                                unsigned long long* __restrict__ pre_lo,
                                unsigned long long* __restrict__ pre_hi, int* __restrict__ sig,
@@ -1852,14 +2140,14 @@ __global__ void k_chunk_prefix(SpecIn in, long long n, SmoothPlan pl,
   __shared__ int any_uf;
   // chunks whose input changed (a chunk within in_radius of them is dirty)
   const int list = kListR0 + in_radius;
-  const ListHead head = list_head(d, list, pl.nch);
+  const ListHead head = list_head(d, list, pl.nch, in.tree);
   const int nitem = head.count;
   int b_next = head.first;
   for (int it = blockIdx.x; it < nitem; it += gridDim.x) {
     const int b = b_next;
     if (it + (int)gridDim.x < nitem) b_next = d.item(list, it + gridDim.x);
-    chunk_prefix(in, n, pl, pre_lo, pre_hi, sig, uflow, x_out, b, warp_tot,
-                 warp_max, any_uf);
+    chunk_prefix<kSpec>(in, n, pl, pre_lo, pre_hi, sig, uflow, x_out, b, warp_tot,
+                 warp_max, any_uf, head.tree != 0);
     __syncthreads();
   }
 }
@@ -1869,7 +2157,12 @@ void launch_chunk_prefix(SpecIn in, long long n, const SmoothPlan& pl, unsigned 
                          Dirty d, int in_radius, cudaStream_t st) {
   int th = pl.Kc < 1024 ? pl.Kc : 1024;  // at most 8 values per thread
   int bl = persistent_grid(pl, pl.nch, pl.res_prefix);
-  k_chunk_prefix<<<bl, th, 0, st>>>(in, n, pl, pre_lo, pre_hi, sig, uflow, x_out, d, in_radius);
+  if (in.acc)
+    k_chunk_prefix<true>
+        <<<bl, th, 0, st>>>(in, n, pl, pre_lo, pre_hi, sig, uflow, x_out, d, in_radius);
+  else
+    k_chunk_prefix<false>
+        <<<bl, th, 0, st>>>(in, n, pl, pre_lo, pre_hi, sig, uflow, x_out, d, in_radius);
 }
 
 // Sum of x[a .. e] inside one chunk as a double (a, e in the chunk, a <= e).
@@ -1894,17 +2187,19 @@ __device__ __forceinline__ double part_sum(const double* __restrict__ x, long lo
   return u128_to_dbl_scaled(sum, sigma);
 }
 
+// kTree: the run's S_gal, whose node sums h are kept up to date.
+template <bool kTree>
 __global__ void k_window_mean(const double* __restrict__ x, long long n, SmoothPlan pl,
                               const unsigned long long* __restrict__ pre_lo,
                               const unsigned long long* __restrict__ pre_hi,
                               const int* __restrict__ sig, const unsigned* __restrict__ uflow,
-                              SgOut o, Dirty d, int out_radius) {
+                              const __grid_constant__ SgOut o, Dirty d, int out_radius) {
   double relmax = 0.0;
   const int h = pl.W / 2;
   const double inv_w = 1.0 / (double)pl.W;
   // output chunks with a dirty chunk within out_radius
   const int list = kListR0 + out_radius;
-  const ListHead head = list_head(d, list, pl.nch);
+  const ListHead head = list_head(d, list, pl.nch, kTree ? &o.rs->tree_live : nullptr);
   const int nitem = head.count;
   int b_next = head.first;
   for (int it = blockIdx.x; it < nitem; it += gridDim.x) {
@@ -1930,10 +2225,17 @@ __global__ void k_window_mean(const double* __restrict__ x, long long n, SmoothP
         sum = __dadd_rn(s1, s2);
       }
       double v = (cnt == pl.W) ? __dmul_rn(sum, inv_w) : __ddiv_rn(sum, (double)cnt);
-      double rel = sg_store(o, j, v);
+      float inv = 0.0f;
+      double rel = sg_store(o, j, v, &inv);
       relmax = rel > relmax ? rel : relmax;
+      // chunks and warps start on multiples of 32 bins: a warp holds one node of level 1
+      if (kTree && head.tree && (j | 31) < n) {
+        const float hv = warp_sum_f32(__fmul_rn(o.Gf[j], inv));
+        if ((threadIdx.x & 31) == 0) o.tree.h[j >> 5] = hv;
+      }
     }
   }
+  if (kTree && head.tree && last_cta(&o.rs->ticket)) tree_h_levels(o.tree);
   if (o.rtol_on) warp_max_atomic((u64)__double_as_longlong(relmax), &o.rs->relchg_bits);
 }
 
@@ -1946,7 +2248,12 @@ void launch_window_mean(const double* x, long long n, const SmoothPlan& pl,
                         cudaStream_t st) {
   int th = mean_threads(pl);
   int bl = persistent_grid(pl, pl.nch, pl.res_mean);
-  k_window_mean<<<bl, th, 0, st>>>(x, n, pl, pre_lo, pre_hi, sig, uflow, o, d, out_radius);
+  if (o.tree.h)
+    k_window_mean<true>
+        <<<bl, th, 0, st>>>(x, n, pl, pre_lo, pre_hi, sig, uflow, o, d, out_radius);
+  else
+    k_window_mean<false>
+        <<<bl, th, 0, st>>>(x, n, pl, pre_lo, pre_hi, sig, uflow, o, d, out_radius);
 }
 
 // ============================================================================ SNR + resolve
@@ -2061,6 +2368,46 @@ __device__ __forceinline__ float screen_margin(int kcount) {
   return 1e-5f + 4e-7f * (float)kcount;
 }
 
+// The same by a whole warp for a sweep in the tree: the bins at its ends and the node sums h
+// between them, the same value in every lane.  A term passes through at most 5 roundings in
+// each level of h, the lane's chain (at most 3 bins, or 6 nodes in a band of 2^20 bins; nlev3
+// / 32 more in a longer one) and the butterfly's 5.  False where the sum of h is outside the
+// range in which FP32 keeps that accuracy (the caller then walks the bins).
+__device__ __forceinline__ bool screen_tree(const Cands& cd, long long c, const int4 pk,
+                                            const Grid& g, const Tables& tb,
+                                            const float* __restrict__ inv_f, float* r2out,
+                                            int* kcount) {
+  const int lane = threadIdx.x & 31;
+  const int ka = pk.x, kb = ka + pk.y - 1;
+  const int k0 = ka < 0 ? 0 : ka, k1 = kb < g.nb ? kb : (int)g.nb - 1;
+  if (k1 - k0 < kTreeBins) return false;
+  const float a2f = __int_as_float(pk.z);
+  const float flo = __int_as_float(pk.w), len = cd.len[c];
+  const float fhi = __fadd_rn(flo, len), invlen = 1.0f / len;
+  const TreeSpan t = tree_span(ka, kb, k0, k1);
+  float r2 = 0.0f, hs = 0.0f;
+  for (int x = lane; x < t.nbins; x += 32) {
+    const int k = tree_bin(t, x);
+    const float p = (float)(k - ka);
+    const float a = fmaxf(flo, p - 0.5f);
+    const float b = fminf(fhi, p + 0.5f);
+    if (b > a) {
+      const float w = __fmul_rn(__fsub_rn(b, a), invlen);
+      r2 = __fadd_rn(r2, __fmul_rn(__fmul_rn(__fmul_rn(a2f, w), tb.Gf[k]), inv_f[k]));
+    }
+  }
+  for (int x = lane; x < t.nnodes; x += 32) {
+    int l, i;
+    tree_node(t, x, &l, &i);
+    hs = __fadd_rn(hs, tb.tree.h[tb.tree.off[l - 1] + i]);
+  }
+  hs = warp_sum_f32(hs);
+  if (!(hs >= 1e-30f && hs <= 1e30f)) return false;
+  *r2out = __fadd_rn(warp_sum_f32(r2), __fmul_rn(__fmul_rn(a2f, invlen), hs));
+  *kcount = 5 * kTreeLevels + 6 + 5 + (tb.tree.n[kTreeLevels - 1] >> 5);
+  return true;
+}
+
 // Decision from the FP32 value: 1 resolve, 0 keep, -1 too close to rho_th to tell (the
 // caller then computes rho^2 exactly).
 __device__ __forceinline__ int screen_decide(float r2, int kcount, float th2f, int mode) {
@@ -2106,6 +2453,27 @@ __device__ __forceinline__ void remove_part(const Cands& cd, long long c, const 
   long long k0 = sw.ka > g.k_lo ? sw.ka : g.k_lo;
   long long k1 = sw.kb < g.k_lo + g.nb - 1 ? sw.kb : g.k_lo + g.nb - 1;
   const double inv = sweep_inv_len(sw);
+  double q;
+  if (step == 32 && tree_takes(tb.tree, a2, inv, k0, k1, &q)) {  // as prepass_slow_warp
+    if (!(q > 0.0)) return;
+    const TreeSpan t = tree_span(sw.ka - g.k_lo, sw.kb - g.k_lo, k0 - g.k_lo, k1 - g.k_lo);
+    for (int x = off; x < t.nbins; x += 32) {
+      const int j = tree_bin(t, x);
+      const double w = sweep_weight_inv(sw, g.k_lo + j, inv);
+      if (w > 0.0) remove_q(acc, j, __dmul_rn(__dmul_rn(a2, w), tb.gq[j]));
+    }
+    u64 c0, c1, c2;
+    q_parts(q, &c0, &c1, &c2);
+    for (int x = off; x < t.nnodes; x += 32) {
+      int l, i;
+      tree_node(t, x, &l, &i);
+      if (c0) atomicAdd(acc + node_word(l, i, 0), (u64)(0ull - c0));
+      if (c1) atomicAdd(acc + node_word(l, i, 1), (u64)(0ull - c1));
+      if (c2) atomicAdd(acc + node_word(l, i, 2), (u64)(0ull - c2));
+    }
+    for (long long c = (k0 - g.k_lo) / Kc + off; c <= (k1 - g.k_lo) / Kc; c += 32) d.mark_next(c);
+    return;
+  }
   for (long long k = k0 + off; k <= k1; k += step) {
     double w = sweep_weight_inv(sw, k, inv);
     if (w > 0.0) {
@@ -2113,6 +2481,33 @@ __device__ __forceinline__ void remove_part(const Cands& cd, long long c, const 
       remove_q(acc, j, __dmul_rn(__dmul_rn(a2, w), tb.gq[j]));
       d.mark_next(j / Kc);
     }
+  }
+}
+
+// The decision on a long sweep whose screen value is r2 (the same in every lane of the warp),
+// and its removal.
+__device__ __forceinline__ void snr_wide_decide(
+    const Cands& cd, long long c, const Grid& g, const Tables& tb, const double* __restrict__ Sg,
+    double th2, float th2f, int mode, float r2, int kcount, unsigned char* __restrict__ resolved,
+    unsigned long long* __restrict__ acc, const DirtyIter& di, int Kc, unsigned& local_new,
+    unsigned& local_exact, unsigned& local_near, unsigned& local_unc) {
+  const int lane = threadIdx.x & 31;
+  int dec = screen_decide(r2, kcount, th2f, mode);
+  if (mode == 1 && lane == 0 && screen_uncertain(r2, kcount, th2f)) ++local_unc;
+  if (dec < 0) {
+    // FP64, the lanes sharing the bins
+    if (lane == 0) ++local_exact;
+    const double v = rho2_exact_warp(g, tb, Sg, cd.a2[c], cd.lo[c], cd.hi[c]);
+    if (lane == 0 && near_threshold(v, th2)) ++local_near;
+    dec = v > th2 ? 1 : 0;
+  }
+  if (dec) {
+    if (lane == 0) {
+      cd.res[c] = 1;
+      resolved[cd.src[c]] = 1;
+      ++local_new;
+    }
+    remove_part(cd, c, g, tb, acc, di, Kc, lane, 32);
   }
 }
 
@@ -2124,7 +2519,7 @@ __device__ __forceinline__ void remove_part(const Cands& cd, long long c, const 
 // on one warp walking many.
 
 __global__ void __launch_bounds__(256) k_snr_resolve(
-    Cands cd, Grid g, Tables tb, const double* __restrict__ Sg, const float* __restrict__ inv_f,
+    const __grid_constant__ Cands cd, const __grid_constant__ Grid g, const __grid_constant__ Tables tb, const double* __restrict__ Sg, const float* __restrict__ inv_f,
     double th2, double rtol, int mode, unsigned char* __restrict__ resolved,
     unsigned long long* __restrict__ acc, RunState* rs, Dirty d, int Kc, int sg_radius) {
   // the loop state, read by one thread per CTA (every thread of the grid loading the same
@@ -2199,12 +2594,28 @@ __global__ void __launch_bounds__(256) k_snr_resolve(
     long long kl = (long long)pkw.x + pkw.y - 1;
     if (kl > g.nb - 1) kl = g.nb - 1;
     bool t = false;
-    if (kl >= 0)
-      for (long long cc = c0 + lane; cc <= kl / Kc; cc += 32) t = t || di.any(cc, sg_radius);
+    if (kl >= 0) {
+      const long long c1 = kl / Kc;
+      if (c1 - c0 >= 32 && d.lists) {
+        // many chunks: the work list of the chunks whose S_gal changed is the shorter walk
+        const int nlist = d.count(kListR0 + sg_radius, d.nch);
+        if (nlist == d.nch) t = true;
+        for (int i = lane; i < nlist && !t; i += 32) {
+          const int cc = d.item(kListR0 + sg_radius, i);
+          t = cc >= c0 && cc <= c1;
+        }
+      } else {
+        for (long long cc = c0 + lane; cc <= c1; cc += 32) t = t || di.any(cc, sg_radius);
+      }
+    }
     if (!__any_sync(0xFFFFFFFFu, t)) continue;
-    {
-      int kcount;
-      float r2 = screen_part(cd, cw, pkw, g, tb, inv_f, lane, 32, kcount);
+    int kcount;
+    float r2;
+    if (screen_tree(cd, cw, pkw, g, tb, inv_f, &r2, &kcount)) {
+      snr_wide_decide(cd, cw, g, tb, Sg, th2, th2f, mode, r2, kcount, resolved, acc, di, Kc,
+                      local_new, local_exact, local_near, local_unc);
+    } else {
+      r2 = screen_part(cd, cw, pkw, g, tb, inv_f, lane, 32, kcount);
       // butterfly sums: every lane ends with the same values.  The sum's longest sequential
       // chain is the largest lane count, and the butterfly adds five roundings: the screen's
       // bound takes that many terms, not every bin of the sweep
@@ -2213,24 +2624,8 @@ __global__ void __launch_bounds__(256) k_snr_resolve(
         r2 = __fadd_rn(r2, __shfl_xor_sync(0xFFFFFFFFu, r2, o));
         kchain = max(kchain, __shfl_xor_sync(0xFFFFFFFFu, kchain, o));
       }
-      const int keff = kchain + 5;
-      int dec = screen_decide(r2, keff, th2f, mode);
-      if (mode == 1 && lane == 0 && screen_uncertain(r2, keff, th2f)) ++local_unc;
-      if (dec < 0) {
-        // FP64, the lanes sharing the bins
-        if (lane == 0) ++local_exact;
-        const double v = rho2_exact_warp(g, tb, Sg, cd.a2[cw], cd.lo[cw], cd.hi[cw]);
-        if (lane == 0 && near_threshold(v, th2)) ++local_near;
-        dec = v > th2 ? 1 : 0;
-      }
-      if (dec) {
-        if (lane == 0) {
-          cd.res[cw] = 1;
-          resolved[cd.src[cw]] = 1;
-          ++local_new;
-        }
-        remove_part(cd, cw, g, tb, acc, di, Kc, lane, 32);
-      }
+      snr_wide_decide(cd, cw, g, tb, Sg, th2, th2f, mode, r2, kchain + 5, resolved, acc, di, Kc,
+                      local_new, local_exact, local_near, local_unc);
     }
   }
   for (int o = 16; o > 0; o >>= 1) {
@@ -2426,7 +2821,7 @@ void launch_control(RunState* rs, int max_iter, double rtol, int* new_hist,
 void plan_grids(SmoothPlan& pl) {
   pl.res_sort = pl.res_median = pl.res_prefix = pl.res_mean = 0;
   if (pl.nsm <= 0) return;
-  with_sort_kernel(pl, [&](auto kern) {
+  with_sort_kernel<true>(pl, [&](auto kern) {
     pl.res_sort = resident_ctas(pl, kern, sort_threads(pl), sort_smem(pl));
   });
   if (pl.fp32_keys)
@@ -2435,8 +2830,8 @@ void plan_grids(SmoothPlan& pl) {
   else
     pl.res_median = resident_ctas(pl, k_median_wm<u64>, median_threads(pl),
                                   median_smem_bytes(pl.Kc, 8));
-  pl.res_prefix = resident_ctas(pl, k_chunk_prefix, pl.Kc < 1024 ? pl.Kc : 1024, 0);
-  pl.res_mean = resident_ctas(pl, k_window_mean, mean_threads(pl), 0);
+  pl.res_prefix = resident_ctas(pl, k_chunk_prefix<true>, pl.Kc < 1024 ? pl.Kc : 1024, 0);
+  pl.res_mean = resident_ctas(pl, k_window_mean<true>, mean_threads(pl), 0);
 }
 
 void configure_kernels() {
@@ -2451,8 +2846,10 @@ void configure_kernels() {
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)sort_smem(widest));
     };
-    with_sort_kernel(p64, set);
-    with_sort_kernel(p32, set);
+    with_sort_kernel<true>(p64, set);
+    with_sort_kernel<true>(p32, set);
+    with_sort_kernel<false>(p64, set);
+    with_sort_kernel<false>(p32, set);
   }
   cudaFuncSetAttribute(k_median_wm<u64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)median_smem_bytes(kMaxWindow, 8));

@@ -26,6 +26,29 @@ struct Cands {
 // Sweeps of at most this many bins are screened by one lane; longer ones by a whole warp.
 constexpr int kSnrLaneBins = 4;
 
+// Long sweeps and the tree of bins.  Every interior bin of a sweep holds the same power per
+// unit of response, c = A^2 / length, so a sweep of many bins is deposited into the nodes of
+// a radix-32 tree over the bins instead of bin by bin: level l (1..3) node i stands for the
+// 32^l bins from i 32^l on, and a sweep takes at most 62 nodes of levels 1 and 2 and n / 32^3
+// of level 3, beside at most 66 bins at its ends.  A bin's power is then its own words plus
+// the nodes above it (tree_units); rho_0 and rho take per-node sums over the bins (gsum, h).
+// Bound before: a warp walked every sweep bin by bin, 10^4 .. 10^6 bins at draws of the paper's
+// priors.  Measured on 1e7 sources of one such draw (7 iterations): catalog pass 139 -> 3.1 ms,
+// SNR 43-80 ms -> 13-43 us per iteration, whole simulation 587 -> 4.9 ms.
+// The line lies at kTreeBins = 512 bins: a chirp driven by gravitational waves alone sweeps at
+// most some 300 bins of the band in 4 years, so a catalog of those keeps no nodes up to date,
+// and a warp walks 512 bins in 16 steps, little more than a sweep's ends and nodes take.
+constexpr int kTreeBins = 512;
+constexpr int kTreeLevels = 3;
+struct Tree {
+  const double* gsum;  // per node: sum of gq over its bins, level 1, then 2, then 3
+  float* h;            // per node: sum of Gf / (1 + S_gal / S_instr) over its bins
+  int n[kTreeLevels];  // nodes of each level (complete ones only)
+  int off[kTreeLevels];  // first node of each level in gsum and h
+  double scale;        // 2^g, the power of two above every gq: c scale is q of a node
+  int g;
+};
+
 // Loop state kept on the device for one run.
 struct RunState {
   int iter;              // iterations completed
@@ -45,7 +68,9 @@ struct RunState {
   unsigned long long nuncertain; // FP32 decisions (mixed precision) inside the screen's bound
   unsigned long long nwide;      // entries of Cands::wide
   unsigned err;
-  unsigned pad;
+  int tree;              // 1: a source was deposited into the tree's nodes
+  int tree_live;         // 1: a kept candidate's sweep is in the tree
+  unsigned ticket;       // CTAs done with the kernel that writes the node sums h
 };
 
 // Grid and per-bin tables.
@@ -68,6 +93,7 @@ struct Tables {
   const double* gq;      // 2^96 (T/5) R / S: fixed-point units per unit of A^2 w
   const float* Gf;       // 4 (T/5) R / S * 2^-160: rho_0^2 per unit of A^2 w * 2^160
   const float* invSf;    // 1 / (S * 2^150)
+  Tree tree;
 };
 
 struct SmoothPlan {
@@ -90,6 +116,10 @@ struct SpecIn {
   const unsigned long long* acc;  // 4 words per bin (three used), or null
   const double* S;                // S_instr when acc is set
   const double* x;                // input doubles when acc is null
+  const double* gq;               // Tables::gq and Tree::g (the tree's share of a bin)
+  long long nb;                   // bins in band
+  int g;
+  const int* tree;                // RunState::tree
 };
 
 // Chunks whose input changed since the previous iteration.  Two byte arrays of nch
@@ -163,15 +193,18 @@ struct DirtyIter {
 // shared with the CTA: when every thread of hundreds of CTAs loads the same words, the
 // requests queue on one L2 line and a late iteration's few working CTAs wait behind them.
 struct ListHead {
-  int count, first, iter;
+  int count, first, iter, tree;
 };
-__device__ __forceinline__ ListHead list_head(const Dirty& d, int which, int all) {
+// tree (may be null): a flag of the loop state read along with them.
+__device__ __forceinline__ ListHead list_head(const Dirty& d, int which, int all,
+                                              const int* tree) {
   __shared__ ListHead sh;
   if (threadIdx.x == 0) {
     ListHead h;
     h.count = d.count(which, all);
     h.first = d.item(which, blockIdx.x);  // the grid is never longer than the list
     h.iter = d.base ? d.rs->iter : 0;
+    h.tree = tree ? *tree : 0;
     sh = h;
   }
   __syncthreads();
@@ -187,6 +220,8 @@ struct SgOut {
   const float* invSf;
   int rtol_on;
   RunState* rs;
+  const float* Gf;       // with inv_f: the node sums h of the tree are kept up to date
+  Tree tree;
 };
 
 // Raise the dynamic shared-memory limits of the kernels that need more than 48 KB.
@@ -252,9 +287,11 @@ void launch_coarse_grain(const double* x, const double* S, const long long* edge
                          long long k_lo, double T, double* S_out, double* f_out,
                          long long* cnt_out, cudaStream_t st);
 
-// P[j] = S_j Q_j 2^-96 for every bin.
-void launch_power_out(const unsigned long long* acc, const double* S, long long n, double* P,
-                      cudaStream_t st);
+// P[j] = S_j Q_j 2^-64 for every bin.
+void launch_power_out(SpecIn in, long long n, double* P, cudaStream_t st);
+
+// Tree::gsum of the tables gq (every level of tr.n).
+void launch_tree_sums(const double* gq, const Tree& tr, double* gsum, cudaStream_t st);
 
 // *max_bits = max(*max_bits, bits of max x) over x[0 .. n) (x >= 0).
 void launch_max_bits(const double* x, long long n, unsigned long long* max_bits, cudaStream_t st);

@@ -105,7 +105,11 @@ extern "C" int sub_running_mean_noalloc(const double* x, double* out, int64_t n,
   in.acc = nullptr;
   in.S = nullptr;
   in.x = x;
-  SgOut o;
+  in.gq = nullptr;
+  in.nb = n;
+  in.g = 0;
+  in.tree = nullptr;
+  SgOut o = {};
   o.out = out;
   o.inv_f = nullptr;
   o.S = nullptr;

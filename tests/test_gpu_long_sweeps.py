@@ -1,0 +1,98 @@
+"""Sources whose sweeps go through the tree of bins (more than 512 bins), through the C ABI,
+against the FP64 oracle: sweeps on both sides of the line, starting and ending on and beside
+the nodes' edges (32, 1024 and 32768 bins), running out of the band at either end, covering all
+of it, and downward; faint and loud, so that some are removed again.  S_gal within 1e-10 of the
+oracle's in every bin, and the resolved set, iterations and counts the oracle's, as for every
+other run."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2602_18560_gb300 import gbsub, synth
+from test_gpu_parity import RTOL, compare_run, rel_err
+
+pytestmark = pytest.mark.gpu
+
+T = 4 * synth.YEAR
+F_MAX = 7e-4                      # 75 738 bins: two nodes of level 3, an incomplete last one
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    import torch
+    assert torch.cuda.is_available(), "these tests need a CUDA GPU"
+    gbsub.lib()
+
+
+def sweeps(n):
+    """(first, length) of every sweep in bins relative to the band."""
+    out = [(-0.3, n + 5.0), (0.2, n - 1.4), (-700.0, 1300.25), (-40000.0, 90000.0),
+           (n - 600.0, 5000.0), (n - 513.0, 600.0), (n + 300.0, -2000.5), (n - 1.0, -n + 2.0)]
+    for length in (500.0, 510.6, 511.0, 511.4, 512.0, 512.6, 513.0, 514.2, 600.0, 1023.7, 2100.3,
+                   33000.5, 66000.0):
+        for first in (31.5, 32.0, 32.5, 1023.4, 1024.0, 1056.5, 32767.5, 32768.0, 4321.123):
+            if first + length < n + 400:
+                out.append((first, length))
+                out.append((first + length, -length))
+    return np.array(out)
+
+
+def catalog(est_seed):
+    k_lo, n = oracle.grid(T, 1e-4, F_MAX)
+    S, R = oracle.tables(T, k_lo, n, True)
+    ratio = R / S
+    sw = sweeps(n)
+    f = (k_lo + sw[:, 0]) / T
+    fdot = sw[:, 1] / T**2
+    rng = np.random.default_rng(est_seed)
+    # rho_0 from 2 to 60, from the mean response over the sweep's bins inside the band
+    rho0 = 2.0 * 30.0 ** rng.random(len(sw))
+    A = np.empty(len(sw))
+    for i, (a, d) in enumerate(sw):
+        lo, hi = max(0, int(min(a, a + d))), min(n, int(max(a, a + d)) + 1)
+        A[i] = rho0[i] / np.sqrt(0.8 * T * ratio[lo:hi].sum() / abs(d))
+    # a dense background, some of it resolvable
+    j = np.repeat(np.arange(n), 2)
+    bg = np.sqrt(5.0 * 0.05 * rng.gamma(2.0, size=2 * n) * S[j] / (T * R[j]))
+    bg[::997] *= 30.0
+    return (np.concatenate([A, bg]), np.concatenate([f, (k_lo + j + 0.1) / T]),
+            np.concatenate([fdot, np.zeros(2 * n)]))
+
+
+@pytest.mark.parametrize("est, W", [(gbsub.MEAN, 400), (gbsub.MEDIAN, 101), (gbsub.MEDIAN, 1024),
+                                    (gbsub.MEDIAN_MEAN, 257)])
+def test_long_sweeps_against_the_oracle(est, W):
+    A, f, fdot = catalog(41 + W)
+    st, _, res, _ = compare_run(A, f, fdot, T, est, W, f_max=F_MAX)
+    n_sweeps = len(sweeps(st.n_bins))
+    assert 5 < res[:n_sweeps].sum() < n_sweeps  # some removed, some not
+    assert st.iterations >= 2
+
+
+def test_long_sweeps_other_precisions():
+    A, f, fdot = catalog(7)
+    prm = oracle.make_params(T_obs=T, estimator=gbsub.MEDIAN_MEAN, window=257, f_max=F_MAX)
+    ref = oracle.run(prm, A, f, fdot)
+    for precision, tol in ((gbsub.FP64_STRICT, RTOL), (gbsub.MIXED, 1e-5)):
+        with gbsub.Subtraction(T_obs=T, estimator=gbsub.MEDIAN_MEAN, window=257, f_max=F_MAX,
+                               precision=precision) as s:
+            s.load(A, f, fdot)
+            st = s.run()
+            assert np.sum(s.resolved().astype(bool) != ref["resolved"]) <= st.n_uncertain
+            if st.n_uncertain == 0:
+                assert rel_err(s.spectrum(), ref["S_gal"]) <= tol
+            # the residual power is the tree's and the bins' together
+            P = s.power()
+            assert np.all(P > 0)
+
+
+def test_power_beyond_the_range_is_still_refused():
+    # one sweep of 2000 bins whose power passes 2^63 S_instr in every bin: as bin by bin
+    k_lo, n = oracle.grid(T, 1e-4, F_MAX)
+    S, R = oracle.tables(T, k_lo, n, True)
+    A = np.array([np.sqrt(5.0 * 2.0**66 * 2000.0 * np.max(S / R) / T)])
+    with gbsub.Subtraction(T_obs=T, window=100, estimator=gbsub.MEAN, f_max=F_MAX) as s:
+        s.load(A, np.array([(k_lo + 3000.0) / T]), np.array([2000.0 / T**2]))
+        with pytest.raises(gbsub.SubError) as ei:
+            s.run()
+        assert ei.value.code == gbsub.ERANGE
