@@ -163,23 +163,15 @@ extern "C" int sub_create(const sub_params* p, void* stream, sub_ctx** out) {
   c->grid.k_lo = k_lo;
   c->grid.nb = n;
   {
-    // T_obs = mT 2^eT with mT the 53-bit integer mantissa (for the exact f T in the prepass)
+    // T_obs = mT 2^eT, mT the 53-bit integer mantissa, split in its top 32 bits and the rest
     int ex = 0;
-    double m = std::frexp(p->T_obs, &ex);  // T = m 2^ex, m in [0.5, 1)
-    c->grid.mT = (unsigned long long)std::ldexp(m, 53);
-    c->grid.eT = ex - 53;
+    const double m = std::frexp(p->T_obs, &ex);  // T = m 2^ex, m in [0.5, 1)
+    const unsigned long long mT = (unsigned long long)std::ldexp(m, 53);
+    c->grid.tq = (unsigned)(mT >> 21);
+    c->grid.tr = (unsigned)(mT << 11);
+    c->grid.ebin = 1020 - (ex - 32);  // T = (tq + tr 2^-32) 2^(ex - 32)
+    if (c->grid.ebin - 39 < 1 || c->grid.ebin > 0x7FE) c->grid.ebin = -(1 << 20);
     c->grid.T2f = (float)(p->T_obs * p->T_obs);
-    // the same with the trailing zero bits of the mantissa dropped: whole seconds of
-    // observation time leave at most 32 bits, and f T then takes two 32-bit products
-    unsigned long long tq = c->grid.mT;
-    int etq = c->grid.eT;
-    while (tq && !(tq & 1ull)) {
-      tq >>= 1;
-      ++etq;
-    }
-    c->grid.short_t = (tq > 0 && tq < (1ull << 32)) ? 1 : 0;
-    c->grid.tq = c->grid.short_t ? (unsigned)tq : 0u;
-    c->grid.etq = etq;
   }
   c->plan = make_plan(p->window, n);
   c->plan.fp32_keys = p->precision == SUB_MIXED ? 1 : 0;  // FP32 median selection
@@ -573,14 +565,14 @@ static SpecIn spectrum_of(const sub_ctx* c) {
   in.gq = c->gq;
   in.nb = c->grid.nb;
   in.g = c->tree.g;
-  in.tree = &c->rs->tree;
+  in.flags = &c->rs->spec;
   return in;
 }
 static SpecIn array_of(const sub_ctx* c, const double* x) {
   SpecIn in = spectrum_of(c);
   in.acc = nullptr;
   in.x = x;
-  in.tree = nullptr;
+  in.flags = nullptr;
   return in;
 }
 

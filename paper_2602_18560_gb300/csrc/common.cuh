@@ -119,6 +119,15 @@ __device__ __forceinline__ void q_parts(double q, u64* c0, u64* c1, u64* c2) {
   *c2 = v.hi;
 }
 
+__device__ __forceinline__ unsigned hi32(u64 x) { return (unsigned)(x >> 32); }
+__device__ __forceinline__ unsigned lo32(u64 x) { return (unsigned)x; }
+// x >> n, 0 for n >= 64.
+__device__ __forceinline__ u64 shr_clamp(u64 x, unsigned n) {
+  u64 r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
+  return r;
+}
+
 // The deposit of a single-bin source, q = A^2 gq (units of 2^-96 of the bin's S_instr;
 // gq = 2^96 (T/5) R / S_instr), from the integer mantissas: the top 64 bits of A's mantissa
 // squared, times gq's, the products truncated.  It is within 2^-61 of the exact A^2 gq (the
@@ -166,58 +175,12 @@ __device__ __forceinline__ bool q_single(double A, double gq, u64* c0, u64* c1, 
   return true;
 }
 
-// f * T rounded to nearest (ties to even), computed exactly in integer arithmetic, returned
-// as x = u + 1/2 split into its integer part k and the top 24 bits of its fraction.  T is
-// given by its 53-bit integer mantissa mT and exponent eT (T = mT 2^eT).  Returns false when
-// the product is out of the range handled here (f not a positive normal number, or
-// f T >= 2^30), in which case the caller uses plain FP64.
-__device__ __forceinline__ bool ft_bin(double f, u64 mT, int eT, long long* k, unsigned* frac24,
-                                       int* fracbits) {
-  u64 b = (u64)__double_as_longlong(f);
-  int e = (int)((b >> 52) & 0x7FF);
-  if ((b >> 63) || e == 0 || e == 0x7FF) return false;
-  u64 mf = (b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
-  u64 lo = mf * mT;
-  u64 hi = __umul64hi(mf, mT);  // product in [2^104, 2^106)
-  int sh = ((hi >> 41) & 1ull) ? 53 : 52;
-  // M = p >> sh with round-to-nearest-even on the dropped bits
-  u64 M = (hi << (64 - sh)) | (lo >> sh);
-  u64 rmask = (1ull << sh) - 1ull;
-  u64 r = lo & rmask;
-  u64 half = 1ull << (sh - 1);
-  if (r > half || (r == half && (M & 1ull))) {
-    ++M;
-    if (M >> 53) {
-      M >>= 1;
-      ++sh;
-    }
-  }
-  int E = (e - 1075) + eT + sh;  // f T = M 2^E
-  if (E > -23 || E < -62) return false;
-  int F = -E;                    // fraction bits of M
-  u64 x = M + (1ull << (F - 1)); // (f T + 1/2) 2^F
-  *k = (long long)(x >> F);
-  u64 fr = x & ((1ull << F) - 1ull);
-  *frac24 = (F >= 24) ? (unsigned)(fr >> (F - 24)) : (unsigned)(fr << (24 - F));
-  *fracbits = F;
-  return true;
-}
-
-// Signed FP32 value of a double (truncated mantissa); 0 below the FP32 normal range.
-__device__ __forceinline__ float dbl_to_f32_signed(double v) {
-  u64 b = (u64)__double_as_longlong(v);
-  int e = (int)((b >> 52) & 0x7FF);
-  int ef = e - 1023 + 127;
-  if (e == 0 || ef <= 0) return 0.0f;
-  if (ef >= 255) return __int_as_float(0x7FC00000);
-  unsigned fb = ((unsigned)(b >> 63) << 31) | ((unsigned)ef << 23) | (unsigned)((b >> 29) & 0x7FFFFFu);
-  return __uint_as_float(fb);
-}
-
-__device__ __forceinline__ U128 q_combine3(u64 w0, u64 w1, u64 w2) {
+// Q of a bin's words.  carried: words 0 and 1 are signed (see kSpecCarried).
+__device__ __forceinline__ U128 q_combine3(u64 w0, u64 w1, u64 w2, bool carried = false) {
   U128 r;
   r.lo = w0 + (w1 << 32);
   r.hi = w2 + (w1 >> 32) + (r.lo < w0 ? 1ull : 0ull);
+  if (carried) r.hi -= (w0 >> 63) + ((w1 >> 63) << 32);
   return r;
 }
 

@@ -20,6 +20,7 @@
 // bits of the doubles, window sums are integer, and the SNR test is screened in FP32 with
 // a proven error margin (exact FP64 recomputation inside the margin).
 
+#include <climits>
 #include <cstring>
 
 #include <cuda_runtime.h>
@@ -167,17 +168,16 @@ __device__ __noinline__ U128 tree_units(const unsigned long long* __restrict__ a
   return r;
 }
 
-// Estimator input of bin j: P_j = S_j Q_j 2^-64 (kSpec), or x[j].  tree: sources were
-// deposited into the tree.  The kernels that read it are built for each kind of input: an
+// Estimator input of bin j: P_j = S_j Q_j 2^-64 (kSpec; flags: RunState::spec), or x[j].  The kernels that read it are built for each kind of input: an
 // estimate of a plain array keeps none of the spectrum's registers.
 template <bool kSpec>
-__device__ __forceinline__ double spec_value(const SpecIn& in, long long j, bool tree) {
+__device__ __forceinline__ double spec_value(const SpecIn& in, long long j, int flags) {
   if (kSpec) {
     const ulonglong2* a = reinterpret_cast<const ulonglong2*>(in.acc + 4 * j);
     ulonglong2 w01 = a[0];
     u64 w2 = in.acc[4 * j + 2];
-    U128 Q = q_combine3(w01.x, w01.y, w2);
-    if (tree) Q = u128_add(Q, tree_units(in.acc, j, in.nb, in.gq[j], in.g));
+    U128 Q = q_combine3(w01.x, w01.y, w2, (flags & kSpecCarried) != 0);
+    if (flags & kSpecTree) Q = u128_add(Q, tree_units(in.acc, j, in.nb, in.gq[j], in.g));
     return __dmul_rn(in.S[j], u128_to_dbl_scaled(Q, 64));
   }
   return in.x[j];
@@ -186,7 +186,7 @@ __device__ __forceinline__ double spec_value(const SpecIn& in, long long j, bool
 __global__ void k_power_out(SpecIn in, long long n, double* __restrict__ P) {
   long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (j >= n) return;
-  P[j] = spec_value<true>(in, j, *in.tree != 0);
+  P[j] = spec_value<true>(in, j, *in.flags);
 }
 
 void launch_power_out(SpecIn in, long long n, double* P, cudaStream_t st) {
@@ -285,14 +285,6 @@ __device__ __forceinline__ bool tree_takes(const Tree& tr, double a2, double inv
 // picking one by its index; a fold adds them into the spectrum after the pass (word 2 takes
 // a part only from a source of at least S_instr in the bin, rare, and goes to the spectrum
 // directly).  Integer sums, so the result does not depend on the split.
-__device__ __forceinline__ void add_parts_rep(AccReplicas rep, unsigned long long* acc,
-                                              long long j, int r, u64 c0, u64 c1, u64 c2) {
-  u64* a = rep.w + 2 * ((size_t)r * rep.nbins + j);
-  if (c0) atomicAdd(a + 0, c0);
-  if (c1) atomicAdd(a + 1, c1);
-  if (c2) atomicAdd(acc + 4 * j + 2, c2);
-}
-
 __global__ void k_fold_replicas(unsigned long long* __restrict__ acc, AccReplicas rep) {
   long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (j >= rep.nbins) return;
@@ -411,7 +403,7 @@ __device__ __forceinline__ double prepass_slow_warp(double A, double fs, double 
       if (c2) atomicAdd(acc + node_word(l, i, 2), c2);
       r = __dadd_rn(r, __dmul_rn(c, tb.tree.gsum[tb.tree.off[l - 1] + i]));
     }
-    if (lane == 0) rs->tree = 1;
+    if (lane == 0 && !(*(volatile int*)&rs->spec & kSpecTree)) atomicOr(&rs->spec, (int)kSpecTree);
   }
   for (int o = 16; o > 0; o >>= 1) r = __dadd_rn(r, __shfl_xor_sync(0xFFFFFFFFu, r, o));
   return r;
@@ -510,22 +502,33 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity) {
 // are rare (well under 1%), but one such lane would hold its whole warp on the slow FP64
 // pipe, so each warp queues them in shared memory and runs them 32 at a time.
 //
-// Layout of a CTA: kPreConsumers consumer warps and one producer warp.  The producer takes
-// tiles of kPreTile sources from a global counter (CTAs that run faster take more tiles) and
-// streams each into one of kPreStages shared-memory stages with bulk asynchronous copies of
-// A, f and fdot (cp.async.bulk, completion counted in bytes on the stage's "full" mbarrier).
-// Each consumer warp takes its own kPreTile / kPreConsumers sources of the stage and, done,
-// arrives on the stage's "empty" mbarrier; the producer refills a stage once every consumer
-// warp has arrived.  No CTA-wide barrier runs in the steady state, so a warp that meets a
-// slow source delays no other warp.
-constexpr int kPreConsumers = 8;
-constexpr int kPrepassThreads = (kPreConsumers + 1) * 32;
-constexpr int kPreTile = 512;                                 // sources per staged tile
-constexpr int kPreStages = 4;                                 // tiles in flight per CTA
-constexpr int kPreWarpSrc = kPreTile / kPreConsumers;         // sources per consumer warp
-constexpr int kPrePer = kPreWarpSrc / 32;                     // sources per lane per tile
-constexpr int kSlowWarpCap = 32 + kPreWarpSrc;                // queue of a warp (drained at 32)
-constexpr size_t kPrepassSmem = (size_t)kPreStages * kPreTile * 3 * sizeof(double);
+// Layout of the pass: one CTA per SM, kPreWarps warps, each on its own.  The steps of kPreStep
+// sources are dealt out in turn over all warps of the grid; a warp streams its steps through
+// kPreStages shared-memory stages with bulk asynchronous copies of A, f and fdot (cp.async.bulk,
+// completion counted in bytes on the stage's mbarrier): once its values are in registers the
+// stage takes the step after the next.  No barrier between warps runs in the steady state, so a
+// warp that meets a slow source delays no other.
+//
+// Bound: before, the requests from the SMs to L2 (two 64-bit atomics and most of a table gather
+// per source, one request a cycle and SM: 0.3 of 0.47 ms for 3e7 sources), and instruction issue.
+// Measured, catalog pass with its memsets and fold, start -> now: 3e7 sources 470 -> 343 us, 1e7
+// 170 -> 127, 1e6 45 -> 43.  What was tried on the way (3e7): steps in runs from a global counter
+// 376 (the counter gives out a number every 1.7 ns, and long runs lose the locality of the
+// stream: 450 at two runs a warp); 24 warps 351, 28 391, 16 with four sources a lane 371; the
+// table entries of the first bins in shared memory too, no gain; gathers issued a step ahead, no
+// gain.
+constexpr int kPreWarps = 20;
+constexpr int kPrepassThreads = kPreWarps * 32;
+constexpr int kPrePer = 2;                                    // sources per lane per step
+constexpr int kPreStep = 32 * kPrePer;                        // sources per step
+constexpr int kPreStages = 2;                                 // steps in flight per warp
+constexpr int kSlowWarpCap = 32 + kPreStep;                   // queue of a warp (drained at 32)
+constexpr int kHotBins = 4096;                                // bins kept in shared memory
+constexpr long long kHotMinSources = 1000000;
+constexpr size_t kPrepassSmem =
+    (size_t)kPreWarps * (kPreStages * 3 * kPreStep * sizeof(double) +
+                         kSlowWarpCap * sizeof(long long)) +
+    (size_t)kHotBins * 3 * sizeof(unsigned);
 
 // Sweeps longer than this many bins are walked by a whole warp (loud high-frequency sources
 // sweep up to hundreds of bins; one lane walking them in FP64 would hold its warp, and the
@@ -540,48 +543,40 @@ __device__ __forceinline__ double3 gen_source_at(const CatalogRef* __restrict__ 
   return r;
 }
 
-// f T + 1/2 split into its integer part k and the top 24 bits of its fraction, from the
-// exact product when T's mantissa has at most 32 significant bits (T = tq 2^etq; whole
-// seconds of observation time qualify).  The mantissa of f is split in 21 + 32 bits, so the
-// product is two 32 x 32 -> 64-bit multiplies.  Exact f T, not its FP64 rounding: the two
-// differ by less than 2^-33 bins in the band, and the caller keeps a source on this path
-// only when the fraction is at least 2^-20 from a cell edge, where both give the same bin.
-// False for f not positive normal, or f T outside the range handled here.
-__device__ __forceinline__ bool ft_bin_short(double f, unsigned tq, int etq, long long* k,
-                                             unsigned* frac24) {
-  const u64 b = (u64)__double_as_longlong(f);
-  const int e = (int)(b >> 52);  // sign bit included: a negative f fails the range test
-  if (e <= 0 || e >= 0x7FF) return false;
-  const u64 mf = (b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
-  const u64 p0 = (u64)(unsigned)mf * tq;           // low 32 bits of mf times tq
-  const u64 p1 = (u64)(unsigned)(mf >> 32) * tq;   // high 21 bits of mf times tq
-  const u64 hi = p1 + (p0 >> 32);                  // f T = (hi 2^32 + lo) 2^(e - 1075 + etq)
-  const int G = 1075 - etq - e - 32;               // fraction bits of f T within hi
-  if (G < 24 || G > 62) return false;
-  const u64 x = hi + (1ull << (G - 1));            // + 1/2
-  *k = (long long)(x >> G);
-  *frac24 = (unsigned)(x >> (G - 24)) & 0xFFFFFFu;
-  return true;
-}
-
-// The common case of one source without any FP64 arithmetic beyond A^2: its bin k0 and the
-// FP32 certificate that the whole sweep [f T, f T + fdot T^2] stays inside cell k0 (else the
-// FP64 path takes it).
-__device__ __forceinline__ bool single_bin(double fs, double fds, const Grid& g, long long* k0) {
-  unsigned fr24 = 0;
-  bool ok;
-  if (g.short_t) {
-    ok = ft_bin_short(fs, g.tq, g.etq, k0, &fr24);
-  } else {
-    int fb;
-    ok = ft_bin(fs, g.mT, g.eT, k0, &fr24, &fb);
-  }
-  if (!ok) return false;
-  const float du = __fmul_rn(dbl_to_f32_signed(fds), g.T2f);
-  const float phi = __fmul_rn((float)fr24, 5.9604644775390625e-8f);             // 2^-24
-  const float m = __fadd_rn(9.5367431640625e-7f, __fmul_rn(4e-7f, fabsf(du)));  // 2^-20 + ...
-  const float x = __fadd_rn(phi, du);
-  return (x >= m) && (x < __fsub_rn(1.0f, m));
+// The common case of one source without FP64 arithmetic: the bin k its sweep starts in, and
+// the certificate that the whole sweep [f T, f T + fdot T^2] stays inside cell k (false: the
+// FP64 path takes the source).
+//
+// f T comes from the 53-bit mantissa of f, split in 21 + 32 bits, times T's in 32 + 21: three
+// 32-bit products, exact but for two units of their 2^53 (2^-32 of a bin in the band; the
+// dropped part of T's low bits).  With at most 30 integer bits, the product is shifted to 23
+// fraction bits.  The certificate is FP32: the start's offset from the bin's centre plus
+// du = fdot T^2 (off by less than 4e-7 |du|) must stay 2^-20 inside the cell, which covers the
+// truncation of the fraction and the FP64 rounding of f T in the reference.  A value that is
+// not finite fails it (f: no exponent in range; fdot: du is not a number or too large).
+//
+// T's mantissa is used with its top bit set: with its trailing zeros dropped instead (20 bits
+// left for 4 years) the product kept too few bits for f above 1 mHz, and every such source,
+// 0.5% of a catalog, went through the FP64 path.
+__device__ __forceinline__ bool source_bin(double fs, double fds, const Grid& g, int* k) {
+  const u64 bf = (u64)__double_as_longlong(fs), bd = (u64)__double_as_longlong(fds);
+  const unsigned fh = hi32(bf), dh = hi32(bd);
+  const unsigned n = (unsigned)(g.ebin - (int)(fh >> 20));  // a negative f: n wraps
+  const unsigned mh = (fh & 0x000FFFFFu) | 0x00100000u;
+  const u64 prod = (u64)mh * g.tq + hi32((u64)lo32(bf) * g.tq) + __umulhi(mh, g.tr);
+  const u64 x = (prod >> (n & 63u)) + (1u << 22);           // f T + 1/2, 23 fraction bits
+  *k = (int)(x >> 23);
+  // the offset from the centre, in [-1/2, 1/2): 1 + fraction as a float, less 3/2 (exact)
+  const float off = __fadd_rn(__uint_as_float((lo32(x) & 0x007FFFFFu) | 0x3F800000u), -1.5f);
+  // fdot as a float: its exponent rebased (1023 - 127 = 0x380, so that the low eight bits
+  // change in the top one only) and its mantissa cut to 23 bits; 0 below the FP32 range
+  const unsigned da = dh & 0x7FFFFFFFu;
+  const unsigned fb = ((__funnelshift_l(lo32(bd), dh, 3) & 0x7FFFFFFFu) ^ 0x40000000u) |
+                      (dh & 0x80000000u);
+  const float fd = da >= (897u << 20) ? __uint_as_float(fb) : 0.0f;
+  const float du = __fmul_rn(fd, g.T2f);
+  const float edge = __fmaf_rn(-4e-7f, fabsf(du), 0.5f - 9.5367431640625e-7f);
+  return n <= 39u && da < (1151u << 20) && fabsf(__fadd_rn(off, du)) < edge;
 }
 
 // Arguments of the catalog pass, one block so that the out-of-line parts take one pointer.
@@ -590,6 +585,8 @@ struct PrepassArgs {
   Grid g;
   Tables tb;
   u64 tk_bits, tl_bits;  // thresholds on r >= 0, as the bits of non-negative doubles
+  int tk_hi;             // high word of tk_bits, INT_MIN when that is 0: a source whose r has a
+                         // smaller high word (as a signed number) is below the threshold
   unsigned long long* acc;
   AccReplicas rep;
   Cands cd;
@@ -602,6 +599,7 @@ struct PrepassArgs {
 // drain is out of line and called once per tile, so that none of its registers are held in the
 // common path.
 constexpr long long kQueueKeep = 1LL << 62;
+constexpr unsigned kMaxAExp = 1535;  // exponent field of 2^512
 
 // Up to 32 queued entries q[0 .. cnt) of one warp (lane i takes entry i; sweeps longer than
 // kSlowLaneBins by the whole warp); returns this lane's count of the paper's candidates.
@@ -614,7 +612,7 @@ __device__ __noinline__ unsigned prepass_drain_warp(const PrepassArgs& pa, const
   const long long entry = valid ? q[lane] : 0;
   const long long s = entry & ~kQueueKeep;
   double a = 0.0, fs = 0.0, fds = 0.0;
-  bool wide = false, live = (entry & kQueueKeep) != 0;
+  bool wide = false, live = (entry & kQueueKeep) != 0;  // (tagged: finite inputs)
   if (valid) {
     if (kGen) {
       const double3 gsrc = gen_source_at(cat, s);
@@ -626,7 +624,12 @@ __device__ __noinline__ unsigned prepass_drain_warp(const PrepassArgs& pa, const
       fs = cat->f[s];
       fds = cat->fdot[s];
     }
-    if (!live) {
+    // finite inputs, and A^2 finite (|A| < 2^512): else the source is skipped and the run
+    // reports it
+    if (!live && !(finite3(a, fs, fds) &&
+                   (((u64)__double_as_longlong(a) >> 52) & 0x7FF) < kMaxAExp)) {
+      atomicOr(&pa.rs->err, ERR_INPUT);
+    } else if (!live) {
       wide = slow_span(fs, fds, pa.g) > kSlowLaneBins;
       if (!wide)
         live = prepass_decide(prepass_slow(a, fs, fds, pa.g, pa.tb, pa.acc, &pa.rs->err),
@@ -661,69 +664,141 @@ __device__ __forceinline__ void prepass_drain_full(const PrepassArgs& pa, const 
   }
 }
 
-// One source of the catalog pass (s < N; every lane of the warp calls it together): the
-// common case deposited here; a source of the FP64 path, or one to keep as a candidate,
-// appended to the warp's queue q (qn entries, the same in every lane).
-__device__ __forceinline__ void prepass_source(
-    long long s, long long N, double a, double fs, double fds, const PrepassArgs& pa, long long* q,
-    int& qn, unsigned& nkappa) {
-  const Grid& g = pa.g;
+// The first bins' words in shared memory (catalog pass over a stored catalog): 96 bits a bin in
+// three 32-bit words, carried over as they are added, so a deposit is two shared-memory atomics
+// there instead of two in L2.  The source density falls so steeply with f that 4 096 bins take
+// about half of a catalog (3e7 sources: 343 us against 470 without; 2 048 or 6 144 bins: +5 us).
+// From kHotMinSources on: below 1e6 sources clearing and adding up the words costs what they
+// save (43 us either way at 1e6).
+struct HotBins {
+  unsigned* w;  // [3][kHotBins]
+  int n;        // bins kept (0: none)
+};
+__device__ __forceinline__ void hot_add(const HotBins& h, int j, unsigned c0, unsigned c1) {
+  const unsigned o0 = atomicAdd(h.w + j, c0);
+  const unsigned a1 = c1 + (o0 + c0 < o0 ? 1u : 0u);
+  const unsigned o1 = atomicAdd(h.w + kHotBins + j, a1);
+  const unsigned a2 = (a1 < c1 ? 1u : 0u) + (o1 + a1 < o1 ? 1u : 0u);
+  if (a2) atomicAdd(h.w + 2 * kHotBins + j, a2);
+}
+
+// One source of the catalog pass in two steps, so that the table gathers of a lane's sources
+// are under way together.
+//
+// Bound: instruction issue.  The pass reads 24 bytes a source (0.1 ms for 3e7 at the measured
+// HBM rate) and used to issue 301 instructions per 32 sources.  What is left out here: tests
+// that the rare paths repeat (finite inputs, the range of q, both thresholds: a source is
+// handed to q_single only when its exponent and top 20 bits say that it may pass the lower
+// one, or when it reaches the third word), 64-bit shifts by zero-extended halves, and the
+// conversions between FP64, integers and FP32.
+struct PlacedSource {
+  int j;       // bin in band, or -1: outside it, or -2: for the FP64 path
+  double gq;
+};
+__device__ __forceinline__ PlacedSource place_source(bool valid, double a, double fs, double fds,
+                                                     const PrepassArgs& pa) {
+  PlacedSource p;
+  int k;
+  const bool single = source_bin(fs, fds, pa.g, &k) &&
+                      (hi32((u64)__double_as_longlong(a)) & 0x7FF00000u) < (kMaxAExp << 20);
+  const unsigned j = (unsigned)(k - (int)pa.g.k_lo);
+  const bool in = single && j < (unsigned)pa.g.nb;
+  p.j = in ? (int)j : (single ? -1 : -2);
+  p.gq = 0.0;
+  if (!valid) p.j = -3;  // beyond the catalog
+  if (p.j >= 0) p.gq = pa.tb.gq[j];
+  return p;
+}
+
+// The deposit of a placed source (q_single's integers) and whether the rare path has to settle
+// it: third word, range, thresholds.  No branches, so that a lane's sources interleave.
+struct SourceParts {
+  unsigned c0, c1;
+  bool rare;
+};
+__device__ __forceinline__ SourceParts source_parts(double a, double gq, int tk_hi) {
+  const u64 ba = (u64)__double_as_longlong(a), bg = (u64)__double_as_longlong(gq);
+  const unsigned ah = hi32(ba), al = lo32(ba), gh = hi32(bg), gl = lo32(bg);
+  const unsigned am = (ah & 0x000FFFFFu) | 0x00100000u, gm = (gh & 0x000FFFFFu) | 0x00100000u;
+  // a2 = floor(mantissa^2 2^-42), pr = floor(a2 gq's mantissa 2^-53): q_single's products
+  const u64 w = (u64)(2u * am) * al + hi32((u64)al * al);
+  const u64 a2 = (u64)(am << 11) * (am << 11) + (w >> 10);
+  const u64 w2 = (u64)lo32(a2) * gm + hi32((u64)lo32(a2) * gl);
+  const u64 w3 = (u64)hi32(a2) * gl + lo32(w2);
+  const u64 top = (u64)hi32(a2) * gm + hi32(w2) + hi32(w3);
+  const unsigned ph = __funnelshift_l(lo32(top), hi32(top), 11);
+  const unsigned pl = __funnelshift_l(lo32(w3), lo32(top), 11);
+  const int t = 2 * (int)((ah >> 20) & 0x7FFu) + (int)(gh >> 20) - 3162;  // Q = pr 2^t
+  // high word of q's bits as a double (q = pr 2^(t + 32), pr in [2^61, 2^64))
+  const int lz = __clz((int)ph);
+  const int e1022 = t - lz + 1117;
+  const int rh = (int)(__funnelshift_l(pl, ph, lz) >> 11) + (e1022 << 20);
+  SourceParts r;
+  r.rare = t > 0 || rh >= tk_hi;
+  // (A or gq zero or subnormal: t is below -64, and nothing is left)
+  const u64 Q = shr_clamp(((u64)ph << 32) | pl, (unsigned)-t);
+  r.c0 = lo32(Q);
+  r.c1 = hi32(Q);
+  return r;
+}
+
+// The deposit, the count and the candidate test; a source of the FP64 path, or one to keep as
+// a candidate, is appended to the warp's queue q (qn entries, the same in every lane; every
+// lane of the warp calls it together).  rep_lane: the replica of this lane's sources.
+__device__ __forceinline__ void deposit_source(const PlacedSource p, SourceParts c, long long s,
+                                               double a, const PrepassArgs& pa,
+                                               const HotBins& hot_bins, u64* rep_lane,
+                                               long long* q, int& qn, unsigned& nkappa) {
   const int lane = threadIdx.x & 31;
-  long long entry = s;
-  bool set_aside = false;
-  if (s < N) {
-    // finite inputs, and A^2 finite (|A| < 2^512): else the source is refused below
-    const bool fin = finite3(a, fs, fds) && (((u64)__double_as_longlong(a) >> 52) & 0x7FF) < 1535;
-    long long k0 = 0;
-    const bool single = fin && single_bin(fs, fds, g, &k0);
-    if (single) {
-      const long long j = k0 - g.k_lo;
-      u64 qb = 0;
-      if (j >= 0 && j < g.nb) {
-        u64 c0, c1, c2;
-        if (q_single(a, pa.tb.gq[j], &c0, &c1, &c2, &qb)) {
-          if (j < pa.rep.nbins)
-            add_parts_rep(pa.rep, pa.acc, j, (int)(s & (kAccReplicas - 1)), c0, c1, c2);
-          else
-            add_parts(pa.acc, j, c0, c1, c2);
-        } else {
-          qb = 0;
-          atomicOr(&pa.rs->err, ERR_RANGE);
-        }
-      }
-      set_aside = prepass_decide(__longlong_as_double((long long)qb), pa.tk_bits, pa.tl_bits,
-                                 nkappa);
-      entry |= kQueueKeep;
-    } else if (fin) {
-      set_aside = true;
-    } else {
-      atomicOr(&pa.rs->err, ERR_INPUT);  // the source is skipped; the run reports it
+  bool set_aside = p.j == -2, keep = false;
+  if (p.j >= 0) {
+    if (c.rare) {
+      u64 qb, c0, c1, c2;
+      if (!q_single(a, p.gq, &c0, &c1, &c2, &qb)) atomicOr(&pa.rs->err, ERR_RANGE);
+      c.c0 = lo32(c0);
+      c.c1 = lo32(c1);
+      if (c2) atomicAdd(pa.acc + 4 * (size_t)p.j + 2, c2);
+      keep = set_aside = prepass_decide(__longlong_as_double((long long)qb), pa.tk_bits,
+                                        pa.tl_bits, nkappa);
     }
+    if (p.j < hot_bins.n) {
+      hot_add(hot_bins, p.j, c.c0, c.c1);
+    } else {
+      u64* d = p.j < pa.rep.nbins ? rep_lane + 2 * (size_t)p.j : pa.acc + 4 * (size_t)p.j;
+      if (c.c0) atomicAdd(d, (u64)c.c0);
+      if (c.c1) atomicAdd(d + 1, (u64)c.c1);
+    }
+  } else if (p.j == -1) {
+    // outside the band: r = 0
+    if (pa.tk_bits == 0) ++nkappa;
   }
   const unsigned sm = __ballot_sync(0xFFFFFFFFu, set_aside);
-  if (set_aside) q[qn + __popc(sm & ((1u << lane) - 1u))] = entry;
-  qn += __popc(sm);
+  if (sm) {
+    if (set_aside) q[qn + __popc(sm & ((1u << lane) - 1u))] = keep ? s | kQueueKeep : s;
+    qn += __popc(sm);
+  }
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
+__device__ __forceinline__ bool mbar_try(uint32_t bar, unsigned parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      " selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 // Wait for phase `parity` of the barrier; false once *abort is set by another warp of the CTA,
 // or after about a second (2^31 clocks), or after 2^24 polls, whichever comes first.
-__device__ __forceinline__ bool mbar_wait_abort(uint64_t* bar, unsigned parity,
-                                                const int* abort) {
-  const uint32_t a = smem_addr(bar);
+__device__ __noinline__ bool mbar_poll(uint32_t bar, unsigned parity, const int* abort) {
   const long long t0 = clock64();
   for (int i = 0; i < (1 << 24); ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(a), "r"(parity)
-        : "memory");
-    if (ok) return true;
+    if (mbar_try(bar, parity)) return true;
     if ((i & 63) == 63) {
       if (*(volatile const int*)abort) return false;
       if (clock64() - t0 > (2LL << 30)) return false;
@@ -732,139 +807,160 @@ __device__ __forceinline__ bool mbar_wait_abort(uint64_t* bar, unsigned parity,
   }
   return false;
 }
+__device__ __forceinline__ bool mbar_wait_abort(uint64_t* bar, unsigned parity,
+                                                const int* abort) {
+  return mbar_try(smem_addr(bar), parity) || mbar_poll(smem_addr(bar), parity, abort);
+}
 
-__global__ void __launch_bounds__(kPrepassThreads, 3)
+__global__ void __launch_bounds__(kPrepassThreads, 1)
     k_prepass(const __grid_constant__ PrepassArgs pa) {
   RunState* const rs = pa.rs;
-  extern __shared__ __align__(128) double pre_tiles[];  // [stage][A | f | fdot][kPreTile]
-  __shared__ __align__(8) uint64_t full[kPreStages], empty[kPreStages];
-  __shared__ long long stage_tile[kPreStages];  // tile held by each stage
-  __shared__ long long slow_q[kPreConsumers][kSlowWarpCap];
+  // per warp [stage][A | f | fdot][kPreStep]; the warps' queues; the hot bins' words
+  extern __shared__ __align__(128) double pre_smem[];
+  __shared__ __align__(8) uint64_t full[kPreWarps][kPreStages];
   __shared__ int abort_flag;
   // the catalog record (and a generated catalog's constants), read once per CTA: every
   // thread of the grid loading it would queue on one L2 line
   __shared__ CatalogRef scat;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) {
     scat = *pa.cat;
-    for (int k = 0; k < kPreStages; ++k) {
-      mbar_init(&full[k], 1);
-      mbar_init(&empty[k], kPreConsumers);
-    }
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     abort_flag = 0;
   }
+  if (lane == 0) {
+    for (int k = 0; k < kPreStages; ++k) mbar_init(&full[warp][k], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
   __syncthreads();
-  const double* __restrict__ A = scat.A;
-  const double* __restrict__ f = scat.f;
-  const double* __restrict__ fdot = scat.fdot;
-  const long long N = scat.n;
-  const bool use_tma = scat.staged == kCatDevice;
   if (scat.staged == kCatGenerated) return;  // k_prepass_gen's catalog
-  const int lane = tid & 31;
-  const int warp = tid >> 5;
-  const long long ntiles = (N + kPreTile - 1) / kPreTile;
-  // full tiles of device memory come through TMA; the ragged one, and every tile of a catalog
-  // in host memory, through plain loads
-  const long long nfull = use_tma ? N / kPreTile : 0;
-
-  if (warp == kPreConsumers) {
-    // ------------------------------------------------ producer (one lane)
-    if (lane != 0) return;
-    // bit k of copying: the copies of stage k's latest tile were started, in its use of
-    // parity bit k of copy_par (they complete that phase of full[k])
-    unsigned copying = 0, copy_par = 0;  // bit k: stage k
-    for (long long i = 0;; ++i) {
-      const int stage = (int)(i % kPreStages);
-      const unsigned use = (unsigned)(i / kPreStages);
-      if (use > 0) {
-        // every consumer warp has let go of the stage's previous tile
-        if (!mbar_wait_abort(&empty[stage], (use - 1) & 1, &abort_flag)) {
+  const long long N = scat.n;
+  double* const stages = pre_smem + (size_t)warp * kPreStages * 3 * kPreStep;
+  long long* const myq = reinterpret_cast<long long*>(
+                             pre_smem + (size_t)kPreWarps * kPreStages * 3 * kPreStep) +
+                         warp * kSlowWarpCap;
+  HotBins hot;
+  hot.w = reinterpret_cast<unsigned*>(pre_smem + (size_t)kPreWarps *
+                                                     (kPreStages * 3 * kPreStep + kSlowWarpCap));
+  hot.n = N >= kHotMinSources && N < (1LL << 31) ? (int)min((long long)kHotBins, pa.rep.nbins) : 0;
+  if (hot.n) {
+    for (int j = tid; j < 3 * kHotBins; j += kPrepassThreads) hot.w[j] = 0u;
+    __syncthreads();
+  }
+  // steps [0, nfull) of device memory come through bulk copies; the ragged one, and every step
+  // of a catalog in host memory, through plain loads
+  const unsigned nsteps = (unsigned)((N + kPreStep - 1) / kPreStep);
+  const unsigned nfull = scat.staged == kCatDevice ? (unsigned)(N / kPreStep) : 0u;
+  unsigned started = 0;  // lane 0: bit k, copies of stage k are under way
+  unsigned par = 0;      // bit k: the phase of stage k's barrier that its copies complete
+  auto start_copies = [&](unsigned u, unsigned k) {
+    if (lane != 0 || u >= nfull || (pa.test_flags & 1)) return;
+    double* d = stages + k * 3 * kPreStep;
+    const size_t off = (size_t)u * kPreStep;
+    uint64_t* bar = &full[warp][k];
+    started |= 1u << k;
+    mbar_expect_tx(bar, 3u * kPreStep * (unsigned)sizeof(double));
+    bulk_g2s(d, scat.A + off, kPreStep * sizeof(double), bar);
+    bulk_g2s(d + kPreStep, scat.f + off, kPreStep * sizeof(double), bar);
+    bulk_g2s(d + 2 * kPreStep, scat.fdot + off, kPreStep * sizeof(double), bar);
+  };
+  // steps dealt out in turn over all warps of the grid (numbered across the CTAs, so that a small
+  // catalog spreads over the SMs)
+  const unsigned nwarps = gridDim.x * kPreWarps;
+  unsigned u_next = warp * gridDim.x + blockIdx.x;
+  auto take_step = [&]() {
+    const unsigned t = u_next;
+    u_next += nwarps;
+    return t;
+  };
+  static_assert(kPreStages == 2, "two stages, taken in turn");
+  unsigned u = take_step();
+  start_copies(u, 0);
+  unsigned u1 = take_step();
+  start_copies(u1, 1);
+  unsigned nkappa = 0;  // a lane's share of the catalog
+  // a source's replica is its index mod kAccReplicas, the same for all of a lane's sources
+  u64* const rep_lane = pa.rep.w + 2 * (size_t)(lane % kAccReplicas) * pa.rep.nbins;
+  int qn = 0;         // entries of the warp's queue (the same in every lane)
+  unsigned done = 0;  // steps done
+  bool timeout = false;
+  for (; u < nsteps; ++done) {
+    const unsigned k = done & 1u;
+    const long long s0 = (long long)u * kPreStep + lane;
+    double av[kPrePer], fv[kPrePer], dv[kPrePer];
+    if (u < nfull) {
+      const bool ok = mbar_wait_abort(&full[warp][k], (par >> k) & 1u, &abort_flag);
+      if (!__all_sync(0xFFFFFFFFu, ok)) {
+        if (lane == 0) {
           atomicOr(&rs->err, ERR_TIMEOUT);
           *(volatile int*)&abort_flag = 1;
-          break;
         }
-        copying &= ~(1u << stage);  // the consumers waited for those copies
+        timeout = true;
+        break;
       }
-      const long long t = (long long)atomicAdd(&rs->next_tile, 1ull);
-      stage_tile[stage] = t;
-      if (t < nfull && !(pa.test_flags & 1)) {
-        copying |= 1u << stage;
-        copy_par = (copy_par & ~(1u << stage)) | ((use & 1u) << stage);
-        double* d = pre_tiles + (size_t)stage * 3 * kPreTile;
-        const size_t off = (size_t)t * kPreTile;
-        mbar_expect_tx(&full[stage], 3u * kPreTile * (unsigned)sizeof(double));
-        bulk_g2s(d, A + off, kPreTile * sizeof(double), &full[stage]);
-        bulk_g2s(d + kPreTile, f + off, kPreTile * sizeof(double), &full[stage]);
-        bulk_g2s(d + 2 * kPreTile, fdot + off, kPreTile * sizeof(double), &full[stage]);
-      } else if (t >= nfull) {
-        mbar_arrive(&full[stage]);  // a ragged or mapped tile, or the end
-      }
-      // (with the test hook a full tile gets no copy and no arrival: its waits run out)
-      if (t >= ntiles) break;
-    }
-    if (*(volatile int*)&abort_flag) {
-      // the consumers gave up: wait (bounded) for every copy this CTA started before its
-      // shared memory goes away
-      for (int k = 0; k < kPreStages; ++k)
-        if ((copying >> k) & 1u) mbar_wait(&full[k], (copy_par >> k) & 1u);
-    }
-    return;
-  }
-
-  // -------------------------------------------------- consumers
-  unsigned nkappa = 0;  // a lane's share of the catalog
-  long long* myq = slow_q[warp];
-  int qn = 0;  // entries of the warp's queue (the same in every lane)
-  for (long long i = 0;; ++i) {
-    const int stage = (int)(i % kPreStages);
-    const unsigned use = (unsigned)(i / kPreStages);
-    const bool ok = mbar_wait_abort(&full[stage], use & 1, &abort_flag);
-    if (!__all_sync(0xFFFFFFFFu, ok)) {
-      if (lane == 0) {
-        atomicOr(&rs->err, ERR_TIMEOUT);
-        *(volatile int*)&abort_flag = 1;
-      }
-      return;
-    }
-    const long long t = stage_tile[stage];
-    if (t >= ntiles) break;
-    const bool staged = t < nfull;
-    const double* sA = pre_tiles + (size_t)stage * 3 * kPreTile;
-    const double* sF = sA + kPreTile;
-    const double* sD = sF + kPreTile;
-    const int base = warp * kPreWarpSrc + lane;
-    // every load of the lane's sources first: from host memory each one takes a
-    // microsecond or more
-    double av[kPrePer], fv[kPrePer], dv[kPrePer];
+      par ^= 1u << k;
+      started &= ~(1u << k);
+      const double* d = stages + k * 3 * kPreStep + lane;
 #pragma unroll
-    for (int k = 0; k < kPrePer; ++k) {
-      const int idx = base + 32 * k;
-      const long long s = t * kPreTile + idx;
-      av[k] = fv[k] = dv[k] = 0.0;
-      if (staged) {
-        av[k] = sA[idx];
-        fv[k] = sF[idx];
-        dv[k] = sD[idx];
-      } else if (s < N) {
-        av[k] = A[s];
-        fv[k] = f[s];
-        dv[k] = fdot[s];
+      for (int i = 0; i < kPrePer; ++i) {
+        av[i] = d[32 * i];
+        fv[i] = d[kPreStep + 32 * i];
+        dv[i] = d[2 * kPreStep + 32 * i];
+      }
+    } else {
+      // every load of the lane's sources first: from host memory each one takes a microsecond
+      // or more
+#pragma unroll
+      for (int i = 0; i < kPrePer; ++i) {
+        const long long s = s0 + 32 * i;
+        av[i] = fv[i] = dv[i] = 0.0;
+        if (s < N) {
+          av[i] = scat.A[s];
+          fv[i] = scat.f[s];
+          dv[i] = scat.fdot[s];
+        }
       }
     }
-    // the stage may be refilled once every warp has its values in registers
+    // every lane has its values: the stage takes a later step
     __syncwarp();
-    if (lane == 0) mbar_arrive(&empty[stage]);
+    u = u1;
+    u1 = take_step();
+    start_copies(u1, k);
+    PlacedSource pl[kPrePer];
 #pragma unroll
-    for (int k = 0; k < kPrePer; ++k)
-      prepass_source(t * kPreTile + base + 32 * k, N, av[k], fv[k], dv[k], pa, myq, qn, nkappa);
+    for (int i = 0; i < kPrePer; ++i)
+      pl[i] = place_source(s0 + 32 * i < N, av[i], fv[i], dv[i], pa);
+    SourceParts sp[kPrePer];
+#pragma unroll
+    for (int i = 0; i < kPrePer; ++i) sp[i] = source_parts(av[i], pl[i].gq, pa.tk_hi);
+#pragma unroll
+    for (int i = 0; i < kPrePer; ++i)
+      deposit_source(pl[i], sp[i], s0 + 32 * i, av[i], pa, hot, rep_lane, myq, qn, nkappa);
     prepass_drain_full<false>(pa, &scat, myq, qn, nkappa);
   }
-  __syncwarp();
-  if (qn > 0)
+  if (timeout) {
+    // wait (bounded) for every copy this warp started before its shared memory goes away
+    if (lane == 0)
+      for (int k = 0; k < kPreStages; ++k)
+        if ((started >> k) & 1u) mbar_wait(&full[warp][k], (par >> k) & 1u);
+    __syncwarp();
+  } else if (qn > 0) {
+    __syncwarp();
     nkappa += prepass_drain_warp<false>(pa, &scat, myq, qn);
+  }
   for (int o = 16; o > 0; o >>= 1) nkappa += __shfl_xor_sync(0xFFFFFFFFu, nkappa, o);
   if (lane == 0 && nkappa) atomicAdd(&rs->ncand, (unsigned long long)nkappa);
+  if (hot.n) {
+    // the hot bins' words into the replicas, a few CTAs to each
+    __syncthreads();
+    if (tid == 0) atomicOr(&rs->spec, (int)kSpecCarried);
+    u64* const r = pa.rep.w + 2 * (size_t)(blockIdx.x % kAccReplicas) * pa.rep.nbins;
+    for (int j = tid; j < hot.n; j += kPrepassThreads) {
+      const unsigned h0 = hot.w[j], h1 = hot.w[kHotBins + j], h2 = hot.w[2 * kHotBins + j];
+      if (h0) atomicAdd(r + 2 * j, (u64)h0);
+      if (h1) atomicAdd(r + 2 * j + 1, (u64)h1);
+      if (h2) atomicAdd(pa.acc + 4 * (size_t)j + 2, (u64)h2);
+    }
+  }
 }
 
 // The catalog pass over a generated catalog: every source computed from (seed, index) where
@@ -886,6 +982,8 @@ __global__ void __launch_bounds__(kGenThreads, 4)
   const long long N = scat.n;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned nkappa = 0;  // a lane's share of the catalog
+  // a source's replica is its index mod kAccReplicas, the same for all of a lane's sources
+  u64* const rep_lane = pa.rep.w + 2 * (size_t)(lane % kAccReplicas) * pa.rep.nbins;
   long long* myq = slow_q[warp];
   int qn = 0;
   constexpr long long kRun = 32LL * kGenPer;
@@ -899,7 +997,9 @@ __global__ void __launch_bounds__(kGenThreads, 4)
       const long long s = base + 32 * k + lane;
       double3 src = make_double3(0.0, 0.0, 0.0);
       if (s < N) src = gen_source_at(&scat, s);
-      prepass_source(s, N, src.x, src.y, src.z, pa, myq, qn, nkappa);
+      const PlacedSource pl = place_source(s < N, src.x, src.y, src.z, pa);
+      deposit_source(pl, source_parts(src.x, pl.gq, pa.tk_hi), s, src.x, pa, HotBins{nullptr, 0},
+                     rep_lane, myq, qn, nkappa);
       prepass_drain_full<true>(pa, &scat, myq, qn, nkappa);
     }
   }
@@ -913,15 +1013,16 @@ __global__ void __launch_bounds__(kGenThreads, 4)
 void launch_prepass(const CatalogRef* cat, long long cap, const Grid& g, const Tables& tb,
                     double thr_kappa, double thr_live, unsigned long long* acc, AccReplicas rep,
                     Cands cd, RunState* rs, int nsm, int test_flags, cudaStream_t st) {
-  long long tiles = (cap + kPreTile - 1) / kPreTile;
-  long long lim = (long long)nsm * 3;  // resident CTAs (launch bounds, shared memory)
-  int bl = (int)(tiles < lim ? (tiles < 1 ? 1 : tiles) : lim);
+  // one CTA per SM, at most one per step of the catalog
+  const long long steps = (cap + kPreStep - 1) / kPreStep;
+  const int bl = (int)(steps < nsm ? (steps < 1 ? 1 : steps) : nsm);
   PrepassArgs pa;
   pa.cat = cat;
   pa.g = g;
   pa.tb = tb;
   memcpy(&pa.tk_bits, &thr_kappa, sizeof(double));
   memcpy(&pa.tl_bits, &thr_live, sizeof(double));
+  pa.tk_hi = pa.tk_bits ? (int)(pa.tk_bits >> 32) : INT_MIN;
   pa.acc = acc;
   pa.rep = rep;
   pa.cd = cd;
@@ -1403,7 +1504,7 @@ __global__ void __launch_bounds__(1024, E == 2 ? 2 : 1) k_chunk_sort(SpecIn in, 
   uint16_t* sm_idx = (uint16_t*)(sm_keys + pl.kpad);
   const int T = blockDim.x, tid = threadIdx.x;
   const int kpad = pl.kpad;  // = T * E
-  const ListHead head = list_head(d, kListR0, pl.nch, in.tree);
+  const ListHead head = list_head(d, kListR0, pl.nch, in.flags);
   const int nitem = head.count;
   // after the first iteration of a tracked run every chunk holds the sorted state of its
   // previous values
@@ -1427,7 +1528,7 @@ __global__ void __launch_bounds__(1024, E == 2 ? 2 : 1) k_chunk_sort(SpecIn in, 
     for (int a = 0; a < E; ++a) {
       const int i = tid * E + a;
       K kv = (K)~(K)0;
-      if (i < len) kv = sort_key<K>(spec_value<kSpec>(in, base + i, head.tree != 0), pl.key_scale);
+      if (i < len) kv = sort_key<K>(spec_value<kSpec>(in, base + i, head.flags), pl.key_scale);
       k[a] = kv;
       x[a] = i;
     }
@@ -1960,14 +2061,14 @@ __global__ void __launch_bounds__(512, 2) k_median_wm(
     double r = median_tile<K>(skey, srank, n, pl, o, u, sm_raw, zeros);
     relmax = r > relmax ? r : relmax;
     __syncthreads();  // before the next tile overwrites shared memory
-    if (head.tree) {
+    if (head.flags) {
       // nodes whose bins all lie in this tile's outputs [(u-1) Kc + h, u Kc + h)
       const long long a = (long long)(u - 1) * pl.Kc + pl.W / 2, b = a + pl.Kc;
       const long long n1 = o.tree.n[0], na = a > 0 ? (a + 31) >> 5 : 0;
       tree_h_nodes(o, (int)na, (int)min(b >> 5, n1));
     }
   }
-  if (head.tree && last_cta(&o.rs->ticket)) {
+  if (head.flags && last_cta(&o.rs->ticket)) {
     // the nodes that straddle two tiles, then the levels above
     if ((pl.W / 2) & 31)
       tree_h_straddle(o.Gf, o.inv_f, o.tree.h, o.tree.n[0], pl.Kc, pl.W / 2, pl.nch);
@@ -2024,7 +2125,7 @@ __device__ __forceinline__ void chunk_prefix(const SpecIn& in, long long n, cons
                                              unsigned long long* __restrict__ pre_hi,
                                              int* __restrict__ sig, unsigned* __restrict__ uflow,
                                              double* __restrict__ x_out, int b, U128* warp_tot,
-                                             u64* warp_max, int& any_uf, bool tree) {
+                                             u64* warp_max, int& any_uf, int flags) {
   const long long base = (long long)b * pl.Kc;
   const int len = (int)((n - base) < pl.Kc ? (n - base) : pl.Kc);
   const int per = (pl.Kc + blockDim.x - 1) / blockDim.x;
@@ -2039,7 +2140,7 @@ __device__ __forceinline__ void chunk_prefix(const SpecIn& in, long long n, cons
       int p = p0 + i;
       double x = 0.0;
       if (p < len) {
-        x = spec_value<kSpec>(in, base + p, tree);
+        x = spec_value<kSpec>(in, base + p, flags);
         if (x_out) x_out[base + p] = x;
       }
       v[i] = x;
@@ -2140,14 +2241,14 @@ __global__ void k_chunk_prefix(SpecIn in, long long n, SmoothPlan pl,
   __shared__ int any_uf;
   // chunks whose input changed (a chunk within in_radius of them is dirty)
   const int list = kListR0 + in_radius;
-  const ListHead head = list_head(d, list, pl.nch, in.tree);
+  const ListHead head = list_head(d, list, pl.nch, in.flags);
   const int nitem = head.count;
   int b_next = head.first;
   for (int it = blockIdx.x; it < nitem; it += gridDim.x) {
     const int b = b_next;
     if (it + (int)gridDim.x < nitem) b_next = d.item(list, it + gridDim.x);
     chunk_prefix<kSpec>(in, n, pl, pre_lo, pre_hi, sig, uflow, x_out, b, warp_tot,
-                 warp_max, any_uf, head.tree != 0);
+                 warp_max, any_uf, head.flags);
     __syncthreads();
   }
 }
@@ -2229,13 +2330,13 @@ __global__ void k_window_mean(const double* __restrict__ x, long long n, SmoothP
       double rel = sg_store(o, j, v, &inv);
       relmax = rel > relmax ? rel : relmax;
       // chunks and warps start on multiples of 32 bins: a warp holds one node of level 1
-      if (kTree && head.tree && (j | 31) < n) {
+      if (kTree && head.flags && (j | 31) < n) {
         const float hv = warp_sum_f32(__fmul_rn(o.Gf[j], inv));
         if ((threadIdx.x & 31) == 0) o.tree.h[j >> 5] = hv;
       }
     }
   }
-  if (kTree && head.tree && last_cta(&o.rs->ticket)) tree_h_levels(o.tree);
+  if (kTree && head.flags && last_cta(&o.rs->ticket)) tree_h_levels(o.tree);
   if (o.rtol_on) warp_max_atomic((u64)__double_as_longlong(relmax), &o.rs->relchg_bits);
 }
 

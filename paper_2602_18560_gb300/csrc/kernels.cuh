@@ -49,6 +49,14 @@ struct Tree {
   int g;
 };
 
+// Properties of a run's spectrum (RunState::spec).
+//   kSpecTree    : a source was deposited into the tree's nodes.
+//   kSpecCarried : the catalog pass added up the first bins in shared memory, carrying from
+//     word to word.  Removing a source still subtracts its own three parts, so words 0 and 1
+//     may go below zero and are read as signed numbers; only for catalogs of less than 2^31
+//     sources, whose sums of 32-bit parts stay below 2^63.
+enum { kSpecTree = 1, kSpecCarried = 2 };
+
 // Loop state kept on the device for one run.
 struct RunState {
   int iter;              // iterations completed
@@ -68,7 +76,7 @@ struct RunState {
   unsigned long long nuncertain; // FP32 decisions (mixed precision) inside the screen's bound
   unsigned long long nwide;      // entries of Cands::wide
   unsigned err;
-  int tree;              // 1: a source was deposited into the tree's nodes
+  int spec;              // kSpecTree, kSpecCarried: how the spectrum's words are read
   int tree_live;         // 1: a kept candidate's sweep is in the tree
   unsigned ticket;       // CTAs done with the kernel that writes the node sums h
 };
@@ -78,12 +86,12 @@ struct Grid {
   double T, T2, t5;      // T_obs, T_obs^2, T_obs / 5
   long long k_lo;        // first DFT index in band
   long long nb;          // bins in band
-  unsigned long long mT; // T_obs = mT 2^eT, mT the 53-bit integer mantissa
-  int eT;
+  // T_obs = (tq 2^32 + tr) 2^(etq - 32), tq in [2^31, 2^32) (source_bin); ebin - e is the count
+  // of fraction bits beyond 23 of f tq for a mantissa exponent e of f (negative for every e
+  // when T_obs is so extreme that f's exponent could leave the normal range)
+  unsigned tq, tr;
+  int ebin;
   float T2f;             // T_obs^2 in FP32
-  unsigned tq;           // T_obs = tq 2^etq with tq odd, when it fits in 32 bits (short_t)
-  int etq;
-  int short_t;
 };
 
 // Per-bin tables, built once per context.
@@ -119,7 +127,7 @@ struct SpecIn {
   const double* gq;               // Tables::gq and Tree::g (the tree's share of a bin)
   long long nb;                   // bins in band
   int g;
-  const int* tree;                // RunState::tree
+  const int* flags;               // RunState::spec
 };
 
 // Chunks whose input changed since the previous iteration.  Two byte arrays of nch
@@ -193,18 +201,18 @@ struct DirtyIter {
 // shared with the CTA: when every thread of hundreds of CTAs loads the same words, the
 // requests queue on one L2 line and a late iteration's few working CTAs wait behind them.
 struct ListHead {
-  int count, first, iter, tree;
+  int count, first, iter, flags;
 };
-// tree (may be null): a flag of the loop state read along with them.
+// flags (may be null): a word of the loop state read along with them.
 __device__ __forceinline__ ListHead list_head(const Dirty& d, int which, int all,
-                                              const int* tree) {
+                                              const int* flags) {
   __shared__ ListHead sh;
   if (threadIdx.x == 0) {
     ListHead h;
     h.count = d.count(which, all);
     h.first = d.item(which, blockIdx.x);  // the grid is never longer than the list
     h.iter = d.base ? d.rs->iter : 0;
-    h.tree = tree ? *tree : 0;
+    h.flags = flags ? *flags : 0;
     sh = h;
   }
   __syncthreads();

@@ -108,7 +108,7 @@ extern "C" int sub_running_mean_noalloc(const double* x, double* out, int64_t n,
   in.gq = nullptr;
   in.nb = n;
   in.g = 0;
-  in.tree = nullptr;
+  in.flags = nullptr;
   SgOut o = {};
   o.out = out;
   o.inv_f = nullptr;
