@@ -599,8 +599,11 @@ static void enqueue_estimate(sub_ctx* c, cudaStream_t st, SpecIn in, int rtol_on
   if (!with_inv) o.tree.h = nullptr;
   switch (c->p.estimator) {
     case SUB_MEAN: {
-      { KTimer t(c, st, SUB_K_PREFIX); launch_chunk_prefix(in, n, pl, c->pre_lo, c->pre_hi, c->sig, c->uflow, c->P, d, 0, st); }
-      { KTimer t(c, st, SUB_K_MEAN); launch_window_mean(c->P, n, pl, c->pre_lo, c->pre_hi, c->sig, c->uflow, o, d, 1, st); }
+      // the window means add up inputs directly where a sum is tiny: the spectrum's values go
+      // through P, a plain array is read where it is
+      const double* x = in.acc ? c->P : in.x;
+      { KTimer t(c, st, SUB_K_PREFIX); launch_chunk_prefix(in, n, pl, c->pre_lo, c->pre_hi, c->sig, c->uflow, in.acc ? c->P : nullptr, d, 0, st); }
+      { KTimer t(c, st, SUB_K_MEAN); launch_window_mean(x, n, pl, c->pre_lo, c->pre_hi, c->sig, c->uflow, o, d, 1, st); }
       break;
     }
     case SUB_MEDIAN: {

@@ -88,19 +88,26 @@ __device__ __forceinline__ double scale_pow2(double x, int k) {
   return ldexp(x, k);
 }
 
-// Round-to-nearest double of v * 2^-sh.
+// Round-to-nearest double of v * 2^-sh.  The rounding is done on the integer (a conversion
+// of a 64-bit integer to double goes through the FP64 pipe, which takes a warp instruction
+// every 64 clocks of a scheduler); only a result outside the normal range takes that path.
 __device__ __forceinline__ double u128_to_dbl_scaled(U128 v, int sh) {
-  if (v.hi == 0ull) {
-    if (v.lo == 0ull) return 0.0;
-    return scale_pow2(__ull2double_rn(v.lo), -sh);
+  if (u128_is_zero(v)) return 0.0;
+  // v = top 2^shift with the top bit of top set, up to the low bits, which become a sticky
+  // bit so that the rounding stays correct
+  const bool wide = v.hi != 0ull;
+  const int lz = __clzll((i64)(wide ? v.hi : v.lo));
+  u64 top = (wide ? v.hi : v.lo) << lz;
+  if (wide && lz) top |= v.lo >> (64 - lz);
+  if (wide && (v.lo << lz) != 0ull) top |= 1ull;
+  const int shift = wide ? 64 - lz : -lz;
+  const int e = 1086 + shift - sh;  // exponent field of the result
+  if (e >= 1 && e <= 2045) {
+    u64 m = top >> 11;
+    const unsigned rem = (unsigned)top & 0x7FFu;
+    m += (rem > 0x400u || (rem == 0x400u && (m & 1ull))) ? 1ull : 0ull;
+    return __longlong_as_double((i64)(((u64)(e - 1) << 52) + m));  // a carry moves the exponent
   }
-  int lz = __clzll((i64)v.hi);      // 0..63
-  int shift = 64 - lz;              // bits to drop so the top 64 bits remain
-  u64 top = (v.hi << lz) | (lz ? (v.lo >> (64 - lz)) : 0ull);
-  // the discarded low bits become a sticky bit so that rounding stays correct
-  u64 low_mask = (lz == 0) ? ~0ull : ((1ull << (64 - lz)) - 1ull);
-  u64 sticky = ((v.lo & low_mask) != 0ull) ? 1ull : 0ull;
-  top |= sticky;
   return scale_pow2(__ull2double_rn(top), shift - sh);
 }
 

@@ -2118,35 +2118,59 @@ __device__ __forceinline__ int sigma_from_max(u64 maxbits) {
   return 1136 - e;
 }
 
-// Prefix sums of chunk b.
-template <bool kSpec>
+// Prefix sums of chunk b: kPer consecutive values per thread, loaded and stored in pairs where
+// the chunk is whole (pairs: a plain array starts on 16 bytes, as the library's own do).
+//
+// Bound: latency of one chunk (a maximum, a scan, two barriers each), so what counts is how
+// many chunks an SM works on at once.  With one value per thread a chunk of 1024 bins took the
+// SM alone (1024 threads of 56 registers).  1.25e6 bins, W = 1000, start -> now: 31 -> 13 us from
+// an array, 33 -> 28 us from the spectrum (W = 2000); running mean of 312 422 bins with its
+// window means 29.7 -> 18.4 us.
+template <bool kSpec, int kPer>
 __device__ __forceinline__ void chunk_prefix(const SpecIn& in, long long n, const SmoothPlan& pl,
                                              unsigned long long* __restrict__ pre_lo,
                                              unsigned long long* __restrict__ pre_hi,
                                              int* __restrict__ sig, unsigned* __restrict__ uflow,
                                              double* __restrict__ x_out, int b, U128* warp_tot,
-                                             u64* warp_max, int& any_uf, int flags) {
+                                             u64* warp_max, int& any_uf, int flags, bool pairs) {
   const long long base = (long long)b * pl.Kc;
   const int len = (int)((n - base) < pl.Kc ? (n - base) : pl.Kc);
-  const int per = (pl.Kc + blockDim.x - 1) / blockDim.x;
-  const int p0 = threadIdx.x * per;
+  const int p0 = threadIdx.x * kPer;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  const bool whole = p0 + kPer <= len;
   // pass 1: values and the chunk maximum
-  double v[8];  // per <= 8 (Kc <= 8192 with 1024 threads)
+  double v[kPer];
   u64 mb = 0;
+  if (kSpec) {
+    // a bin of the spectrum is 40 bytes in two arrays: neighbouring threads take neighbouring
+    // bins, and hand them over through shared memory
+    extern __shared__ double prefix_x[];  // [kPer blockDim.x]
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    if (i < per) {
-      int p = p0 + i;
-      double x = 0.0;
-      if (p < len) {
-        x = spec_value<kSpec>(in, base + p, flags);
-        if (x_out) x_out[base + p] = x;
-      }
-      v[i] = x;
-      u64 bits = (u64)__double_as_longlong(x);
-      if (!(bits >> 63) && bits > mb) mb = bits;
+    for (int i = 0; i < kPer; ++i) {
+      const int p = threadIdx.x + i * blockDim.x;
+      const double x = p < len ? spec_value<true>(in, base + p, flags) : 0.0;
+      prefix_x[p] = x;
+      if (x_out && p < len) x_out[base + p] = x;
     }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) v[i] = prefix_x[p0 + i];
+  } else if (whole && pairs) {
+#pragma unroll
+    for (int i = 0; i < kPer; i += 2) {
+      const double2 w = *reinterpret_cast<const double2*>(in.x + base + p0 + i);
+      v[i] = w.x;
+      v[i + 1] = w.y;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < kPer; ++i)
+      v[i] = p0 + i < len ? in.x[base + p0 + i] : 0.0;
+  }
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    const u64 bits = (u64)__double_as_longlong(v[i]);
+    if (!(bits >> 63) && bits > mb) mb = bits;
   }
   for (int o = 16; o > 0; o >>= 1) {
     u64 t = __shfl_xor_sync(0xFFFFFFFFu, mb, o);
@@ -2155,87 +2179,99 @@ __device__ __forceinline__ void chunk_prefix(const SpecIn& in, long long n, cons
   if (lane == 0) warp_max[warp] = mb;
   if (threadIdx.x == 0) any_uf = 0;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    u64 t = threadIdx.x < nwarp ? warp_max[threadIdx.x] : 0ull;
-    for (int o = 16; o > 0; o >>= 1) {
-      u64 u = __shfl_xor_sync(0xFFFFFFFFu, t, o);
-      t = u > t ? u : t;
-    }
-    if (threadIdx.x == 0) warp_max[0] = t;
+  // every warp takes the maximum over the warps itself
+  mb = lane < nwarp ? warp_max[lane] : 0ull;
+  for (int o = 16; o > 0; o >>= 1) {
+    u64 t = __shfl_xor_sync(0xFFFFFFFFu, mb, o);
+    mb = t > mb ? t : mb;
   }
-  __syncthreads();
-  const int sigma = sigma_from_max(warp_max[0]);
-  if (warp_max[0] == 0ull) {
+  const int sigma = sigma_from_max(mb);
+  u64 lo[kPer], hi[kPer];
+  if (mb == 0ull) {
     // a chunk of zeros: every prefix is 0 and nothing fell below one unit
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      if (i < per && p0 + i < len) {
-        pre_lo[base + p0 + i] = 0ull;
-        pre_hi[base + p0 + i] = 0ull;
-      }
-    }
+    for (int i = 0; i < kPer; ++i) lo[i] = hi[i] = 0ull;
     if (threadIdx.x == 0) {
       uflow[b] = 0u;
       sig[b] = sigma;
     }
-    return;
-  }
-  // pass 2: thread totals in fixed point; note inputs > 0 below one unit
-  U128 run{0ull, 0ull};
-  int uf = 0;
+  } else {
+    // pass 2: the thread's prefixes in fixed point; note inputs > 0 below one unit
+    U128 run{0ull, 0ull};
+    int uf = 0;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    if (i < per && p0 + i < len) {
-      U128 q = dbl_to_u128_scaled(v[i], sigma);
+    for (int i = 0; i < kPer; ++i) {
+      const U128 q = dbl_to_u128_scaled(v[i], sigma);
       if (v[i] > 0.0 && u128_is_zero(q)) uf = 1;
       run = u128_add(run, q);
+      lo[i] = run.lo;
+      hi[i] = run.hi;
     }
-  }
-  if (uf) any_uf = 1;
-  // exclusive scan of thread totals
-  U128 inc = run;
-  for (int o = 1; o < 32; o <<= 1) {
-    U128 t;
-    t.lo = __shfl_up_sync(0xFFFFFFFFu, inc.lo, o);
-    t.hi = __shfl_up_sync(0xFFFFFFFFu, inc.hi, o);
-    if (lane >= o) inc = u128_add(inc, t);
-  }
-  if (lane == 31) warp_tot[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    U128 t2 = lane < nwarp ? warp_tot[lane] : U128{0ull, 0ull};
+    if (uf) any_uf = 1;
+    // exclusive scan of thread totals
+    U128 inc = run;
     for (int o = 1; o < 32; o <<= 1) {
       U128 t;
-      t.lo = __shfl_up_sync(0xFFFFFFFFu, t2.lo, o);
-      t.hi = __shfl_up_sync(0xFFFFFFFFu, t2.hi, o);
-      if (lane >= o) t2 = u128_add(t2, t);
+      t.lo = __shfl_up_sync(0xFFFFFFFFu, inc.lo, o);
+      t.hi = __shfl_up_sync(0xFFFFFFFFu, inc.hi, o);
+      if (lane >= o) inc = u128_add(inc, t);
     }
-    if (lane < nwarp) warp_tot[lane] = t2;  // inclusive over warps
-  }
-  __syncthreads();
-  U128 offs = u128_sub(inc, run);  // exclusive within warp
-  if (warp > 0) offs = u128_add(offs, warp_tot[warp - 1]);
-  // pass 3: write inclusive prefixes
+    if (lane == 31) warp_tot[warp] = inc;
+    __syncthreads();
+    // the warps before this one
+    U128 offs = lane < warp ? warp_tot[lane] : U128{0ull, 0ull};
+    for (int o = 16; o > 0; o >>= 1) {
+      U128 t;
+      t.lo = __shfl_xor_sync(0xFFFFFFFFu, offs.lo, o);
+      t.hi = __shfl_xor_sync(0xFFFFFFFFu, offs.hi, o);
+      offs = u128_add(offs, t);
+    }
+    offs = u128_add(offs, u128_sub(inc, run));  // exclusive within warp
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    if (i < per && p0 + i < len) {
-      offs = u128_add(offs, dbl_to_u128_scaled(v[i], sigma));
-      pre_lo[base + p0 + i] = offs.lo;
-      pre_hi[base + p0 + i] = offs.hi;
+    for (int i = 0; i < kPer; ++i) {
+      const U128 q = u128_add(offs, U128{lo[i], hi[i]});
+      lo[i] = q.lo;
+      hi[i] = q.hi;
+    }
+    if (threadIdx.x == 0) {
+      uflow[b] = (unsigned)any_uf;
+      sig[b] = sigma;
     }
   }
-  if (threadIdx.x == 0) {
-    uflow[b] = (unsigned)any_uf;
-    sig[b] = sigma;
+  // the inclusive prefixes
+  if (whole) {
+#pragma unroll
+    for (int i = 0; i < kPer; i += 2) {
+      *reinterpret_cast<ulonglong2*>(pre_lo + base + p0 + i) = make_ulonglong2(lo[i], lo[i + 1]);
+      *reinterpret_cast<ulonglong2*>(pre_hi + base + p0 + i) = make_ulonglong2(hi[i], hi[i + 1]);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < kPer; ++i)
+      if (p0 + i < len) {
+        pre_lo[base + p0 + i] = lo[i];
+        pre_hi[base + p0 + i] = hi[i];
+      }
   }
 }
 
-template <bool kSpec>
-__global__ void k_chunk_prefix(SpecIn in, long long n, SmoothPlan pl,
-                               unsigned long long* __restrict__ pre_lo,
-                               unsigned long long* __restrict__ pre_hi, int* __restrict__ sig,
-                               unsigned* __restrict__ uflow, double* __restrict__ x_out, Dirty d,
-                               int in_radius) {
+// Values per thread: at most 1024 threads for chunks of up to 8192 bins, and few registers.
+constexpr int kPrefixPer = 4, kPrefixPerLong = 8;
+static int prefix_per(const SmoothPlan& pl) { return pl.Kc > 4096 ? kPrefixPerLong : kPrefixPer; }
+static size_t prefix_smem(const SmoothPlan& pl, bool spec) {
+  return spec ? (size_t)prefix_per(pl) * ((pl.Kc / prefix_per(pl) + 31) / 32 * 32) * sizeof(double)
+              : 0;
+}
+static int prefix_threads(const SmoothPlan& pl) {
+  return (pl.Kc / prefix_per(pl) + 31) / 32 * 32;
+}
+
+template <bool kSpec, int kPer>
+__global__ void __launch_bounds__(1024)
+    k_chunk_prefix(SpecIn in, long long n, SmoothPlan pl, unsigned long long* __restrict__ pre_lo,
+                   unsigned long long* __restrict__ pre_hi, int* __restrict__ sig,
+                   unsigned* __restrict__ uflow, double* __restrict__ x_out, Dirty d,
+                   int in_radius) {
   __shared__ U128 warp_tot[32];
   __shared__ u64 warp_max[32];
   __shared__ int any_uf;
@@ -2243,12 +2279,13 @@ __global__ void k_chunk_prefix(SpecIn in, long long n, SmoothPlan pl,
   const int list = kListR0 + in_radius;
   const ListHead head = list_head(d, list, pl.nch, in.flags);
   const int nitem = head.count;
+  const bool pairs = (reinterpret_cast<uintptr_t>(in.x) & 15u) == 0;
   int b_next = head.first;
   for (int it = blockIdx.x; it < nitem; it += gridDim.x) {
     const int b = b_next;
     if (it + (int)gridDim.x < nitem) b_next = d.item(list, it + gridDim.x);
-    chunk_prefix<kSpec>(in, n, pl, pre_lo, pre_hi, sig, uflow, x_out, b, warp_tot,
-                 warp_max, any_uf, head.flags);
+    chunk_prefix<kSpec, kPer>(in, n, pl, pre_lo, pre_hi, sig, uflow, x_out, b, warp_tot, warp_max,
+                              any_uf, head.flags, pairs);
     __syncthreads();
   }
 }
@@ -2256,41 +2293,45 @@ __global__ void k_chunk_prefix(SpecIn in, long long n, SmoothPlan pl,
 void launch_chunk_prefix(SpecIn in, long long n, const SmoothPlan& pl, unsigned long long* pre_lo,
                          unsigned long long* pre_hi, int* sig, unsigned* uflow, double* x_out,
                          Dirty d, int in_radius, cudaStream_t st) {
-  int th = pl.Kc < 1024 ? pl.Kc : 1024;  // at most 8 values per thread
-  int bl = persistent_grid(pl, pl.nch, pl.res_prefix);
-  if (in.acc)
-    k_chunk_prefix<true>
-        <<<bl, th, 0, st>>>(in, n, pl, pre_lo, pre_hi, sig, uflow, x_out, d, in_radius);
-  else
-    k_chunk_prefix<false>
-        <<<bl, th, 0, st>>>(in, n, pl, pre_lo, pre_hi, sig, uflow, x_out, d, in_radius);
+  const int th = prefix_threads(pl), bl = persistent_grid(pl, pl.nch, pl.res_prefix);
+  auto launch = [&](auto kern) {
+    kern<<<bl, th, prefix_smem(pl, in.acc != nullptr), st>>>(in, n, pl, pre_lo, pre_hi, sig, uflow,
+                                                             x_out, d, in_radius);
+  };
+  if (prefix_per(pl) == kPrefixPer) {
+    if (in.acc) launch(k_chunk_prefix<true, kPrefixPer>);
+    else launch(k_chunk_prefix<false, kPrefixPer>);
+  } else {
+    if (in.acc) launch(k_chunk_prefix<true, kPrefixPerLong>);
+    else launch(k_chunk_prefix<false, kPrefixPerLong>);
+  }
 }
 
-// Sum of x[a .. e] inside one chunk as a double (a, e in the chunk, a <= e).
-__device__ __forceinline__ double part_sum(const double* __restrict__ x, long long cbase, long long a,
-                                           long long e, const unsigned long long* __restrict__ pre_lo,
-                                           const unsigned long long* __restrict__ pre_hi, int sigma,
-                                           unsigned uf) {
-  U128 pe{pre_lo[e], pre_hi[e]};
-  U128 sum = pe;
-  if (a > cbase) sum = u128_sub(pe, U128{pre_lo[a - 1], pre_hi[a - 1]});
-  long long cnt = e - a + 1;
+// A window's share of one chunk, units 2^-sigma of its bins [a, e]: the sum as a double.
+__device__ __forceinline__ double part_sum(const double* __restrict__ x, int a, int e, U128 sum,
+                                           int sigma, unsigned uf) {
   // Each input lost less than one unit; if the sum holds fewer than cnt * 2^40 units the
   // relative error could exceed 2^-40, so add the doubles directly instead.  A zero sum
   // is exact only if no input of the chunk fell below one unit.
   if (u128_is_zero(sum) && !uf) return 0.0;
-  bool small = (sum.hi == 0ull) && (sum.lo < ((unsigned long long)cnt << 40));
-  if (small) {
+  if (sum.hi == 0ull && sum.lo < ((unsigned long long)(e - a + 1) << 40)) {
     double acc = 0.0;
-    for (long long i = a; i <= e; ++i) acc = __dadd_rn(acc, x[i]);
+    for (int i = a; i <= e; ++i) acc = __dadd_rn(acc, x[i]);
     return acc;
   }
   return u128_to_dbl_scaled(sum, sigma);
 }
 
+// Window means, a CTA per kMeanThreads outputs of a chunk and an output per thread: an output is
+// a dozen independent loads and a few dozen instructions, so small CTAs keep an SM's loads in
+// flight (with a chunk's 1024 outputs per CTA of 40 registers an SM held one, and waited for
+// each), and bins are 32-bit numbers.  1.25e6 bins, start -> now: 26 -> 19 us; a late
+// iteration's few chunks 8 -> 6 us.
 // kTree: the run's S_gal, whose node sums h are kept up to date.
+constexpr int kMeanThreads = 256;
 template <bool kTree>
-__global__ void k_window_mean(const double* __restrict__ x, long long n, SmoothPlan pl,
+__global__ void __launch_bounds__(kMeanThreads, 6)
+k_window_mean(const double* __restrict__ x, long long n, SmoothPlan pl,
                               const unsigned long long* __restrict__ pre_lo,
                               const unsigned long long* __restrict__ pre_hi,
                               const int* __restrict__ sig, const unsigned* __restrict__ uflow,
@@ -2298,31 +2339,37 @@ __global__ void k_window_mean(const double* __restrict__ x, long long n, SmoothP
   double relmax = 0.0;
   const int h = pl.W / 2;
   const double inv_w = 1.0 / (double)pl.W;
-  // output chunks with a dirty chunk within out_radius
+  // output chunks with a dirty chunk within out_radius, in parts of blockDim.x outputs
   const int list = kListR0 + out_radius;
-  const ListHead head = list_head(d, list, pl.nch, kTree ? &o.rs->tree_live : nullptr);
-  const int nitem = head.count;
-  int b_next = head.first;
+  const int parts = (pl.Kc + blockDim.x - 1) / blockDim.x;
+  const ListHead head =
+      list_head(d, list, pl.nch, kTree ? &o.rs->tree_live : nullptr, parts);
+  const int nitem = head.count * parts;
+  long long b_next = head.first;
   for (int it = blockIdx.x; it < nitem; it += gridDim.x) {
     const long long b = b_next;
-    if (it + (int)gridDim.x < nitem) b_next = d.item(list, it + gridDim.x);
-    const long long b0 = b * pl.Kc;
-    const long long jend = b0 + pl.Kc < n ? b0 + pl.Kc : n;
-    for (long long j = b0 + threadIdx.x; j < jend; j += blockDim.x) {
-      long long s = j - h > 0 ? j - h : 0;
-      long long e = j - h + pl.W - 1 < n - 1 ? j - h + pl.W - 1 : n - 1;
-      // s and e lie within one chunk of chunk b (h < W <= Kc): no 64-bit division
-      const long long ds = s - b0, de = e - b0;
-      const long long cs = b + (ds < 0 ? -1 : (ds >= pl.Kc ? 1 : 0));
-      const long long ce = b + (de < 0 ? -1 : (de >= pl.Kc ? 1 : 0));
-      long long cnt = e - s + 1;
+    if (it + (int)gridDim.x < nitem) b_next = d.item(list, (it + gridDim.x) / parts);
+    // bins and outputs as 32-bit numbers (a band holds at most 16e6)
+    const int b0 = (int)b * pl.Kc, nb = (int)n;
+    const int jend = min(b0 + pl.Kc, nb);
+    const int j = b0 + (it % parts) * (int)blockDim.x + threadIdx.x;
+    if (j < jend) {
+      const int s = max(j - h, 0), e = min(j - h + pl.W - 1, nb - 1), cnt = e - s + 1;
+      // s and e lie within one chunk of chunk b (h < W <= Kc)
+      const int cs = (int)b + (s < b0 ? -1 : (s >= b0 + pl.Kc ? 1 : 0));
+      const int ce = (int)b + (e < b0 ? -1 : (e >= b0 + pl.Kc ? 1 : 0));
+      const int s0 = cs * pl.Kc;  // first bin of the window's first chunk
+      const U128 pe{pre_lo[e], pre_hi[e]};
+      U128 ps{0ull, 0ull};
+      if (s > s0) ps = U128{pre_lo[s - 1], pre_hi[s - 1]};
       double sum;
       if (cs == ce) {
-        sum = part_sum(x, cs * pl.Kc, s, e, pre_lo, pre_hi, sig[cs], uflow[cs]);
+        sum = part_sum(x, s, e, u128_sub(pe, ps), sig[cs], uflow[cs]);
       } else {
-        long long last = cs * pl.Kc + pl.Kc - 1;
-        double s1 = part_sum(x, cs * pl.Kc, s, last, pre_lo, pre_hi, sig[cs], uflow[cs]);
-        double s2 = part_sum(x, ce * pl.Kc, ce * pl.Kc, e, pre_lo, pre_hi, sig[ce], uflow[ce]);
+        const int last = s0 + pl.Kc - 1;
+        const U128 pl1{pre_lo[last], pre_hi[last]};
+        const double s1 = part_sum(x, s, last, u128_sub(pl1, ps), sig[cs], uflow[cs]);
+        const double s2 = part_sum(x, last + 1, e, pe, sig[ce], uflow[ce]);
         sum = __dadd_rn(s1, s2);
       }
       double v = (cnt == pl.W) ? __dmul_rn(sum, inv_w) : __ddiv_rn(sum, (double)cnt);
@@ -2340,15 +2387,14 @@ __global__ void k_window_mean(const double* __restrict__ x, long long n, SmoothP
   if (o.rtol_on) warp_max_atomic((u64)__double_as_longlong(relmax), &o.rs->relchg_bits);
 }
 
-// One output of the chunk per thread.
-static int mean_threads(const SmoothPlan& pl) { return pl.Kc < 1024 ? pl.Kc : 1024; }
+static int mean_threads(const SmoothPlan& pl) { return pl.Kc < kMeanThreads ? pl.Kc : kMeanThreads; }
 
 void launch_window_mean(const double* x, long long n, const SmoothPlan& pl,
                         const unsigned long long* pre_lo, const unsigned long long* pre_hi,
                         const int* sig, const unsigned* uflow, SgOut o, Dirty d, int out_radius,
                         cudaStream_t st) {
   int th = mean_threads(pl);
-  int bl = persistent_grid(pl, pl.nch, pl.res_mean);
+  int bl = persistent_grid(pl, pl.nch * ((pl.Kc + th - 1) / th), pl.res_mean);
   if (o.tree.h)
     k_window_mean<true>
         <<<bl, th, 0, st>>>(x, n, pl, pre_lo, pre_hi, sig, uflow, o, d, out_radius);
@@ -2931,12 +2977,19 @@ void plan_grids(SmoothPlan& pl) {
   else
     pl.res_median = resident_ctas(pl, k_median_wm<u64>, median_threads(pl),
                                   median_smem_bytes(pl.Kc, 8));
-  pl.res_prefix = resident_ctas(pl, k_chunk_prefix<true>, pl.Kc < 1024 ? pl.Kc : 1024, 0);
+  if (prefix_per(pl) == kPrefixPer)
+    pl.res_prefix = resident_ctas(pl, k_chunk_prefix<true, kPrefixPer>, prefix_threads(pl),
+                                  prefix_smem(pl, true));
+  else
+    pl.res_prefix = resident_ctas(pl, k_chunk_prefix<true, kPrefixPerLong>, prefix_threads(pl),
+                                  prefix_smem(pl, true));
   pl.res_mean = resident_ctas(pl, k_window_mean<true>, mean_threads(pl), 0);
 }
 
 void configure_kernels() {
   cudaFuncSetAttribute(k_prepass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPrepassSmem);
+  cudaFuncSetAttribute(k_chunk_prefix<true, kPrefixPerLong>,
+                       cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxWindow * 8);
   SmoothPlan p64 = {}, p32 = {};
   p32.fp32_keys = 1;
   for (int kp : {64, 4096, 8192}) {  // one of each instantiation; 8192: the widest sort

@@ -204,13 +204,14 @@ struct ListHead {
   int count, first, iter, flags;
 };
 // flags (may be null): a word of the loop state read along with them.
+// parts: CTAs that share an item, block by block.
 __device__ __forceinline__ ListHead list_head(const Dirty& d, int which, int all,
-                                              const int* flags) {
+                                              const int* flags, int parts = 1) {
   __shared__ ListHead sh;
   if (threadIdx.x == 0) {
     ListHead h;
     h.count = d.count(which, all);
-    h.first = d.item(which, blockIdx.x);  // the grid is never longer than the list
+    h.first = d.item(which, blockIdx.x / parts);  // the grid is never longer than the list
     h.iter = d.base ? d.rs->iter : 0;
     h.flags = flags ? *flags : 0;
     sh = h;
@@ -315,8 +316,8 @@ void launch_running_median(const unsigned long long* skey, const uint16_t* srank
 size_t median_smem_bytes(int Kc, int key_bytes);
 
 // Exact 128-bit prefix sums of the input inside each chunk at a per-chunk scale sig[b];
-// uflow[b] = 1 when an input > 0 of chunk b is below one unit.  x_out (may be null)
-// receives the input values.
+// uflow[b] = 1 when an input > 0 of chunk b is below one unit.  x_out (may be null; only with
+// the spectrum as the input) receives the input values.
 // (in_radius: the input of chunk b changed when a chunk within in_radius of b is dirty.)
 void launch_chunk_prefix(SpecIn in, long long n, const SmoothPlan& pl, unsigned long long* pre_lo,
                          unsigned long long* pre_hi, int* sig, unsigned* uflow, double* x_out,
