@@ -1318,15 +1318,68 @@ __device__ __forceinline__ double key_value<uint32_t>(uint32_t k, double inv_sca
   return __dmul_rn((double)__uint_as_float(k), inv_scale);
 }
 
-// Bitonic sort of (key, position) with E consecutive elements per thread: stages whose
-// partners are less than E apart run in registers, less than 32 E apart through warp
-// shuffles, and only the longest ones through shared memory (a barrier per stage).
-template <typename K>
-__device__ __forceinline__ void cmp_keep(K& k, int& x, K ko, int xo, bool keep_min) {
-  const bool gt = (k > ko) || (k == ko && x > xo);  // this element after the other one
-  if (gt == keep_min) {
-    k = ko;
-    x = xo;
+// Bitonic sort of 64-bit numbers, kpad of them, E consecutive ones per thread (element i in
+// thread i / E).  Every merge begins with a stage of mirrored partners (i with i ^ (k - 1)), so
+// that all comparisons run upwards: an element keeps the smaller or the larger of a pair by one
+// bit of its index.  Partners less than E apart meet in registers, less than 32 E apart through
+// warp shuffles, and the others through shared memory (two buffers in turn: a barrier per stage).
+// buf: 2 kpad numbers.
+// Bound: instruction issue, when every chunk is sorted.  As (key, position) pairs with a direction
+// bit per stage a dense chunk of 1024 bins took 45 K warp instructions, 1.25e6 bins 71.6 us; as
+// single numbers, all ascending, 32 K and 56 us.
+__device__ __forceinline__ void keep_ordered(u64& c, u64 o, bool lower) {
+  if ((o < c) == lower) c = o;
+}
+__device__ __forceinline__ void order_pair(u64& lo, u64& hi) {
+  const u64 x = lo, y = hi;
+  const bool swap = y < x;
+  lo = swap ? y : x;
+  hi = swap ? x : y;
+}
+template <int E>
+__device__ __forceinline__ void bitonic_sort(u64 (&c)[E], int kpad, u64* buf) {
+  const int T = blockDim.x, tid = threadIdx.x;
+  u64* cur = buf;
+  u64* nxt = buf + kpad;
+  for (int kk = 2; kk <= kpad; kk <<= 1) {
+    // the mirrored stage, then distances kk/4 .. 1
+    bool mirror = true;
+    for (int jj = kk >> 1; jj >= E; jj >>= 1) {
+      const int m = (mirror ? kk - 1 : jj) / E;  // partner thread
+      const bool lower = (tid & (jj / E)) == 0;
+      u64 o[E];
+      if (m < 32) {
+#pragma unroll
+        for (int a = 0; a < E; ++a) o[a] = __shfl_xor_sync(0xFFFFFFFFu, c[a], m);
+      } else {
+#pragma unroll
+        for (int a = 0; a < E; ++a) cur[a * T + tid] = c[a];
+        __syncthreads();
+#pragma unroll
+        for (int a = 0; a < E; ++a) o[a] = cur[a * T + (tid ^ m)];
+        u64* t = cur;
+        cur = nxt;
+        nxt = t;
+      }
+#pragma unroll
+      for (int a = 0; a < E; ++a) keep_ordered(c[a], mirror ? o[E - 1 - a] : o[a], lower);
+      mirror = false;
+    }
+    // in registers: partners a and a ^ (2 jl - 1) in the mirrored stage of a merge that fits a
+    // thread, a and a | jl otherwise
+#pragma unroll
+    for (int jl = E / 2; jl >= 1; jl >>= 1) {
+      if (jl > (kk >> 1)) continue;
+      if (jl == (kk >> 1)) {
+#pragma unroll
+        for (int a = 0; a < E; ++a)
+          if ((a & jl) == 0) order_pair(c[a], c[a ^ (2 * jl - 1)]);
+      } else {
+#pragma unroll
+        for (int a = 0; a < E; ++a)
+          if ((a & jl) == 0) order_pair(c[a], c[a | jl]);
+      }
+    }
   }
 }
 
@@ -1500,8 +1553,6 @@ __global__ void __launch_bounds__(1024, E == 2 ? 2 : 1) k_chunk_sort(SpecIn in, 
                                                      K* __restrict__ skey,
                                                      uint16_t* __restrict__ srank, Dirty d) {
   extern __shared__ __align__(16) unsigned char sort_raw[];
-  K* sm_keys = (K*)sort_raw;
-  uint16_t* sm_idx = (uint16_t*)(sm_keys + pl.kpad);
   const int T = blockDim.x, tid = threadIdx.x;
   const int kpad = pl.kpad;  // = T * E
   const ListHead head = list_head(d, kListR0, pl.nch, in.flags);
@@ -1516,7 +1567,7 @@ __global__ void __launch_bounds__(1024, E == 2 ? 2 : 1) k_chunk_sort(SpecIn in, 
     const long long base = (long long)b * pl.Kc;
     const int len = (int)((n - base) < pl.Kc ? (n - base) : pl.Kc);
     K k[E], kold[E];
-    int x[E], rold[E];
+    int rold[E];
     // the previous sorted state, loaded beside the new values
 #pragma unroll
     for (int a = 0; a < E; ++a) {
@@ -1530,7 +1581,6 @@ __global__ void __launch_bounds__(1024, E == 2 ? 2 : 1) k_chunk_sort(SpecIn in, 
       K kv = (K)~(K)0;
       if (i < len) kv = sort_key<K>(spec_value<kSpec>(in, base + i, head.flags), pl.key_scale);
       k[a] = kv;
-      x[a] = i;
     }
     if (resort &&
         resort_few_changes<E, K>(k, kold, rold, len, kpad, skey + base, srank + base, sort_raw)) {
@@ -1571,85 +1621,73 @@ __global__ void __launch_bounds__(1024, E == 2 ? 2 : 1) k_chunk_sort(SpecIn in, 
         }
       }
     }
-    bool first_smem = true;
-    for (int kk = 2; kk <= kpad; kk <<= 1) {
-      int jj = kk >> 1;
-      if (jj >= 32 * E) {
-        if (!first_smem) __syncthreads();  // everyone has read the previous round back
-        first_smem = false;
+    // the whole order: by the key's bits above the position's, with the position in their
+    // place, as one 64-bit number (a 4-byte key leaves room for all of it)
+    const u64 low = (u64)kpad - 1;
+    u64* keys = (u64*)sort_raw;                    // [kpad] by position (8-byte keys)
+    u64* buf = keys + (sizeof(K) == 8 ? kpad : 0);  // [2 kpad]
+    u64 c[E];
 #pragma unroll
-        for (int a = 0; a < E; ++a) {
-          sm_keys[tid * E + a] = k[a];
-          sm_idx[tid * E + a] = (uint16_t)x[a];
-        }
-        __syncthreads();
-        for (; jj >= 32 * E; jj >>= 1) {
-          for (int q = tid; q < kpad / 2; q += T) {
-            const int i = ((q & ~(jj - 1)) << 1) | (q & (jj - 1));
-            const int ixj = i | jj;
-            K ki = sm_keys[i], kj = sm_keys[ixj];
-            uint16_t ii = sm_idx[i], ij = sm_idx[ixj];
-            bool gt = (ki > kj) || (ki == kj && ii > ij);
-            bool asc = ((i & kk) == 0);
-            if (gt == asc) {
-              sm_keys[i] = kj;
-              sm_keys[ixj] = ki;
-              sm_idx[i] = ij;
-              sm_idx[ixj] = ii;
-            }
-          }
-          __syncthreads();
-        }
-#pragma unroll
-        for (int a = 0; a < E; ++a) {
-          k[a] = sm_keys[tid * E + a];
-          x[a] = sm_idx[tid * E + a];
-        }
+    for (int a = 0; a < E; ++a) {
+      const int i = tid * E + a;
+      if (sizeof(K) == 8) {
+        keys[i] = (u64)k[a];
+        c[a] = ((u64)k[a] & ~low) | (u64)i;
+      } else {
+        c[a] = ((u64)k[a] << 32) | (u64)i;
       }
-      for (; jj >= E; jj >>= 1) {
-        const int lm = jj / E;  // partner lane offset (< 32)
+    }
+    for (int pass = 0;; ++pass) {
+      bitonic_sort<E>(c, kpad, buf);
+      if (sizeof(K) == 4) break;
+      // Keys that differ in the bits left out only may stand in the wrong order.  Such a
+      // chunk is sorted by (those bits, position) and then by (the others, place in that
+      // order), which is the order wanted.
+      uint16_t* posof = (uint16_t*)(buf + 2 * (size_t)kpad);  // [kpad]
+      if (pass == 0) {
+        __shared__ u64 first[32];
+        const int lane = tid & 31;
+        __syncthreads();  // keys are in place (a chunk of one warp meets no other barrier)
+#pragma unroll
+        for (int a = 0; a < E; ++a) k[a] = (K)keys[c[a] & low];
+        u64 after = __shfl_down_sync(0xFFFFFFFFu, (u64)k[0], 1);
+        if (lane == 0) first[tid >> 5] = (u64)k[0];
+        __syncthreads();
+        if (lane == 31) after = tid + 1 < T ? first[(tid >> 5) + 1] : ~0ull;
+        bool bad = (u64)k[E - 1] > after;
+#pragma unroll
+        for (int a = 0; a + 1 < E; ++a) bad = bad || k[a] > k[a + 1];
+        if (!__syncthreads_or(bad)) break;
+#pragma unroll
+        for (int a = 0; a < E; ++a) c[a] = (((u64)k[a] & low) << 13) | (c[a] & low);
+      } else if (pass == 1) {
 #pragma unroll
         for (int a = 0; a < E; ++a) {
           const int i = tid * E + a;
-          const K ko = __shfl_xor_sync(0xFFFFFFFFu, k[a], lm);
-          const int xo = __shfl_xor_sync(0xFFFFFFFFu, x[a], lm);
-          const bool lower = (i & jj) == 0, asc = (i & kk) == 0;
-          cmp_keep<K>(k[a], x[a], ko, xo, lower == asc);
+          const int pos = (int)(c[a] & low);
+          posof[i] = (uint16_t)pos;
+          c[a] = (keys[pos] & ~low) | (u64)i;
         }
-      }
-      // in-thread stages: distances E/2 .. 1 (those below kk), unrolled so that the
-      // element arrays stay in registers
-#pragma unroll
-      for (int jl = E / 2; jl >= 1; jl >>= 1) {
-        if (jl > (kk >> 1)) continue;
+      } else {
+        __syncthreads();
 #pragma unroll
         for (int a = 0; a < E; ++a) {
-          if ((a & jl) == 0) {
-            const int c = a | jl;
-            const int i = tid * E + a;
-            const bool asc = (i & kk) == 0;
-            const K ka = k[a], kc = k[c];
-            const int xa = x[a], xc = x[c];
-            const bool gt = (ka > kc) || (ka == kc && xa > xc);
-            if (gt == asc) {
-              k[a] = kc;
-              k[c] = ka;
-              x[a] = xc;
-              x[c] = xa;
-            }
-          }
+          const int pos = posof[c[a] & low];
+          k[a] = (K)keys[pos];
+          c[a] = (u64)pos;
         }
+        break;
       }
     }
 #pragma unroll
     for (int a = 0; a < E; ++a) {
       const int sidx = tid * E + a;
       if (sidx < len) {
-        skey[base + sidx] = k[a];
-        srank[base + x[a]] = (uint16_t)sidx;
+        skey[base + sidx] = sizeof(K) == 8 ? k[a] : (K)(c[a] >> 32);
+        srank[base + (int)(c[a] & low)] = (uint16_t)sidx;
       }
     }
-    if (!first_smem) __syncthreads();  // before the next chunk overwrites shared memory
+    __syncthreads();  // before the next chunk overwrites shared memory
   }
 }
 
@@ -1686,7 +1724,8 @@ static int sort_per_thread(const SmoothPlan& pl) {
 static int sort_threads(const SmoothPlan& pl) { return pl.kpad / sort_per_thread(pl); }
 static size_t sort_smem(const SmoothPlan& pl) {
   const size_t kb = pl.fp32_keys ? 4 : 8;
-  const size_t full = (size_t)pl.kpad * (kb + sizeof(uint16_t));
+  // the exchange buffers; 8-byte keys by position and an order beside them
+  const size_t full = (size_t)pl.kpad * (16 + (kb == 8 ? 8 + sizeof(uint16_t) : 0));
   const size_t few = (size_t)pl.kpad * (kb + 2 + 1) + (size_t)(pl.kpad + 2) * 2 +
                      (size_t)kResortMax * 2 * (kb + 2);
   return full > few ? full : few;
