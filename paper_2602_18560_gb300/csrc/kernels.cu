@@ -1240,11 +1240,23 @@ __device__ __forceinline__ float sum32(const float4 (&v)[8]) {
 // Levels 2 and up from level 1 (the whole CTA): a thread per node adds its 32 values, all of
 // them loaded at once.  (A warp per node left the one CTA waiting on a load per node: 20 us
 // for a band of 1.25e6 bins, against 4.)
-__device__ __noinline__ void tree_h_levels(const Tree& tr) {
+// Only the nodes above the changed bins: the outputs of the CTAs' items are the bins
+// [item b0 + shift, + Kc), item from the work list (all of them when it is long).
+__device__ __noinline__ void tree_h_levels(const Tree& tr, const Dirty& d, int list, int nitem,
+                                           int Kc, int shift) {
   for (int l = 1; l < kTreeLevels; ++l) {
     const float4* in = reinterpret_cast<const float4*>(tr.h + tr.off[l - 1]);
     float* out = tr.h + tr.off[l];
-    for (int i = threadIdx.x; i < tr.n[l]; i += blockDim.x) {
+    const int sh = 5 * (l + 1), per = (Kc >> sh) + 2;  // nodes that Kc bins can lie in
+    const bool some = d.lists && (long long)nitem * per < tr.n[l];
+    const int count = some ? nitem * per : tr.n[l];
+    for (int x = threadIdx.x; x < count; x += blockDim.x) {
+      int i = x;
+      if (some) {
+        const int a = max(d.item(list, x / per) * Kc + shift, 0);
+        i = (a >> sh) + x % per;
+      }
+      if (i < 0 || i >= tr.n[l]) continue;
       float4 v[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) v[k] = __ldcg(in + (size_t)i * 8 + k);
@@ -1796,14 +1808,14 @@ __device__ __forceinline__ void sts_u16(uint32_t addr, unsigned v) {
   asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"((unsigned short)v) : "memory");
 }
 
-// Wavelet matrix of the permutation seq0 (M elements) when every warp owns exactly WPW words
-// of a level: each level loads the warp's elements once, all of them before the first ballot,
-// and the ballots serve both the count and the stable partition into the other buffer.
+// Wavelet matrix of the permutation seq0 (M elements, every warp owning exactly WPW words of a
+// level; the caller fills the last words up with ranks beyond the span's): each level loads the
+// warp's elements once, all of them before the first ballot, and the ballots serve both the count and the stable partition into the other buffer.
 // Level l stores its words in rk[l ws ..] (bits in the low half, ones of the earlier words
 // in the high half) and its number of zeros in zeros[l].  seq0 and seq1 are both
 // overwritten.
 template <int WPW>
-__device__ __forceinline__ void wm_build_fixed(uint16_t* seq0, uint16_t* seq1, u64* rk, int ws,
+__device__ __forceinline__ void wm_build(uint16_t* seq0, uint16_t* seq1, u64* rk, int ws,
                                                int* zeros, int* warp_ones, int M, int LV,
                                                int nwm) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
@@ -1894,6 +1906,26 @@ __device__ __forceinline__ void wm_build_any(uint16_t* seq0, uint16_t* seq1, u64
   }
 }
 
+// Positions of a tile of M filled up to whole words for every warp of T threads, so that the
+// build's loads are unrolled: one, two, four or eight words per warp, as long as the ranks of
+// the positions added keep LV bits.  Otherwise M (few threads for a long window, or more than a
+// short one needs).  Before, only the windows whose words divide so had it; now W = 300 takes
+// 189 us for every tile of 1.25e6 bins (195 with the loads in a loop), W = 2000 212 (219), a late
+// tile there 30 us (33).
+static int median_pad(int M, int T) {
+  const int nwarp = T >> 5, w = ((M >> 5) + nwarp - 1) / nwarp;
+  const int wpw = w <= 2 ? w : w <= 4 ? 4 : w <= 8 ? 8 : 0;
+  const int Mp = 32 * wpw * nwarp;
+  int top = 1;  // 2^LV
+  while (top < M) top <<= 1;
+  return wpw > 0 && Mp <= top ? Mp : M;
+}
+// Bytes of the keys' region, which later holds Mp positions' and M ranks' 16-bit numbers.
+__host__ __device__ __forceinline__ size_t median_keys_bytes(int M, int Mp, size_t key_bytes) {
+  const size_t k = key_bytes * M, later = 2 * ((size_t)M + Mp);
+  return ((k > later ? k : later) + 15) & ~(size_t)15;
+}
+
 // Ones of a level's bitset before position i (the word holds its bits in the low half and
 // the ones of all earlier words in the high half).
 __device__ __forceinline__ int wm_rank1(const u64* rkl, int i) {
@@ -1908,8 +1940,10 @@ __device__ __forceinline__ double median_tile(const K* __restrict__ skey,
                                               const SmoothPlan& pl, const SgOut& o, long long u,
                                               unsigned char* sm_raw, int* zeros) {
   const int T = blockDim.x, tid = threadIdx.x;
+  // the span's positions, and the same filled up to whole words for every warp
   const int Kc = pl.Kc, M = 2 * Kc, LV = wm_levels(M);
-  const int nwm = M >> 5, ws = nwm + 1;  // words per level (one zero word of padding)
+  const int Mp = pl.median_mp;
+  const int nwm = Mp >> 5, ws = nwm + 1;  // words per level (one zero word of padding)
   const int h = pl.W / 2;
   long long j_lo = (u - 1) * Kc + h, j_hi = u * Kc + h;
   if (j_lo < 0) j_lo = 0;
@@ -1922,12 +1956,12 @@ __device__ __forceinline__ double median_tile(const K* __restrict__ skey,
   if (u < pl.nch) len1 = (n - span - Kc) < Kc ? (int)(n - span - Kc) : Kc;
   double relmax = 0.0;
   K* sk = (K*)sm_raw;                                        // [M] sorted keys (step 1)
-  uint16_t* seq1 = (uint16_t*)sm_raw;                        // [M] (steps 2-3, over sk)
-  uint16_t* src = seq1 + M;                                  // [M] rank -> element
-  uint16_t* seq0 = (uint16_t*)(sm_raw + sizeof(K) * (size_t)M);  // [M]
+  uint16_t* seq1 = (uint16_t*)sm_raw;                        // [Mp] (steps 2-3, over sk)
+  uint16_t* src = seq1 + Mp;                                 // [M] rank -> element
+  uint16_t* seq0 = (uint16_t*)(sm_raw + median_keys_bytes(M, Mp, sizeof(K)));  // [Mp]
   // [LV][ws]: per bitset word, its 32 bits (low half) and the ones before it (high half),
   // so that a rank is one 64-bit load
-  u64* rk = (u64*)(seq0 + M);
+  u64* rk = (u64*)(seq0 + Mp);
   uint16_t* mr = (uint16_t*)rk;  // [M] merged index of (chunk, sorted index) (step 1, over rk)
   __shared__ int warp_ones[32];
 
@@ -2000,25 +2034,19 @@ __device__ __forceinline__ double median_tile(const K* __restrict__ skey,
     }
     seq0[p] = (uint16_t)v;
   }
+  for (int p = M + tid; p < Mp; p += T) seq0[p] = (uint16_t)p;
   __syncthreads();
 
-  // 2. wavelet matrix.  Warp w owns the words [w wpw, (w + 1) wpw) of every level (M is a
-  // multiple of 64: whole words).  A level takes two barriers: one after the warps have
-  // counted their ones, one after the stable partition.
-  {
-    const int nwarp = T >> 5;
-    const int wpw = (nwm + nwarp - 1) / nwarp;
-    const bool full = wpw * nwarp == nwm;
-    if (full && wpw == 4)
-      wm_build_fixed<4>(seq0, seq1, rk, ws, zeros, warp_ones, M, LV, nwm);
-    else if (full && wpw == 2)
-      wm_build_fixed<2>(seq0, seq1, rk, ws, zeros, warp_ones, M, LV, nwm);
-    else if (full && wpw == 8)
-      wm_build_fixed<8>(seq0, seq1, rk, ws, zeros, warp_ones, M, LV, nwm);
-    else if (full && wpw == 1)
-      wm_build_fixed<1>(seq0, seq1, rk, ws, zeros, warp_ones, M, LV, nwm);
-    else
-      wm_build_any(seq0, seq1, rk, ws, zeros, warp_ones, M, LV, nwm);
+  // 2. wavelet matrix.  Warp w owns the words [w wpw, (w + 1) wpw) of every level.  A level
+  // takes two barriers: one after the warps have counted their ones, one after the stable
+  // partition.
+  const int nwarp = T >> 5, wpw = nwm % nwarp == 0 ? nwm / nwarp : 0;
+  switch (wpw) {
+    case 1: wm_build<1>(seq0, seq1, rk, ws, zeros, warp_ones, Mp, LV, nwm); break;
+    case 2: wm_build<2>(seq0, seq1, rk, ws, zeros, warp_ones, Mp, LV, nwm); break;
+    case 4: wm_build<4>(seq0, seq1, rk, ws, zeros, warp_ones, Mp, LV, nwm); break;
+    case 8: wm_build<8>(seq0, seq1, rk, ws, zeros, warp_ones, Mp, LV, nwm); break;
+    default: wm_build_any(seq0, seq1, rk, ws, zeros, warp_ones, Mp, LV, nwm); break;
   }
 
   // 3. selections
@@ -2085,7 +2113,8 @@ __device__ __forceinline__ double median_tile(const K* __restrict__ skey,
 template <typename K>
 __global__ void __launch_bounds__(512, 2) k_median_wm(
     const K* __restrict__ skey, const uint16_t* __restrict__ srank,
-    long long n, SmoothPlan pl, const __grid_constant__ SgOut o, Dirty d) {
+    long long n, SmoothPlan pl, const __grid_constant__ SgOut o,
+    const __grid_constant__ Dirty d) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   __shared__ int zeros[16];
   double relmax = 0.0;
@@ -2111,11 +2140,13 @@ __global__ void __launch_bounds__(512, 2) k_median_wm(
     // the nodes that straddle two tiles, then the levels above
     if ((pl.W / 2) & 31)
       tree_h_straddle(o.Gf, o.inv_f, o.tree.h, o.tree.n[0], pl.Kc, pl.W / 2, pl.nch);
-    tree_h_levels(o.tree);
+    tree_h_levels(o.tree, d, kListTile, nitem, pl.Kc, pl.W / 2 - pl.Kc);
   }
   if (o.rtol_on) warp_max_atomic((u64)__double_as_longlong(relmax), &o.rs->relchg_bits);
 }
 
+// Two outputs per thread: a few tiles' latency is what a late iteration waits for.  At most 512
+// threads, so that two CTAs share an SM (W = 2000, every tile: 212 us, 228 with 1024).
 static int median_threads(const SmoothPlan& pl) {
   if (pl.median_th) return pl.median_th;
   int t = ((pl.Kc / 2 + 31) / 32) * 32;
@@ -2124,23 +2155,26 @@ static int median_threads(const SmoothPlan& pl) {
   return t;
 }
 
-size_t median_smem_bytes(int Kc, int key_bytes) {
-  int M = 2 * Kc, LV = 0;
+size_t median_smem_bytes(int Kc, int threads, int key_bytes) {
+  const int M = 2 * Kc, Mp = median_pad(M, threads);
+  int LV = 0;
   while ((1 << LV) < M) ++LV;
-  size_t ws = (size_t)M / 32 + 1;
+  size_t ws = (size_t)Mp / 32 + 1;
   size_t rk = (size_t)LV * ws * 8, mr = (size_t)2 * M;  // the merged indices sit over rk
-  return (size_t)key_bytes * M + (size_t)2 * M + (rk > mr ? rk : mr);
+  return median_keys_bytes(M, Mp, key_bytes) + (size_t)2 * Mp + (rk > mr ? rk : mr);
 }
 
 void launch_running_median(const unsigned long long* skey, const uint16_t* srank, long long n,
                            const SmoothPlan& pl, SgOut o, Dirty d, cudaStream_t st) {
   int th = median_threads(pl);
-  size_t smem = median_smem_bytes(pl.Kc, pl.fp32_keys ? 4 : 8);
+  size_t smem = median_smem_bytes(pl.Kc, th, pl.fp32_keys ? 4 : 8);
   int bl = persistent_grid(pl, pl.nch + 1, pl.res_median);
+  SmoothPlan p = pl;
+  p.median_mp = median_pad(2 * pl.Kc, th);
   if (pl.fp32_keys)
-    k_median_wm<uint32_t><<<bl, th, smem, st>>>((const uint32_t*)skey, srank, n, pl, o, d);
+    k_median_wm<uint32_t><<<bl, th, smem, st>>>((const uint32_t*)skey, srank, n, p, o, d);
   else
-    k_median_wm<u64><<<bl, th, smem, st>>>(skey, srank, n, pl, o, d);
+    k_median_wm<u64><<<bl, th, smem, st>>>(skey, srank, n, p, o, d);
 }
 
 // ============================================================================ window mean
@@ -2374,7 +2408,8 @@ k_window_mean(const double* __restrict__ x, long long n, SmoothPlan pl,
                               const unsigned long long* __restrict__ pre_lo,
                               const unsigned long long* __restrict__ pre_hi,
                               const int* __restrict__ sig, const unsigned* __restrict__ uflow,
-                              const __grid_constant__ SgOut o, Dirty d, int out_radius) {
+                              const __grid_constant__ SgOut o, const __grid_constant__ Dirty d,
+                              int out_radius) {
   double relmax = 0.0;
   const int h = pl.W / 2;
   const double inv_w = 1.0 / (double)pl.W;
@@ -2422,7 +2457,8 @@ k_window_mean(const double* __restrict__ x, long long n, SmoothPlan pl,
       }
     }
   }
-  if (kTree && head.flags && last_cta(&o.rs->ticket)) tree_h_levels(o.tree);
+  if (kTree && head.flags && last_cta(&o.rs->ticket))
+    tree_h_levels(o.tree, d, list, head.count, pl.Kc, 0);
   if (o.rtol_on) warp_max_atomic((u64)__double_as_longlong(relmax), &o.rs->relchg_bits);
 }
 
@@ -3012,10 +3048,10 @@ void plan_grids(SmoothPlan& pl) {
   });
   if (pl.fp32_keys)
     pl.res_median = resident_ctas(pl, k_median_wm<uint32_t>, median_threads(pl),
-                                  median_smem_bytes(pl.Kc, 4));
+                                  median_smem_bytes(pl.Kc, median_threads(pl), 4));
   else
     pl.res_median = resident_ctas(pl, k_median_wm<u64>, median_threads(pl),
-                                  median_smem_bytes(pl.Kc, 8));
+                                  median_smem_bytes(pl.Kc, median_threads(pl), 8));
   if (prefix_per(pl) == kPrefixPer)
     pl.res_prefix = resident_ctas(pl, k_chunk_prefix<true, kPrefixPer>, prefix_threads(pl),
                                   prefix_smem(pl, true));
@@ -3045,9 +3081,9 @@ void configure_kernels() {
     with_sort_kernel<false>(p32, set);
   }
   cudaFuncSetAttribute(k_median_wm<u64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)median_smem_bytes(kMaxWindow, 8));
+                       224 * 1024);
   cudaFuncSetAttribute(k_median_wm<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)median_smem_bytes(kMaxWindow, 4));
+                       224 * 1024);
 }
 
 }  // namespace gbsub

@@ -116,6 +116,7 @@ struct SmoothPlan {
   int res_sort, res_median, res_prefix, res_mean;  // CTAs resident at once (plan_grids)
   int sort_e;     // elements per sorting thread (2, 4, 8), 0: chosen from kpad
   int median_th;  // threads per median tile (multiple of 32, <= 512), 0: chosen from Kc
+  int median_mp;  // positions of a median tile filled up to whole words per warp (at launch)
 };
 
 // Source of an estimator's input: the run's fixed-point spectrum (P_k = S_k Q_k 2^-96) or
@@ -313,7 +314,7 @@ void launch_chunk_sort(SpecIn in, long long n, const SmoothPlan& pl, unsigned lo
 // changed.
 void launch_running_median(const unsigned long long* skey, const uint16_t* srank, long long n,
                            const SmoothPlan& pl, SgOut o, Dirty d, cudaStream_t st);
-size_t median_smem_bytes(int Kc, int key_bytes);
+size_t median_smem_bytes(int Kc, int threads, int key_bytes);
 
 // Exact 128-bit prefix sums of the input inside each chunk at a per-chunk scale sig[b];
 // uflow[b] = 1 when an input > 0 of chunk b is below one unit.  x_out (may be null; only with
