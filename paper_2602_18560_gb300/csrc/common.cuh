@@ -126,6 +126,35 @@ __device__ __forceinline__ void q_parts(double q, u64* c0, u64* c1, u64* c2) {
   *c2 = v.hi;
 }
 
+// The deposit of one cell of a sweep, q = c gq with c = A^2 w (w the cell's weight) from the
+// integer mantissas, truncated: within 2^-62 of the exact product and without FP64 arithmetic.
+// c0, c1, c2 and the return value as q_single; c and gq finite, >= 0, zero or subnormal: q = 0.
+__device__ __forceinline__ bool q_cell(double c, double gq, u64* c0, u64* c1, u64* c2) {
+  const u64 bc = (u64)__double_as_longlong(c), bg = (u64)__double_as_longlong(gq);
+  const int ec = (int)((bc >> 52) & 0x7FF), eg = (int)((bg >> 52) & 0x7FF);
+  *c0 = *c1 = *c2 = 0ull;
+  if (ec == 0 || eg == 0) return true;
+  const u64 a = ((bc & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << 11;
+  const u64 g = ((bg & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << 11;
+  const u64 p = __umul64hi(a, g);   // in [2^62, 2^64): q = p 2^sh
+  const int sh = ec + eg - 2108;
+  if (sh + 63 - __clzll((long long)p) >= 159) return false;
+  const int t = sh - 32;            // Q = q 2^-32 = p 2^t
+  u64 lo = 0ull, hi = 0ull;
+  if (t >= 64) {
+    hi = p << (t - 64);
+  } else if (t > 0) {
+    lo = p << t;
+    hi = p >> (64 - t);
+  } else if (t > -64) {
+    lo = p >> (-t);
+  }
+  *c0 = lo & 0xFFFFFFFFull;
+  *c1 = lo >> 32;
+  *c2 = hi;
+  return true;
+}
+
 __device__ __forceinline__ unsigned hi32(u64 x) { return (unsigned)(x >> 32); }
 __device__ __forceinline__ unsigned lo32(u64 x) { return (unsigned)x; }
 // x >> n, 0 for n >= 64.

@@ -82,31 +82,6 @@ void launch_tables(const Grid& g, int tdi2, double* S, double* R, double* gq, fl
 
 // ============================================================================ spectrum I/O
 
-__device__ __forceinline__ void deposit_q(unsigned long long* acc, long long j, double q,
-                                          unsigned* err) {
-  // q >= 0: compare the bits with those of 2^159 (no FP64 instruction)
-  if ((u64)__double_as_longlong(q) >= kQLimitBits) {
-    atomicOr(err, ERR_RANGE);
-    return;
-  }
-  u64 c0, c1, c2;
-  q_parts(q, &c0, &c1, &c2);
-  u64* a = acc + 4 * j;
-  if (c0) atomicAdd(a + 0, c0);
-  if (c1) atomicAdd(a + 1, c1);
-  if (c2) atomicAdd(a + 2, c2);
-}
-
-__device__ __forceinline__ void remove_q(unsigned long long* acc, long long j, double q) {
-  if ((u64)__double_as_longlong(q) >= kQLimitBits) return;  // never deposited
-  u64 c0, c1, c2;
-  q_parts(q, &c0, &c1, &c2);
-  u64* a = acc + 4 * j;
-  if (c0) atomicAdd(a + 0, (u64)(0ull - c0));
-  if (c1) atomicAdd(a + 1, (u64)(0ull - c1));
-  if (c2) atomicAdd(a + 2, (u64)(0ull - c2));
-}
-
 // The parts of a single-bin deposit (q_single) added to, or taken from, bin j.
 __device__ __forceinline__ void add_parts(unsigned long long* acc, long long j, u64 c0, u64 c1,
                                           u64 c2) {
@@ -300,111 +275,55 @@ __global__ void k_fold_replicas(unsigned long long* __restrict__ acc, AccReplica
 }
 
 
-// FP64 path of the catalog pass: the sweep of one source, its pieces deposited; returns
-// the sum of its contributions.  Kept out of line so that none of it is speculated into
-// the common path.
-// Bins of a source's sweep that the FP64 path walks: [k0, k1] (absolute bin numbers),
-// empty when the sweep leaves the band.
+// Bins of a source's sweep inside the band: [k0, k1] (absolute bin numbers), empty when the
+// sweep leaves it.
 __device__ __forceinline__ void sweep_bins(const Sweep& sw, const Grid& g, long long* k0,
                                            long long* k1) {
   *k0 = sw.ka > g.k_lo ? sw.ka : g.k_lo;
   *k1 = sw.kb < g.k_lo + g.nb - 1 ? sw.kb : g.k_lo + g.nb - 1;
 }
 
-// Deposit bins k0 + off, k0 + off + step, ... <= k1 of a multi-bin sweep; returns the sum
-// of their contributions in that order.
-__device__ __forceinline__ double sweep_deposit(const Sweep& sw, const Grid& g, const Tables& tb,
-                                                double a2, long long k0, long long k1, int off,
-                                                int step, unsigned long long* acc,
-                                                unsigned* err) {
-  double r = 0.0;
-  const double inv = sweep_inv_len(sw);
-  for (long long k = k0 + off; k <= k1; k += step) {
-    double w = sweep_weight_inv(sw, k, inv);
-    if (w > 0.0) {
-      long long j = k - g.k_lo;
-      double q = __dmul_rn(__dmul_rn(a2, w), tb.gq[j]);
-      deposit_q(acc, j, q, err);
-      r = __dadd_rn(r, q);
-    }
-  }
-  return r;
+// The cells of a sweep over several bins, for the catalog pass (a lane each): the bins
+// j0 .. j0 + n - 1 of the band hold A^2 w = mid, except the sweep's own first and last bin
+// where they are inside the band.  The same products as RN(A^2 RN((b - a) inv)) in every cell:
+// an interior cell's b - a is 1.
+struct SweepCells {
+  int j0, n;
+  bool first_in, last_in;
+  double mid, first, last;
+};
+__device__ __forceinline__ double cell_power(const SweepCells& s, int t) {
+  return t == 0 && s.first_in ? s.first : t == s.n - 1 && s.last_in ? s.last : s.mid;
 }
 
-// FP64 path of the catalog pass for one source: the sweep, its pieces deposited; returns
-// the sum of its contributions.  Kept out of line so that none of it is speculated into the
-// common path.
-// A single-bin sweep is deposited as q_single(A, gq) exactly as the common path deposits it, so
-// that every single-bin source is removed the same way whichever path deposited it.
-__device__ __forceinline__ double prepass_slow(double A, double fs, double fds, const Grid& g,
-                                            const Tables& tb, unsigned long long* acc,
-                                            unsigned* err) {
-  Sweep sw = make_sweep(fs, fds, g.T, g.T2);
-  if (sw.ka == sw.kb) {
-    long long j = sw.ka - g.k_lo;
-    if (j >= 0 && j < g.nb) {
-      u64 c0, c1, c2, qb;
-      if (!q_single(A, tb.gq[j], &c0, &c1, &c2, &qb)) {
-        atomicOr(err, ERR_RANGE);
-        return 0.0;
-      }
-      add_parts(acc, j, c0, c1, c2);
-      return __longlong_as_double((long long)qb);
-    }
-    return 0.0;
-  }
-  long long k0, k1;
-  sweep_bins(sw, g, &k0, &k1);
-  return sweep_deposit(sw, g, tb, __dmul_rn(A, A), k0, k1, 0, 1, acc, err);
-}
-
-// Bins the FP64 path of a source would walk (0 for a single-bin sweep).
-__device__ __forceinline__ long long slow_span(double fs, double fds, const Grid& g) {
-  Sweep sw = make_sweep(fs, fds, g.T, g.T2);
-  if (sw.ka == sw.kb) return 0;
-  long long k0, k1;
-  sweep_bins(sw, g, &k0, &k1);
-  return k1 >= k0 ? k1 - k0 + 1 : 0;
-}
-
-// The FP64 path of one long sweep, by a whole warp: the lanes share its bins, or, beyond
-// kTreeBins of them, the bins at its ends and the nodes of the tree between; the sum of the
-// contributions comes back in every lane.
-__device__ __forceinline__ double prepass_slow_warp(double A, double fs, double fds, const Grid& g,
-                                                 const Tables& tb, unsigned long long* acc,
-                                                 RunState* rs) {
+// A long sweep (tree_takes), by a whole warp: the bins at its ends and the nodes between; the
+// sum of the contributions (units of 2^-96 S_instr) comes back in every lane.  qn: q of a node.
+__device__ __forceinline__ double tree_deposit(const SweepCells& c, double qn, const Tables& tb,
+                                               unsigned long long* acc, RunState* rs) {
   const int lane = threadIdx.x & 31;
-  Sweep sw = make_sweep(fs, fds, g.T, g.T2);
-  long long k0, k1;
-  sweep_bins(sw, g, &k0, &k1);
-  const double a2 = __dmul_rn(A, A), inv = sweep_inv_len(sw);
-  double r = 0.0, q;
-  if (!tree_takes(tb.tree, a2, inv, k0, k1, &q)) {
-    r = sweep_deposit(sw, g, tb, a2, k0, k1, lane, 32, acc, &rs->err);
-  } else if (q > 0.0) {
-    const TreeSpan t = tree_span(sw.ka - g.k_lo, sw.kb - g.k_lo, k0 - g.k_lo, k1 - g.k_lo);
-    for (int x = lane; x < t.nbins; x += 32) {
-      const int j = tree_bin(t, x);
-      const double w = sweep_weight_inv(sw, g.k_lo + j, inv);
-      if (w > 0.0) {
-        const double qj = __dmul_rn(__dmul_rn(a2, w), tb.gq[j]);
-        deposit_q(acc, j, qj, &rs->err);
-        r = __dadd_rn(r, qj);
-      }
-    }
+  const TreeSpan t = tree_span(c.first_in ? c.j0 : c.j0 - 1, c.last_in ? c.j0 + c.n - 1 : c.j0 + c.n,
+                               c.j0, c.j0 + c.n - 1);
+  U128 sum{0ull, 0ull};
+  for (int x = lane; x < t.nbins; x += 32) {
+    const int j = tree_bin(t, x);
     u64 c0, c1, c2;
-    q_parts(q, &c0, &c1, &c2);
-    const double c = __dmul_rn(a2, inv);
-    for (int x = lane; x < t.nnodes; x += 32) {
-      int l, i;
-      tree_node(t, x, &l, &i);
-      if (c0) atomicAdd(acc + node_word(l, i, 0), c0);
-      if (c1) atomicAdd(acc + node_word(l, i, 1), c1);
-      if (c2) atomicAdd(acc + node_word(l, i, 2), c2);
-      r = __dadd_rn(r, __dmul_rn(c, tb.tree.gsum[tb.tree.off[l - 1] + i]));
-    }
-    if (lane == 0 && !(*(volatile int*)&rs->spec & kSpecTree)) atomicOr(&rs->spec, (int)kSpecTree);
+    if (!q_cell(cell_power(c, j - c.j0), tb.gq[j], &c0, &c1, &c2)) atomicOr(&rs->err, ERR_RANGE);
+    add_parts(acc, j, c0, c1, c2);
+    sum = u128_add(sum, U128{c0 | (c1 << 32), c2});
   }
+  u64 c0, c1, c2;
+  q_parts(qn, &c0, &c1, &c2);
+  double gs = 0.0;
+  for (int x = lane; x < t.nnodes; x += 32) {
+    int l, i;
+    tree_node(t, x, &l, &i);
+    if (c0) atomicAdd(acc + node_word(l, i, 0), c0);
+    if (c1) atomicAdd(acc + node_word(l, i, 1), c1);
+    if (c2) atomicAdd(acc + node_word(l, i, 2), c2);
+    gs = __dadd_rn(gs, tb.tree.gsum[tb.tree.off[l - 1] + i]);
+  }
+  if (lane == 0 && !(*(volatile int*)&rs->spec & kSpecTree)) atomicOr(&rs->spec, (int)kSpecTree);
+  double r = __dadd_rn(__dmul_rn(c.mid, gs), u128_to_dbl_scaled(sum, -32));
   for (int o = 16; o > 0; o >>= 1) r = __dadd_rn(r, __shfl_xor_sync(0xFFFFFFFFu, r, o));
   return r;
 }
@@ -530,18 +449,6 @@ constexpr size_t kPrepassSmem =
                          kSlowWarpCap * sizeof(long long)) +
     (size_t)kHotBins * 3 * sizeof(unsigned);
 
-// Sweeps longer than this many bins are walked by a whole warp (loud high-frequency sources
-// sweep up to hundreds of bins; one lane walking them in FP64 would hold its warp, and the
-// launch, long after every other warp is done).
-constexpr long long kSlowLaneBins = 4;
-
-// Source s of a generated catalog.
-__device__ __forceinline__ double3 gen_source_at(const CatalogRef* __restrict__ cat, long long s) {
-  const GenParams g = cat->gen;
-  double3 r;
-  gen_source(g, s, &r.x, &r.y, &r.z);
-  return r;
-}
 
 // The common case of one source without FP64 arithmetic: the bin k its sweep starts in, and
 // the certificate that the whole sweep [f T, f T + fdot T^2] stays inside cell k (false: the
@@ -596,29 +503,46 @@ struct PrepassArgs {
 
 // What a warp sets aside in its queue: a source of the FP64 path, or (tagged) one that the
 // common path deposited and that is to be kept as a candidate.  Both are rare, and the queue's
-// drain is out of line and called once per tile, so that none of its registers are held in the
-// common path.
+// drain is out of line and called once per step, so that none of its registers are held in the
+// common path.  A generated catalog's entries carry their values, which are FP32 numbers.
 constexpr long long kQueueKeep = 1LL << 62;
 constexpr unsigned kMaxAExp = 1535;  // exponent field of 2^512
+struct SlowQueue {
+  long long* s;
+  float *a, *f, *d;  // generated catalogs only
+};
 
-// Up to 32 queued entries q[0 .. cnt) of one warp (lane i takes entry i; sweeps longer than
-// kSlowLaneBins by the whole warp); returns this lane's count of the paper's candidates.
+// Up to 32 queued entries from `at` on (lane i takes entry i); returns this lane's count of the
+// paper's candidates.
+//
+// FP64 arithmetic (a warp instruction every 64 clocks of a scheduler) is done once per source,
+// a lane each: its sweep and the powers of its first, interior and last cells.  The cells of all
+// 32 sources are then laid end to end and dealt out to the lanes, whatever their lengths, as
+// integer products, and each source's sum comes back by a segmented scan.  Before, a sweep of
+// more than 4 bins was walked by the whole warp in FP64, two of three lanes idle.  With the queues
+// of the generated pass: catalog pass of 1e7 sources of a prior draw 3.2 -> 1.2 ms, of 3e6 stored
+// ones with long sweeps 140 -> 90 us.
 template <bool kGen>
 __device__ __noinline__ unsigned prepass_drain_warp(const PrepassArgs& pa, const CatalogRef* cat,
-                                                    const long long* q, int cnt) {
+                                                    const SlowQueue& q, int at, int cnt) {
   const int lane = threadIdx.x & 31;
+  const Grid& g = pa.g;
   unsigned nkappa = 0;
   const bool valid = lane < cnt;
-  const long long entry = valid ? q[lane] : 0;
+  const long long entry = valid ? q.s[at + lane] : 0;
   const long long s = entry & ~kQueueKeep;
-  double a = 0.0, fs = 0.0, fds = 0.0;
-  bool wide = false, live = (entry & kQueueKeep) != 0;  // (tagged: finite inputs)
+  double a = 0.0, fs = 0.0, fds = 0.0, qn = 0.0;
+  bool live = (entry & kQueueKeep) != 0, counted = false, tree = false;  // tagged: finite inputs
+  SweepCells c;
+  c.j0 = c.n = 0;
+  c.first_in = c.last_in = false;
+  c.mid = c.first = c.last = 0.0;
+  double r = 0.0;
   if (valid) {
     if (kGen) {
-      const double3 gsrc = gen_source_at(cat, s);
-      a = gsrc.x;
-      fs = gsrc.y;
-      fds = gsrc.z;
+      a = (double)q.a[at + lane];
+      fs = (double)q.f[at + lane];
+      fds = (double)q.d[at + lane];
     } else {
       a = cat->A[s];
       fs = cat->f[s];
@@ -630,35 +554,131 @@ __device__ __noinline__ unsigned prepass_drain_warp(const PrepassArgs& pa, const
                    (((u64)__double_as_longlong(a) >> 52) & 0x7FF) < kMaxAExp)) {
       atomicOr(&pa.rs->err, ERR_INPUT);
     } else if (!live) {
-      wide = slow_span(fs, fds, pa.g) > kSlowLaneBins;
-      if (!wide)
-        live = prepass_decide(prepass_slow(a, fs, fds, pa.g, pa.tb, pa.acc, &pa.rs->err),
-                              pa.tk_bits, pa.tl_bits, nkappa);
+      counted = true;
+      const Sweep sw = make_sweep(fs, fds, g.T, g.T2);
+      if (sw.ka == sw.kb) {
+        // deposited as the common path deposits it, so that every single-bin source is removed
+        // the same way
+        const long long j = sw.ka - g.k_lo;
+        if (j >= 0 && j < g.nb) {
+          u64 c0, c1, c2, qb;
+          if (q_single(a, pa.tb.gq[j], &c0, &c1, &c2, &qb)) {
+            add_parts(pa.acc, j, c0, c1, c2);
+            r = __longlong_as_double((long long)qb);
+          } else {
+            atomicOr(&pa.rs->err, ERR_RANGE);
+          }
+        }
+      } else {
+        long long k0, k1;
+        sweep_bins(sw, g, &k0, &k1);
+        if (k1 >= k0) {
+          const double a2 = __dmul_rn(a, a), inv = sweep_inv_len(sw);
+          c.j0 = (int)(k0 - g.k_lo);
+          c.n = (int)(k1 - k0 + 1);
+          c.first_in = k0 == sw.ka;
+          c.last_in = k1 == sw.kb;
+          c.mid = __dmul_rn(a2, inv);
+          c.first = __dmul_rn(a2, sweep_weight_inv(sw, sw.ka, inv));
+          c.last = __dmul_rn(a2, sweep_weight_inv(sw, sw.kb, inv));
+          tree = tree_takes(pa.tb.tree, a2, inv, k0, k1, &qn);
+        }
+      }
     }
   }
-  unsigned pending = __ballot_sync(0xFFFFFFFFu, wide);
+  // the long sweeps, one after another by the whole warp
+  unsigned pending = __ballot_sync(0xFFFFFFFFu, tree);
   while (pending) {
     const int src = __ffs(pending) - 1;
     pending &= pending - 1;
-    const double sw_a = __shfl_sync(0xFFFFFFFFu, a, src);
-    const double sw_f = __shfl_sync(0xFFFFFFFFu, fs, src);
-    const double sw_fd = __shfl_sync(0xFFFFFFFFu, fds, src);
-    const double rw = prepass_slow_warp(sw_a, sw_f, sw_fd, pa.g, pa.tb, pa.acc, pa.rs);
-    if (lane == src) live = prepass_decide(rw, pa.tk_bits, pa.tl_bits, nkappa);
+    SweepCells t;
+    t.j0 = __shfl_sync(0xFFFFFFFFu, c.j0, src);
+    t.n = __shfl_sync(0xFFFFFFFFu, c.n, src);
+    t.first_in = __shfl_sync(0xFFFFFFFFu, (int)c.first_in, src) != 0;
+    t.last_in = __shfl_sync(0xFFFFFFFFu, (int)c.last_in, src) != 0;
+    t.mid = __shfl_sync(0xFFFFFFFFu, c.mid, src);
+    t.first = __shfl_sync(0xFFFFFFFFu, c.first, src);
+    t.last = __shfl_sync(0xFFFFFFFFu, c.last, src);
+    const double tq = __shfl_sync(0xFFFFFFFFu, qn, src);
+    if (tq > 0.0) {
+      const double rt = tree_deposit(t, tq, pa.tb, pa.acc, pa.rs);
+      if (lane == src) r = rt;
+    }
   }
-  prepass_keep(live, s, a, fs, fds, pa.g, pa.cd, pa.rs);
+  // the others' cells, end to end
+  const int n = tree ? 0 : c.n;
+  int off = n;  // inclusive, then exclusive scan
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xFFFFFFFFu, off, o);
+    if (lane >= o) off += v;
+  }
+  const int total = __shfl_sync(0xFFFFFFFFu, off, 31);
+  off -= n;
+  U128 sum{0ull, 0ull};
+  for (int base = 0; base < total; base += 32) {
+    const int x = base + lane;
+    int src = 0;  // the last source whose cells begin at x or before
+#pragma unroll
+    for (int step = 16; step > 0; step >>= 1) {
+      const int o = __shfl_sync(0xFFFFFFFFu, off, src + step);
+      if (o <= x) src += step;
+    }
+    SweepCells t;
+    const int t_off = __shfl_sync(0xFFFFFFFFu, off, src);
+    t.j0 = __shfl_sync(0xFFFFFFFFu, c.j0, src);
+    t.n = __shfl_sync(0xFFFFFFFFu, n, src);
+    const int ends = __shfl_sync(0xFFFFFFFFu, (c.first_in ? 1 : 0) | (c.last_in ? 2 : 0), src);
+    t.first_in = ends & 1;
+    t.last_in = ends & 2;
+    t.mid = __shfl_sync(0xFFFFFFFFu, c.mid, src);
+    t.first = __shfl_sync(0xFFFFFFFFu, c.first, src);
+    t.last = __shfl_sync(0xFFFFFFFFu, c.last, src);
+    u64 lo = 0ull, hi = 0ull;
+    if (x < total) {
+      const int i = x - t_off, j = t.j0 + i;
+      u64 c0, c1, c2;
+      if (!q_cell(cell_power(t, i), pa.tb.gq[j], &c0, &c1, &c2))
+        atomicOr(&pa.rs->err, ERR_RANGE);
+      add_parts(pa.acc, j, c0, c1, c2);
+      lo = c0 | (c1 << 32);
+      hi = c2;
+    }
+    // sums over the lanes of one source
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      U128 v;
+      v.lo = __shfl_up_sync(0xFFFFFFFFu, lo, o);
+      v.hi = __shfl_up_sync(0xFFFFFFFFu, hi, o);
+      const int vs = __shfl_up_sync(0xFFFFFFFFu, src, o);
+      if (lane >= o && vs == src) {
+        const U128 w = u128_add(v, U128{lo, hi});
+        lo = w.lo;
+        hi = w.hi;
+      }
+    }
+    // each source's last lane of this round
+    const int end = min(off + n, base + 32) - 1 - base;
+    U128 mine;
+    mine.lo = __shfl_sync(0xFFFFFFFFu, lo, end & 31);
+    mine.hi = __shfl_sync(0xFFFFFFFFu, hi, end & 31);
+    if (n > 0 && off < base + 32 && end >= 0) sum = u128_add(sum, mine);
+  }
+  if (n > 0) r = u128_to_dbl_scaled(sum, -32);
+  if (counted) live = prepass_decide(r, pa.tk_bits, pa.tl_bits, nkappa);
+  prepass_keep(live, s, a, fs, fds, g, pa.cd, pa.rs);
   return nkappa;
 }
 
 // Drain the warp's queue while it holds 32 entries or more.
 template <bool kGen>
 __device__ __forceinline__ void prepass_drain_full(const PrepassArgs& pa, const CatalogRef* cat,
-                                                   const long long* q, int& qn,
+                                                   const SlowQueue& q, int& qn,
                                                    unsigned& nkappa) {
   while (qn >= 32) {
     // the last 32 entries: nothing moves down
     __syncwarp();
-    nkappa += prepass_drain_warp<kGen>(pa, cat, q + qn - 32, 32);
+    nkappa += prepass_drain_warp<kGen>(pa, cat, q, qn - 32, 32);
     qn -= 32;
     __syncwarp();
   }
@@ -745,10 +765,13 @@ __device__ __forceinline__ SourceParts source_parts(double a, double gq, int tk_
 // The deposit, the count and the candidate test; a source of the FP64 path, or one to keep as
 // a candidate, is appended to the warp's queue q (qn entries, the same in every lane; every
 // lane of the warp calls it together).  rep_lane: the replica of this lane's sources.
+// kGen: f and fdot go with it (FP32 numbers).
+template <bool kGen>
 __device__ __forceinline__ void deposit_source(const PlacedSource p, SourceParts c, long long s,
-                                               double a, const PrepassArgs& pa,
-                                               const HotBins& hot_bins, u64* rep_lane,
-                                               long long* q, int& qn, unsigned& nkappa) {
+                                               double a, float f, float fdot,
+                                               const PrepassArgs& pa, const HotBins& hot_bins,
+                                               u64* rep_lane, const SlowQueue& q, int& qn,
+                                               unsigned& nkappa) {
   const int lane = threadIdx.x & 31;
   bool set_aside = p.j == -2, keep = false;
   if (p.j >= 0) {
@@ -774,7 +797,15 @@ __device__ __forceinline__ void deposit_source(const PlacedSource p, SourceParts
   }
   const unsigned sm = __ballot_sync(0xFFFFFFFFu, set_aside);
   if (sm) {
-    if (set_aside) q[qn + __popc(sm & ((1u << lane) - 1u))] = keep ? s | kQueueKeep : s;
+    if (set_aside) {
+      const int at = qn + __popc(sm & ((1u << lane) - 1u));
+      q.s[at] = keep ? s | kQueueKeep : s;
+      if (kGen) {
+        q.a[at] = (float)a;
+        q.f[at] = f;
+        q.d[at] = fdot;
+      }
+    }
     qn += __popc(sm);
   }
 }
@@ -835,9 +866,9 @@ __global__ void __launch_bounds__(kPrepassThreads, 1)
   if (scat.staged == kCatGenerated) return;  // k_prepass_gen's catalog
   const long long N = scat.n;
   double* const stages = pre_smem + (size_t)warp * kPreStages * 3 * kPreStep;
-  long long* const myq = reinterpret_cast<long long*>(
-                             pre_smem + (size_t)kPreWarps * kPreStages * 3 * kPreStep) +
-                         warp * kSlowWarpCap;
+  SlowQueue myq = {};
+  myq.s = reinterpret_cast<long long*>(pre_smem + (size_t)kPreWarps * kPreStages * 3 * kPreStep) +
+          warp * kSlowWarpCap;
   HotBins hot;
   hot.w = reinterpret_cast<unsigned*>(pre_smem + (size_t)kPreWarps *
                                                      (kPreStages * 3 * kPreStep + kSlowWarpCap));
@@ -934,7 +965,8 @@ __global__ void __launch_bounds__(kPrepassThreads, 1)
     for (int i = 0; i < kPrePer; ++i) sp[i] = source_parts(av[i], pl[i].gq, pa.tk_hi);
 #pragma unroll
     for (int i = 0; i < kPrePer; ++i)
-      deposit_source(pl[i], sp[i], s0 + 32 * i, av[i], pa, hot, rep_lane, myq, qn, nkappa);
+      deposit_source<false>(pl[i], sp[i], s0 + 32 * i, av[i], 0.0f, 0.0f, pa, hot, rep_lane, myq,
+                            qn, nkappa);
     prepass_drain_full<false>(pa, &scat, myq, qn, nkappa);
   }
   if (timeout) {
@@ -945,7 +977,7 @@ __global__ void __launch_bounds__(kPrepassThreads, 1)
     __syncwarp();
   } else if (qn > 0) {
     __syncwarp();
-    nkappa += prepass_drain_warp<false>(pa, &scat, myq, qn);
+    nkappa += prepass_drain_warp<false>(pa, &scat, myq, 0, qn);
   }
   for (int o = 16; o > 0; o >>= 1) nkappa += __shfl_xor_sync(0xFFFFFFFFu, nkappa, o);
   if (lane == 0 && nkappa) atomicAdd(&rs->ncand, (unsigned long long)nkappa);
@@ -964,48 +996,135 @@ __global__ void __launch_bounds__(kPrepassThreads, 1)
 }
 
 // The catalog pass over a generated catalog: every source computed from (seed, index) where
-// the pass over a stored catalog loads it, then the same per-source step.  Generation is
-// ~300 FP32 and integer instructions per source, so there is nothing to stage: each warp takes
-// runs of 32 kGenPer sources from the tile counter.  The other pass leaves a generated catalog
-// to this one, and this one leaves every other catalog to it.
+// the pass over a stored catalog loads it, then the same per-source step.  The other pass leaves
+// a generated catalog to this one, and this one leaves every other catalog to it.
+//
+// Bound: instruction issue.  An attempt at a source's Gamma variate is refused one time in four;
+// with a loop per lane a warp went on until its last lane was done, 3.5 attempts and half its
+// lanes idle (1 377 instructions per 32 sources; 1 034 now, 3e7 sources 1 340 -> 940 us).  So a warp keeps refused sources in a queue and
+// tries 32 of them at a time, and sources with their variate in another (for the paper's
+// population one for each way through the incomplete gamma function), from which it computes
+// the rest 32 at a time.  The order of the sources changes nothing: deposits are integers.
 constexpr int kGenThreads = 256;
-constexpr int kGenPer = 8;  // sources per lane per run
+constexpr int kGenPer = 8;     // sources per lane per run
+constexpr int kGenQueue = 64;  // less than 32 entries before 32 are added
+struct GenQueues {
+  long long retry_s[kGenQueue], ready_s[2][kGenQueue], slow_s[kGenQueue];
+  float ready_x[2][kGenQueue], slow_a[kGenQueue], slow_f[kGenQueue], slow_d[kGenQueue];
+  int retry_t[kGenQueue];
+};
 
 __global__ void __launch_bounds__(kGenThreads, 4)
     k_prepass_gen(const __grid_constant__ PrepassArgs pa) {
   RunState* const rs = pa.rs;
   __shared__ CatalogRef scat;
-  __shared__ long long slow_q[kGenThreads / 32][kSlowWarpCap];
+  __shared__ GenQueues queues[kGenThreads / 32];
   if (threadIdx.x == 0) scat = *pa.cat;
   __syncthreads();
   if (scat.staged != kCatGenerated) return;
   const long long N = scat.n;
+  const GenParams& gen = scat.gen;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned below = (1u << lane) - 1u;
+  GenQueues& q = queues[warp];
+  SlowQueue slow;
+  slow.s = q.slow_s;
+  slow.a = q.slow_a;
+  slow.f = q.slow_f;
+  slow.d = q.slow_d;
   unsigned nkappa = 0;  // a lane's share of the catalog
-  // a source's replica is its index mod kAccReplicas, the same for all of a lane's sources
   u64* const rep_lane = pa.rep.w + 2 * (size_t)(lane % kAccReplicas) * pa.rep.nbins;
-  long long* myq = slow_q[warp];
-  int qn = 0;
+  int qn = 0, nretry = 0, nready0 = 0, nready1 = 0;
   constexpr long long kRun = 32LL * kGenPer;
+  long long next = 0, run_end = 0;  // the warp's run of fresh sources
+  bool more = true;
   for (;;) {
-    unsigned long long r0 = 0;
-    if (lane == 0) r0 = atomicAdd(&rs->next_tile, 1ull);
-    const long long base = (long long)__shfl_sync(0xFFFFFFFFu, r0, 0) * kRun;
-    if (base >= N) break;
-#pragma unroll 1
-    for (int k = 0; k < kGenPer; ++k) {
-      const long long s = base + 32 * k + lane;
-      double3 src = make_double3(0.0, 0.0, 0.0);
-      if (s < N) src = gen_source_at(&scat, s);
-      const PlacedSource pl = place_source(s < N, src.x, src.y, src.z, pa);
-      deposit_source(pl, source_parts(src.x, pl.gq, pa.tk_hi), s, src.x, pa, HotBins{nullptr, 0},
-                     rep_lane, myq, qn, nkappa);
-      prepass_drain_full<true>(pa, &scat, myq, qn, nkappa);
+    int what;  // 0, 1: the rest of sources of that class; 2: refused sources again; 3: fresh ones
+    if (nready0 >= 32) {
+      what = 0;
+    } else if (nready1 >= 32) {
+      what = 1;
+    } else if (nretry >= 32) {
+      what = 2;
+    } else {
+      if (more && next >= run_end) {
+        unsigned long long r0 = 0;
+        if (lane == 0) r0 = atomicAdd(&rs->next_tile, 1ull);
+        next = (long long)__shfl_sync(0xFFFFFFFFu, r0, 0) * kRun;
+        run_end = next + kRun;
+        more = next < N;
+      }
+      if (more)
+        what = 3;
+      else if (nretry > 0)
+        what = 2;
+      else if (nready0 > 0)
+        what = 0;
+      else if (nready1 > 0)
+        what = 1;
+      else
+        break;
+    }
+    if (what >= 2) {
+      long long s = next + lane;
+      int t = 0;
+      bool valid = s < N;
+      if (what == 2) {
+        const int cnt = min(nretry, 32);
+        nretry -= cnt;
+        valid = lane < cnt;
+        s = valid ? q.retry_s[nretry + lane] : 0;
+        t = valid ? q.retry_t[nretry + lane] : 0;
+        __syncwarp();
+      } else {
+        next += 32;
+        more = next < N;
+      }
+      float X;
+      bool ok = gen_gamma_try(gen, (unsigned)(unsigned long long)s,
+                              (unsigned)((unsigned long long)s >> 32), t, &X);
+      if (!ok && t + 1 >= kGammaTries) {
+        X = gen.d;
+        ok = true;
+      }
+      const unsigned no = __ballot_sync(0xFFFFFFFFu, valid && !ok);
+      if (valid && !ok) {
+        const int at = nretry + __popc(no & below);
+        q.retry_s[at] = s;
+        q.retry_t[at] = t + 1;
+      }
+      nretry += __popc(no);
+      const int cls = gen_class(gen, X);
+      const unsigned y0 = __ballot_sync(0xFFFFFFFFu, valid && ok && cls == 0);
+      const unsigned y1 = __ballot_sync(0xFFFFFFFFu, valid && ok && cls == 1);
+      if (valid && ok) {
+        const int at = cls ? nready1 + __popc(y1 & below) : nready0 + __popc(y0 & below);
+        q.ready_s[cls][at] = s;
+        q.ready_x[cls][at] = X;
+      }
+      nready0 += __popc(y0);
+      nready1 += __popc(y1);
+      __syncwarp();
+    } else {
+      const int have = what ? nready1 : nready0, cnt = min(have, 32), at = have - cnt + lane;
+      if (what)
+        nready1 -= cnt;
+      else
+        nready0 -= cnt;
+      const bool valid = lane < cnt;
+      const long long s = valid ? q.ready_s[what][at] : 0;
+      const float X = valid ? q.ready_x[what][at] : (what ? gen.alpha + 2.0f : 0.5f);
+      __syncwarp();
+      float a, f, fd;
+      gen_rest(gen, s, X, &a, &f, &fd);
+      const PlacedSource pl = place_source(valid, (double)a, (double)f, (double)fd, pa);
+      deposit_source<true>(pl, source_parts((double)a, pl.gq, pa.tk_hi), s, (double)a, f, fd, pa,
+                           HotBins{nullptr, 0}, rep_lane, slow, qn, nkappa);
+      prepass_drain_full<true>(pa, &scat, slow, qn, nkappa);
     }
   }
   __syncwarp();
-  if (qn > 0)
-    nkappa += prepass_drain_warp<true>(pa, &scat, myq, qn);
+  if (qn > 0) nkappa += prepass_drain_warp<true>(pa, &scat, slow, 0, qn);
   for (int o = 16; o > 0; o >>= 1) nkappa += __shfl_xor_sync(0xFFFFFFFFu, nkappa, o);
   if (lane == 0 && nkappa) atomicAdd(&rs->ncand, (unsigned long long)nkappa);
 }
@@ -2652,6 +2771,13 @@ __device__ __forceinline__ bool near_threshold(double r2, double th2) {
   return fabs(__dsub_rn(r2, th2)) < __dmul_rn(2e-9, th2);
 }
 
+// Take a cell's deposit from its bin (one beyond the range was never deposited).
+__device__ __forceinline__ void remove_cell(unsigned long long* acc, long long j, double c,
+                                            double gq) {
+  u64 c0, c1, c2;
+  if (q_cell(c, gq, &c0, &c1, &c2)) sub_parts(acc, j, c0, c1, c2);
+}
+
 // Remove the parts of candidate c that the catalog pass deposited: bins k0 + off,
 // k0 + off + step, ... of its sweep.
 __device__ __forceinline__ void remove_part(const Cands& cd, long long c, const Grid& g,
@@ -2676,13 +2802,13 @@ __device__ __forceinline__ void remove_part(const Cands& cd, long long c, const 
   long long k1 = sw.kb < g.k_lo + g.nb - 1 ? sw.kb : g.k_lo + g.nb - 1;
   const double inv = sweep_inv_len(sw);
   double q;
-  if (step == 32 && tree_takes(tb.tree, a2, inv, k0, k1, &q)) {  // as prepass_slow_warp
+  if (step == 32 && tree_takes(tb.tree, a2, inv, k0, k1, &q)) {  // as tree_deposit
     if (!(q > 0.0)) return;
     const TreeSpan t = tree_span(sw.ka - g.k_lo, sw.kb - g.k_lo, k0 - g.k_lo, k1 - g.k_lo);
     for (int x = off; x < t.nbins; x += 32) {
       const int j = tree_bin(t, x);
       const double w = sweep_weight_inv(sw, g.k_lo + j, inv);
-      if (w > 0.0) remove_q(acc, j, __dmul_rn(__dmul_rn(a2, w), tb.gq[j]));
+      if (w > 0.0) remove_cell(acc, j, __dmul_rn(a2, w), tb.gq[j]);
     }
     u64 c0, c1, c2;
     q_parts(q, &c0, &c1, &c2);
@@ -2700,7 +2826,7 @@ __device__ __forceinline__ void remove_part(const Cands& cd, long long c, const 
     double w = sweep_weight_inv(sw, k, inv);
     if (w > 0.0) {
       long long j = k - g.k_lo;
-      remove_q(acc, j, __dmul_rn(__dmul_rn(a2, w), tb.gq[j]));
+      remove_cell(acc, j, __dmul_rn(a2, w), tb.gq[j]);
       d.mark_next(j / Kc);
     }
   }
