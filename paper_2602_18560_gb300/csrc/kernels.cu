@@ -2645,6 +2645,61 @@ __device__ double rho2_exact_warp(const Grid& g, const Tables& tb, const double*
   return __dmul_rn(4.0, acc);
 }
 
+// 1 / x for x > 0 within about 2^-43: the FP32 reciprocal of the mantissa and one FP64 Newton step,
+// two FP64 instructions where a division takes some twenty.
+__device__ __forceinline__ double rcp_newton(double x) {
+  const u64 b = (u64)__double_as_longlong(x);
+  const int e = (int)(b >> 52) & 0x7FF;
+  if (e == 0 || e > 2040) return __drcp_rn(x);
+  const float m = __uint_as_float(0x3F800000u | (unsigned)((b >> 29) & 0x7FFFFFu));
+  const unsigned r = __float_as_uint(__fdividef(1.0f, m));  // in (1/2, 1]
+  const int er = 2046 - e + ((int)(r >> 23) - 127);
+  if (er < 1) return __drcp_rn(x);
+  const double y = __longlong_as_double((i64)(((u64)er << 52) | ((u64)(r & 0x7FFFFFu) << 29)));
+  return __fma_rn(__fma_rn(-x, y, 1.0), y, y);
+}
+
+// rho^2 of a sweep of very many bins by the whole CTA, for a decision that its screen left open:
+// the terms of rho2_exact with the common factors outside the sum and the reciprocals of S_n
+// within 2^-43, so within 1e-12 of it, far inside the near-threshold band.  The value is in every
+// thread.  (One warp with a division per bin took some 30 ms for a sweep of the whole 4-year
+// band, and held the launch: a simulation that met one 9.7 ms on average over three seeds, now 3.0.)
+__device__ double rho2_cta(const Grid& g, const Tables& tb, const double* __restrict__ Sg,
+                           double a2, double lo, double hi) {
+  __shared__ double part[32];
+  Sweep sw;
+  sw.lo = lo;
+  sw.hi = hi;
+  sw.ka = (i64)floor(__dadd_rn(lo, 0.5));
+  sw.kb = (i64)floor(__dadd_rn(hi, 0.5));
+  const long long k0 = sw.ka > g.k_lo ? sw.ka : g.k_lo;
+  const long long k1 = sw.kb < g.k_lo + g.nb - 1 ? sw.kb : g.k_lo + g.nb - 1;
+  double acc = 0.0;
+#pragma unroll 4
+  for (long long k = k0 + threadIdx.x; k <= k1; k += blockDim.x) {
+    const long long j = k - g.k_lo;
+    const double y = rcp_newton(__dadd_rn(tb.S[j], Sg[j]));
+    const bool inner = k > sw.ka && k < sw.kb;
+    acc = __fma_rn(tb.R[j], inner ? y : 0.0, acc);
+  }
+  acc = __dmul_rn(acc, sweep_inv_len(sw));
+  if (threadIdx.x < 2) {  // the sweep's first and last cells, with their own weights
+    const long long k = threadIdx.x ? sw.kb : sw.ka;
+    if (k >= k0 && k <= k1) {
+      const long long j = k - g.k_lo;
+      const double sn = __dadd_rn(tb.S[j], Sg[j]);
+      acc = __dadd_rn(acc, __ddiv_rn(__dmul_rn(tb.R[j], sweep_weight(sw, k)), sn));
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) acc = __dadd_rn(acc, __shfl_xor_sync(0xFFFFFFFFu, acc, o));
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  double v = 0.0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = __dadd_rn(v, part[w]);
+  return __dmul_rn(4.0, __dmul_rn(__dmul_rn(g.t5, a2), v));
+}
+
 __device__ double rho2_exact(const Grid& g, const Tables& tb, const double* __restrict__ Sg,
                              double a2, double lo, double hi) {
   Sweep sw;
@@ -2866,6 +2921,9 @@ __device__ __forceinline__ void snr_wide_decide(
 // grid, the lanes sharing the bins: no launch waits on one thread walking a long sweep, nor
 // on one warp walking many.
 
+constexpr int kOpenMax = 16;     // sweeps a CTA sets aside
+constexpr int kOpenBins = 4096;  // of more bins than this
+
 __global__ void __launch_bounds__(256) k_snr_resolve(
     const __grid_constant__ Cands cd, const __grid_constant__ Grid g, const __grid_constant__ Tables tb, const double* __restrict__ Sg, const float* __restrict__ inv_f,
     double th2, double rtol, int mode, unsigned char* __restrict__ resolved,
@@ -2931,7 +2989,12 @@ __global__ void __launch_bounds__(256) k_snr_resolve(
       }
     }
   }
-  // the long sweeps, one per warp at a time
+  // the long sweeps, one per warp at a time; the very long ones that the screen leaves open are
+  // set aside for the whole CTA (the few that find no room are decided by their warp)
+  __shared__ long long open_c[kOpenMax];
+  __shared__ int open_n;
+  if (threadIdx.x == 0) open_n = 0;
+  __syncthreads();
   const long long nwide = snr_head[3];
   for (long long wi = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; wi < nwide;
        wi += nwarps) {
@@ -2960,6 +3023,15 @@ __global__ void __launch_bounds__(256) k_snr_resolve(
     int kcount;
     float r2;
     if (screen_tree(cd, cw, pkw, g, tb, inv_f, &r2, &kcount)) {
+      if (mode == 0 && pkw.y > kOpenBins && screen_decide(r2, kcount, th2f, mode) < 0) {
+        int at = 0;
+        if (lane == 0) at = atomicAdd(&open_n, 1);
+        at = __shfl_sync(0xFFFFFFFFu, at, 0);
+        if (at < kOpenMax) {
+          if (lane == 0) open_c[at] = cw;
+          continue;
+        }
+      }
       snr_wide_decide(cd, cw, g, tb, Sg, th2, th2f, mode, r2, kcount, resolved, acc, di, Kc,
                       local_new, local_exact, local_near, local_unc);
     } else {
@@ -2974,6 +3046,23 @@ __global__ void __launch_bounds__(256) k_snr_resolve(
       }
       snr_wide_decide(cd, cw, g, tb, Sg, th2, th2f, mode, r2, kchain + 5, resolved, acc, di, Kc,
                       local_new, local_exact, local_near, local_unc);
+    }
+  }
+  __syncthreads();
+  for (int i = 0; i < min(open_n, kOpenMax); ++i) {
+    const long long co = open_c[i];
+    const double v = rho2_cta(g, tb, Sg, cd.a2[co], cd.lo[co], cd.hi[co]);
+    if (threadIdx.x == 0) {
+      ++local_exact;
+      if (near_threshold(v, th2)) ++local_near;
+    }
+    if (v > th2 && threadIdx.x < 32) {
+      if (lane == 0) {
+        cd.res[co] = 1;
+        resolved[cd.src[co]] = 1;
+        ++local_new;
+      }
+      remove_part(cd, co, g, tb, acc, di, Kc, lane, 32);
     }
   }
   for (int o = 16; o > 0; o >>= 1) {

@@ -96,3 +96,30 @@ def test_power_beyond_the_range_is_still_refused():
         with pytest.raises(gbsub.SubError) as ei:
             s.run()
         assert ei.value.code == gbsub.ERANGE
+
+
+@pytest.mark.parametrize("first, length", [(-20.3, 75_838.7), (3000.2, 5000.4), (40000.4, -5100.1)])
+@pytest.mark.parametrize("delta", [1e-6, -1e-6, 3e-8, -3e-8])
+def test_decisions_left_open_by_the_screen(first, length, delta):
+    # one long sweep at rho = rho_th (1 + delta) on a faint background: its FP32 screen cannot
+    # tell, the FP64 sum of the whole CTA does
+    k_lo, n = oracle.grid(T, 1e-4, F_MAX)
+    S, R = oracle.tables(T, k_lo, n, True)
+    j = np.arange(n)
+    f = np.append((k_lo + j + 0.1) / T, (k_lo + first) / T)
+    fdot = np.append(np.zeros(n), length / T**2)
+    A = np.append(np.sqrt(5.0 * 0.1 * S / (T * R)), 1e-23)
+    for _ in range(8):  # the sweep's own power moves S_gal a little
+        P = oracle.power(T, R, oracle.deposit(T, k_lo, n, A, f, fdot))
+        rho2 = oracle.snr2(T, k_lo, n, S, R, oracle.smooth(gbsub.MEAN, 1001, P), A[-1:], f[-1:],
+                           fdot[-1:])[0]
+        A[-1] *= 7.0 * (1.0 + delta) / np.sqrt(rho2)
+    kw = dict(T_obs=T, estimator=gbsub.MEAN, window=1001, f_max=F_MAX)
+    ref = oracle.run(oracle.make_params(**kw), A, f, fdot)
+    assert bool(ref["resolved"][-1]) == (delta > 0)
+    with gbsub.Subtraction(**kw) as s:
+        s.load(A, f, fdot)
+        st = s.run()
+        res = s.resolved().astype(bool)
+    assert st.n_exact > 0
+    assert np.array_equal(res, ref["resolved"])
