@@ -536,18 +536,9 @@ static Dirty dirty_of(sub_ctx* c, bool track) {
 }
 
 static cudaError_t enqueue_pre(sub_ctx* c, cudaStream_t st) {
-  const int64_t n = c->grid.nb;
-  cudaError_t e;
-  if ((e = cudaMemsetAsync(c->acc, 0, (size_t)n * 32, st))) return e;
-  if ((e = cudaMemsetAsync(c->rep.w, 0, (size_t)kAccReplicas * c->rep.nbins * 16, st))) return e;
-  if ((e = cudaMemsetAsync(c->rs, 0, sizeof(RunState), st))) return e;
-  // the first iteration reads set 0: every chunk is new
-  if ((e = cudaMemsetAsync(c->dirty, 1, (size_t)c->plan.nch, st))) return e;
-  if ((e = cudaMemsetAsync(c->dirty + c->plan.nch, 0, (size_t)c->plan.nch, st))) return e;
-  launch_build_lists(dirty_of(c, true), c->lists, c->list_counts, c->rs, st);
-  if ((e = cudaMemsetAsync(c->new_hist, 0, (size_t)c->p.max_iter * 4, st))) return e;
   // sized by the capacity, not the catalog: the captured graph serves every catalog that fits
-  if ((e = cudaMemsetAsync(c->resolved, 0, (size_t)c->cap_N, st))) return e;
+  launch_begin(c->acc, c->grid.nb, c->rep, c->resolved, c->cap_N, c->dirty, c->plan.nch, c->lists,
+               c->list_counts, c->new_hist, c->p.max_iter, c->rs, c->nsm_run, st);
   {
     KTimer t(c, st, SUB_K_PREPASS);
     launch_prepass(c->dcat, c->cap_N, c->grid, tables_of(c), thr_kappa_of(c), thr_live_of(c),

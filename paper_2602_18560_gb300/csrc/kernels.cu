@@ -1184,7 +1184,7 @@ void launch_prepass(const CatalogRef* cat, long long cap, const Grid& g, const T
   pa.cd = cd;
   pa.rs = rs;
   pa.test_flags = test_flags;
-  k_prepass<<<bl, kPrepassThreads, kPrepassSmem, st>>>(pa);
+  launch_after(k_prepass, bl, kPrepassThreads, kPrepassSmem, st, pa);  // after launch_begin
   // the generated-catalog pass: resident CTAs, at most one per run of sources
   const long long runs = (cap + 32LL * kGenPer - 1) / (32LL * kGenPer);
   const long long glim = (long long)nsm * 4 * (kGenThreads / 32);
@@ -3233,14 +3233,53 @@ __device__ void build_lists_cta(const unsigned char* __restrict__ cur, int nch,
   if (threadIdx.x < kNumLists) counts[threadIdx.x] = cnt[threadIdx.x];
 }
 
-__global__ void k_build_lists(Dirty d, int* lists, int* counts, RunState* rs) {
-  build_lists_cta(d.base + (size_t)(d.rs->iter & 1) * d.nch, d.nch, lists, counts);
-  __syncthreads();
-  if (threadIdx.x < kNumLists) rs->work[threadIdx.x] += (unsigned long long)counts[threadIdx.x];
+// The state a run begins with: the spectrum's words, their replicas and the resolved mask zero,
+// every chunk marked in the set the first iteration reads, none in the other one, and that
+// iteration's work lists full.  Writes of (32 n + replicas + N) bytes, a few us at the most; as
+// seven clears and a one-CTA list kernel the launches made it 12-18 us more of every run (1 yr, 1e4
+// sources 187 -> 173 us; 24 served requests 4.03 -> 3.69 ms).
+__global__ void __launch_bounds__(256) k_begin(ulonglong2* acc, long long n_acc, ulonglong2* rep,
+                                               long long n_rep, ulonglong2* resolved,
+                                               long long n_resolved, unsigned char* dirty, int nch,
+                                               int* lists, int* counts, int* new_hist,
+                                               int max_iter, RunState* rs) {
+  const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const long long step = (long long)gridDim.x * blockDim.x;
+  chain_next();
+  const ulonglong2 z = make_ulonglong2(0ull, 0ull);
+  for (long long i = t0; i < n_acc; i += step) acc[i] = z;
+  for (long long i = t0; i < n_rep; i += step) rep[i] = z;
+  for (long long i = t0; i < n_resolved; i += step) resolved[i] = z;
+  for (long long i = t0; i < max_iter; i += step) new_hist[i] = 0;
+  for (long long i = t0; i <= nch; i += step) {
+    if (i < nch) {
+      dirty[i] = 1;
+      dirty[nch + i] = 0;
+    }
+#pragma unroll
+    for (int l = 0; l < kNumLists; ++l)
+      if (i < nch || l == kListTile) lists[(size_t)l * (nch + 1) + i] = (int)i;
+  }
+  if (t0 == 0) {
+    RunState r{};
+    for (int l = 0; l < kNumLists; ++l) {
+      counts[l] = nch + (l == kListTile ? 1 : 0);
+      r.work[l] = (unsigned long long)counts[l];
+    }
+    *rs = r;
+  }
 }
 
-void launch_build_lists(Dirty d, int* lists, int* counts, RunState* rs, cudaStream_t st) {
-  k_build_lists<<<1, 1024, 0, st>>>(d, lists, counts, rs);
+void launch_begin(unsigned long long* acc, long long nb, AccReplicas rep, unsigned char* resolved,
+                  long long cap, unsigned char* dirty, int nch, int* lists, int* counts,
+                  int* new_hist, int max_iter, RunState* rs, int nsm, cudaStream_t st) {
+  const long long n_acc = nb * 2, n_rep = (long long)kAccReplicas * rep.nbins;
+  const long long n_res = (cap + 15) / 16;  // the mask's allocation is a multiple of 256 bytes
+  const long long most = n_acc > n_res ? n_acc : n_res;
+  const long long want = (most + 255) / 256, lim = (long long)nsm * 8;
+  k_begin<<<(unsigned)(want < lim ? want : lim), 256, 0, st>>>(
+      (ulonglong2*)acc, n_acc, (ulonglong2*)rep.w, n_rep, (ulonglong2*)resolved, n_res, dirty, nch,
+      lists, counts, new_hist, max_iter, rs);
 }
 
 __global__ void k_control(RunState* rs, int max_iter, double rtol, int* new_hist,
