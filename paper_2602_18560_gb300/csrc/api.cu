@@ -775,8 +775,10 @@ void gbsub::ctx_set_test_flags(sub_ctx* c, int flags) {
 // Persistent grids from the plan's launch settings, at 1/grid_div of the GPU.
 static void replan(sub_ctx* c) {
   const int div = c->grid_div;
+  c->plan.shared = div > 1 ? 1 : 0;
   plan_grids(c->plan);
-  int* res[] = {&c->plan.res_sort, &c->plan.res_median, &c->plan.res_prefix, &c->plan.res_mean};
+  int* res[] = {&c->plan.res_sort, &c->plan.res_median, &c->plan.res_median_all,
+                &c->plan.res_prefix, &c->plan.res_mean};
   for (int* r : res) *r = (*r / div) > 0 ? *r / div : 1;
   c->nsm_run = c->nsm / div > 0 ? c->nsm / div : 1;
 }

@@ -2306,12 +2306,17 @@ __global__ void __launch_bounds__(512, 2) k_median_wm(
 
 // Two outputs per thread: a few tiles' latency is what a late iteration waits for.  At most 512
 // threads, so that two CTAs share an SM (W = 2000, every tile: 212 us, 228 with 1024).
-static int median_threads(const SmoothPlan& pl) {
+// Where tiles are many (all: every one of them; shared: other contexts' tiles too) their rate
+// counts, and four CTAs of 256 threads cover each other's barriers better than two of 512, as long
+// as the build stays unrolled (eight words per warp: chunks of up to 1024).  W = 1000, 1.25e6 bins:
+// an estimate of every tile 213 us (220.5 with 512 threads), 64 runs at once 11.95 ms (12.2); a
+// run by itself over 3e7 sources, with its late iterations, 1262 us (1209), so it keeps 512.
+static int median_threads(const SmoothPlan& pl, bool all) {
   if (pl.median_th) return pl.median_th;
   int t = ((pl.Kc / 2 + 31) / 32) * 32;
   if (t < 32) t = 32;
-  if (t > 512) t = 512;
-  return t;
+  const int most = (all || pl.shared) && pl.Kc <= 1024 ? 256 : 512;
+  return t < most ? t : most;
 }
 
 size_t median_smem_bytes(int Kc, int threads, int key_bytes) {
@@ -2325,9 +2330,10 @@ size_t median_smem_bytes(int Kc, int threads, int key_bytes) {
 
 void launch_running_median(const unsigned long long* skey, const uint16_t* srank, long long n,
                            const SmoothPlan& pl, SgOut o, Dirty d, cudaStream_t st) {
-  int th = median_threads(pl);
+  const bool all = d.lists == nullptr;
+  const int th = median_threads(pl, all);
   size_t smem = median_smem_bytes(pl.Kc, th, pl.fp32_keys ? 4 : 8);
-  int bl = persistent_grid(pl, pl.nch + 1, pl.res_median);
+  int bl = persistent_grid(pl, pl.nch + 1, all ? pl.res_median_all : pl.res_median);
   SmoothPlan p = pl;
   p.median_mp = median_pad(2 * pl.Kc, th);
   if (pl.fp32_keys)
@@ -3344,17 +3350,18 @@ void launch_control(RunState* rs, int max_iter, double rtol, int* new_hist,
 }
 
 void plan_grids(SmoothPlan& pl) {
-  pl.res_sort = pl.res_median = pl.res_prefix = pl.res_mean = 0;
+  pl.res_sort = pl.res_median = pl.res_median_all = pl.res_prefix = pl.res_mean = 0;
   if (pl.nsm <= 0) return;
   with_sort_kernel<true>(pl, [&](auto kern) {
     pl.res_sort = resident_ctas(pl, kern, sort_threads(pl), sort_smem(pl));
   });
-  if (pl.fp32_keys)
-    pl.res_median = resident_ctas(pl, k_median_wm<uint32_t>, median_threads(pl),
-                                  median_smem_bytes(pl.Kc, median_threads(pl), 4));
-  else
-    pl.res_median = resident_ctas(pl, k_median_wm<u64>, median_threads(pl),
-                                  median_smem_bytes(pl.Kc, median_threads(pl), 8));
+  for (bool all : {false, true}) {
+    const int th = median_threads(pl, all);
+    const size_t smem = median_smem_bytes(pl.Kc, th, pl.fp32_keys ? 4 : 8);
+    (all ? pl.res_median_all : pl.res_median) =
+        pl.fp32_keys ? resident_ctas(pl, k_median_wm<uint32_t>, th, smem)
+                     : resident_ctas(pl, k_median_wm<u64>, th, smem);
+  }
   if (prefix_per(pl) == kPrefixPer)
     pl.res_prefix = resident_ctas(pl, k_chunk_prefix<true, kPrefixPer>, prefix_threads(pl),
                                   prefix_smem(pl, true));

@@ -113,7 +113,9 @@ struct SmoothPlan {
   int nsm;      // SMs for persistent grids (0: one CTA per work item)
   int fp32_keys;  // median on the FP32-rounded values (mixed precision): 4-byte keys
   double key_scale;  // power of two the values are scaled by before rounding to FP32
-  int res_sort, res_median, res_prefix, res_mean;  // CTAs resident at once (plan_grids)
+  // CTAs resident at once (plan_grids); res_median_all: where every tile is computed
+  int res_sort, res_median, res_median_all, res_prefix, res_mean;
+  int shared;     // 1: the GPU is shared with other contexts' runs (SUB_TUNE_GRID_DIV)
   int sort_e;     // elements per sorting thread (2, 4, 8), 0: chosen from kpad
   int median_th;  // threads per median tile (multiple of 32, <= 512), 0: chosen from Kc
   int median_mp;  // positions of a median tile filled up to whole words per warp (at launch)
