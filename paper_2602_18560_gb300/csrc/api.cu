@@ -629,7 +629,7 @@ static cudaError_t enqueue_body(sub_ctx* c, cudaStream_t st, unsigned long long 
                        c->p.conv_rtol, snr_mode(c), c->resolved, c->acc, rs, dirty_of(c, true),
                        c->plan.Kc, sg_radius_of(c), c->nsm_run, st);
   }
-  { KTimer t(c, st, SUB_K_CONTROL); launch_control(rs, c->p.max_iter, c->p.conv_rtol, c->new_hist, handle, use_cond, c->dirty, c->plan.nch, c->lists, c->list_counts, st); }
+  { KTimer t(c, st, SUB_K_CONTROL); launch_control(rs, c->p.max_iter, c->p.conv_rtol, c->new_hist, handle, use_cond, c->dirty, c->plan.nch, c->lists, c->list_counts, c->h_rs, st); }
   return cudaGetLastError();
 }
 
@@ -710,7 +710,6 @@ static int run_host_loop(sub_ctx* c) {
 }
 
 static int fill_stats(sub_ctx* c, sub_stats* st) {
-  CU(cudaMemcpyAsync(c->h_rs, c->rs, sizeof(RunState), cudaMemcpyDeviceToHost, c->stream), c);
   CU(cudaStreamSynchronize(c->stream), c);
   const RunState& r = *c->h_rs;
   int status = SUB_OK;
@@ -869,7 +868,6 @@ extern "C" int sub_get_resolved_mask(sub_ctx* c, uint8_t* mask, int64_t n, int w
 extern "C" int sub_get_history(sub_ctx* c, int32_t* hist, int32_t cap) {
   if (!c || (cap > 0 && !hist)) return SUB_EINVAL;
   if (!c->ran) { set_err(c, "no run yet"); return SUB_ESTATE; }
-  CU(cudaMemcpyAsync(c->h_rs, c->rs, sizeof(RunState), cudaMemcpyDeviceToHost, c->stream), c);
   CU(cudaStreamSynchronize(c->stream), c);
   int m = c->h_rs->iter < cap ? c->h_rs->iter : cap;
   if (m > 0) {
@@ -998,7 +996,6 @@ extern "C" int sub_get_timing(sub_ctx* c, float* prepass_ms, float* loop_ms, flo
 extern "C" int sub_get_work(sub_ctx* c, int64_t* work, int32_t n) {
   if (!c || (n > 0 && !work)) return SUB_EINVAL;
   if (!c->ran) { set_err(c, "no run yet"); return SUB_ESTATE; }
-  CU(cudaMemcpyAsync(c->h_rs, c->rs, sizeof(RunState), cudaMemcpyDeviceToHost, c->stream), c);
   CU(cudaStreamSynchronize(c->stream), c);
   for (int i = 0; i < n && i < 4; ++i) work[i] = (int64_t)c->h_rs->work[i];
   return SUB_OK;
@@ -1026,7 +1023,6 @@ extern "C" int sub_snr_check(sub_ctx* c, int64_t* src, float* rho2_screen, doubl
                              int32_t* nbins, int64_t cap, int64_t* n_out) {
   if (!c) return SUB_EINVAL;
   if (!c->ran) { set_err(c, "no run yet"); return SUB_ESTATE; }
-  CU(cudaMemcpyAsync(c->h_rs, c->rs, sizeof(RunState), cudaMemcpyDeviceToHost, c->stream), c);
   CU(cudaStreamSynchronize(c->stream), c);
   const int64_t m = (int64_t)c->h_rs->nlive;
   if (n_out) *n_out = m;

@@ -67,7 +67,7 @@ struct sub_ctx {
   // run state
   RunState* rs = nullptr;
   int* new_hist = nullptr;
-  RunState* h_rs = nullptr;  // pinned copy
+  RunState* h_rs = nullptr;  // page-locked: the state the last run ended with
   bool ran = false;
   // graph
   cudaGraphExec_t exec = nullptr;

@@ -3290,7 +3290,7 @@ void launch_begin(unsigned long long* acc, long long nb, AccReplicas rep, unsign
 
 __global__ void k_control(RunState* rs, int max_iter, double rtol, int* new_hist,
                           unsigned long long cond_handle, int use_cond, unsigned char* dirty,
-                          int nch, int* lists, int* counts) {
+                          int nch, int* lists, int* counts, RunState* host) {
   chain_wait();
   // every thread reads the count before thread 0 advances it (after the barriers below)
   const int it0 = rs->iter;
@@ -3336,7 +3336,10 @@ __global__ void k_control(RunState* rs, int max_iter, double rtol, int* new_hist
   }
   rs->count_new = 0ull;
   rs->relchg_bits = 0ull;
-  if (!go) rs->stopped = 1;
+  if (!go) {
+    rs->stopped = 1;
+    *host = *rs;
+  }
   if (go && dirty)  // the lists just built go to the next iteration's kernels
     for (int i = 0; i < kNumLists; ++i) rs->work[i] = work[i] + (unsigned long long)counts[i];
   if (use_cond) cudaGraphSetConditional((cudaGraphConditionalHandle)cond_handle, go);
@@ -3344,9 +3347,9 @@ __global__ void k_control(RunState* rs, int max_iter, double rtol, int* new_hist
 
 void launch_control(RunState* rs, int max_iter, double rtol, int* new_hist,
                     unsigned long long cond_handle, int use_cond, unsigned char* dirty, int nch,
-                    int* lists, int* counts, cudaStream_t st) {
+                    int* lists, int* counts, RunState* host, cudaStream_t st) {
   launch_after(k_control, 1, 1024, 0, st, rs, max_iter, rtol, new_hist, cond_handle, use_cond, dirty,
-               nch, lists, counts);
+               nch, lists, counts, host);
 }
 
 void plan_grids(SmoothPlan& pl) {

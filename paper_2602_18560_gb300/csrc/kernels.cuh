@@ -351,9 +351,11 @@ void launch_begin(unsigned long long* acc, long long nb, AccReplicas rep, unsign
                   int* new_hist, int max_iter, RunState* rs, int nsm, cudaStream_t st);
 
 // Loop control; it also clears the dirty set the finished iteration read and builds the
-// work lists of the next one.
+// work lists of the next one.  The state the run ends with goes to *host as well (page-locked
+// memory), where the host finds it once the stream is done: a copy after the run was one more
+// operation and wait for each of a batch's contexts and a server's jobs.
 void launch_control(RunState* rs, int max_iter, double rtol, int* new_hist,
                     unsigned long long cond_handle, int use_cond, unsigned char* dirty, int nch,
-                    int* lists, int* counts, cudaStream_t st);
+                    int* lists, int* counts, RunState* host, cudaStream_t st);
 
 }  // namespace gbsub
