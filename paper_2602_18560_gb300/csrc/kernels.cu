@@ -34,9 +34,14 @@ namespace gbsub {
 // ============================================================================ tables
 
 // Programmatic dependent launch along a chain of kernels: a kernel launched by launch_after may
-// be set up while the one before it still runs, and waits (chain_wait, its first statement, in
-// every thread) until that one has ended and its writes can be seen.  As every kernel of a chain
-// waits, the end of one is the end of all before it.  What such a kernel reads of its
+// be set up while the one before it still runs, and waits (chain_wait, in every thread of every
+// path) until that one has ended and its writes can be seen.  As every kernel of a chain
+// waits, the end of one is the end of all before it.  Before the wait a kernel only reads what
+// was there when the chain began: the catalog, and in the loop the iteration's work lists, the
+// candidates and the counts, which the previous iteration's control kernel (not of the chain)
+// came after.  That takes a trip or two to memory per kernel off a late iteration (3e7 sources
+// 1206 -> 1175 us, 1 yr, 1e4 sources 175 -> 169).
+// What such a kernel reads of its
 // predecessors' output goes through plain pointers: the compiler may move loads through
 // const __restrict__ parameters above the wait.
 // chain_next lets the next kernel's CTAs in once every CTA of this one has called it or ended.
@@ -880,7 +885,6 @@ __device__ __forceinline__ bool mbar_wait_abort(uint64_t* bar, unsigned parity,
 
 __global__ void __launch_bounds__(kPrepassThreads, 1)
     k_prepass(const __grid_constant__ PrepassArgs pa) {
-  chain_wait();
   RunState* const rs = pa.rs;
   // per warp [stage][A | f | fdot][kPreStep]; the warps' queues; the hot bins' words
   extern __shared__ __align__(128) double pre_smem[];
@@ -899,7 +903,10 @@ __global__ void __launch_bounds__(kPrepassThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  if (scat.staged == kCatGenerated) return;  // k_prepass_gen's catalog
+  if (scat.staged == kCatGenerated) {  // k_prepass_gen's catalog
+    chain_wait();
+    return;
+  }
   const long long N = scat.n;
   double* const stages = pre_smem + (size_t)warp * kPreStages * 3 * kPreStep;
   SlowQueue myq = {};
@@ -944,6 +951,7 @@ __global__ void __launch_bounds__(kPrepassThreads, 1)
   start_copies(u, 0);
   unsigned u1 = take_step();
   start_copies(u1, 1);
+  chain_wait();  // the words are zero now
   unsigned nkappa = 0;  // a lane's share of the catalog
   // a source's replica is its index mod kAccReplicas, the same for all of a lane's sources
   u64* const rep_lane = pa.rep.w + 2 * (size_t)(lane % kAccReplicas) * pa.rep.nbins;
@@ -1052,12 +1060,12 @@ struct GenQueues {
 
 __global__ void __launch_bounds__(kGenThreads, 4)
     k_prepass_gen(const __grid_constant__ PrepassArgs pa) {
-  chain_wait();
   RunState* const rs = pa.rs;
   __shared__ CatalogRef scat;
   __shared__ GenQueues queues[kGenThreads / 32];
   if (threadIdx.x == 0) scat = *pa.cat;
   __syncthreads();
+  chain_wait();
   if (scat.staged != kCatGenerated) return;
   const long long N = scat.n;
   const GenParams& gen = scat.gen;
@@ -2272,12 +2280,12 @@ template <typename K>
 __global__ void __launch_bounds__(512, 2) k_median_wm(
     const K* skey, const uint16_t* srank, long long n, SmoothPlan pl,
     const __grid_constant__ SgOut o, const __grid_constant__ Dirty d) {
-  chain_wait();
   extern __shared__ __align__(16) unsigned char sm_raw[];
   __shared__ int zeros[16];
   double relmax = 0.0;
   const ListHead head =
       list_head(d, kListTile, pl.nch + 1, o.tree.h ? &o.rs->tree_live : nullptr);
+  chain_wait();
   const int nitem = head.count;
   if (nitem <= (int)gridDim.x) chain_next();
   int u_next = head.first;
@@ -2513,10 +2521,10 @@ __global__ void __launch_bounds__(1024)
   __shared__ U128 warp_tot[32];
   __shared__ u64 warp_max[32];
   __shared__ int any_uf;
-  chain_wait();
   // chunks whose input changed (a chunk within in_radius of them is dirty)
   const int list = kListR0 + in_radius;
   const ListHead head = list_head(d, list, pl.nch, in.flags);
+  chain_wait();
   const int nitem = head.count;
   if (nitem <= (int)gridDim.x) chain_next();
   const bool pairs = (reinterpret_cast<uintptr_t>(in.x) & 15u) == 0;
@@ -2579,7 +2587,6 @@ k_window_mean(const double* x, long long n, SmoothPlan pl, const unsigned long l
                               const unsigned long long* pre_hi, const int* sig,
                               const unsigned* uflow, const __grid_constant__ SgOut o,
                               const __grid_constant__ Dirty d, int out_radius) {
-  chain_wait();
   double relmax = 0.0;
   const int h = pl.W / 2;
   const double inv_w = 1.0 / (double)pl.W;
@@ -2588,6 +2595,7 @@ k_window_mean(const double* x, long long n, SmoothPlan pl, const unsigned long l
   const int parts = (pl.Kc + blockDim.x - 1) / blockDim.x;
   const ListHead head =
       list_head(d, list, pl.nch, kTree ? &o.rs->tree_live : nullptr, parts);
+  chain_wait();
   const int nitem = head.count * parts;
   if (nitem <= (int)gridDim.x) chain_next();
   long long b_next = head.first;
@@ -2980,19 +2988,16 @@ __global__ void __launch_bounds__(256) k_snr_resolve(
     const __grid_constant__ Cands cd, const __grid_constant__ Grid g, const __grid_constant__ Tables tb, const double* Sg, const float* inv_f,
     double th2, double rtol, int mode, unsigned char* __restrict__ resolved,
     unsigned long long* __restrict__ acc, RunState* rs, Dirty d, int Kc, int sg_radius) {
-  chain_wait();
-  chain_next();
   // the loop state, read by one thread per CTA (every thread of the grid loading the same
   // words would queue on one L2 line)
   __shared__ long long snr_head[4];  // stop, iteration, live candidates, long sweeps
   if (threadIdx.x == 0) {
-    snr_head[0] = (rs->final_pass || rtol_stop(rs, rtol)) ? 1 : 0;
+    snr_head[0] = rs->final_pass ? 1 : 0;
     snr_head[1] = rs->iter;
     snr_head[2] = (long long)rs->nlive;
     snr_head[3] = (long long)rs->nwide;
   }
   __syncthreads();
-  if (snr_head[0]) return;
   const long long nlive = snr_head[2];
   const DirtyIter di(d, (int)snr_head[1]);
   const int lane = threadIdx.x & 31;
@@ -3003,19 +3008,18 @@ __global__ void __launch_bounds__(256) k_snr_resolve(
   // sit together in the list (the catalog pass emits the long sweeps of its FP64 path in
   // runs) are spread over many warps
   const long long ngroups = (nlive + 31) / 32;
-  for (long long grp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; grp < ngroups;
-       grp += nwarps) {
-    bool todo = false;
-    const long long c = grp + (long long)lane * ngroups;
-    int4 pk = make_int4(0, 0, 0, 0);
+  // the lane's candidate of a group is unresolved, a short sweep, and S_gal changed on it
+  auto wanted = [&](long long c, int4* pk) {
+    *pk = make_int4(0, 0, 0, 0);
     unsigned char done = 1;
     if (c < nlive) {  // both loads at once
       done = cd.res[c];
-      pk = cd.pk[c];
+      *pk = cd.pk[c];
     }
-    if (!done && pk.y <= kSnrLaneBins) {  // the long sweeps are taken below
-      const int ka = pk.x;
-      const int nbin = pk.y;
+    bool todo = false;
+    if (!done && pk->y <= kSnrLaneBins) {  // the long sweeps are taken below
+      const int ka = pk->x;
+      const int nbin = pk->y;
       long long c0 = ka < 0 ? 0 : ka / Kc;
       long long kl = (long long)ka + nbin - 1;
       if (kl > g.nb - 1) kl = g.nb - 1;
@@ -3024,6 +3028,22 @@ __global__ void __launch_bounds__(256) k_snr_resolve(
         for (long long cc = c0; cc <= c1 && !todo; ++cc) todo = di.any(cc, sg_radius);
       }
     }
+    return todo;
+  };
+  // the warp's first group, while the estimate still runs
+  long long grp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  int4 pk = make_int4(0, 0, 0, 0);
+  bool todo = false;
+  if (grp < ngroups) todo = wanted(grp + (long long)lane * ngroups, &pk);
+  chain_wait();
+  chain_next();
+  if (rtol > 0.0) {
+    if (threadIdx.x == 0 && rtol_stop(rs, rtol)) snr_head[0] = 1;
+    __syncthreads();
+  }
+  if (snr_head[0]) return;
+  for (; grp < ngroups;) {
+    const long long c = grp + (long long)lane * ngroups;
     if (todo) {
       int kcount;
       const float r2 = screen_part(cd, c, pk, g, tb, inv_f, 0, 1, kcount);
@@ -3042,6 +3062,8 @@ __global__ void __launch_bounds__(256) k_snr_resolve(
         remove_part(cd, c, g, tb, acc, di, Kc, 0, 1);
       }
     }
+    grp += nwarps;
+    if (grp < ngroups) todo = wanted(grp + (long long)lane * ngroups, &pk);
   }
   // the long sweeps, one per warp at a time; the very long ones that the screen leaves open are
   // set aside for the whole CTA (the few that find no room are decided by their warp)
@@ -3291,9 +3313,9 @@ void launch_begin(unsigned long long* acc, long long nb, AccReplicas rep, unsign
 __global__ void k_control(RunState* rs, int max_iter, double rtol, int* new_hist,
                           unsigned long long cond_handle, int use_cond, unsigned char* dirty,
                           int nch, int* lists, int* counts, RunState* host) {
-  chain_wait();
   // every thread reads the count before thread 0 advances it (after the barriers below)
   const int it0 = rs->iter;
+  chain_wait();
   // thread 0 loads the rest of the loop state now, so that its latency overlaps the lists
   int final_pass = 0;
   unsigned err = 0u;
