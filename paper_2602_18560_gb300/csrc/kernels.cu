@@ -31,8 +31,7 @@
 
 namespace gbsub {
 
-// ============================================================================ tables
-
+// ============================================================================ launches
 // Programmatic dependent launch along a chain of kernels: a kernel launched by launch_after may
 // be set up while the one before it still runs, and waits (chain_wait, in every thread of every
 // path) until that one has ended and its writes can be seen.  As every kernel of a chain
@@ -40,10 +39,9 @@ namespace gbsub {
 // was there when the chain began: the catalog, and in the loop the iteration's work lists, the
 // candidates and the counts, which the previous iteration's control kernel (not of the chain)
 // came after.  That takes a trip or two to memory per kernel off a late iteration (3e7 sources
-// 1206 -> 1175 us, 1 yr, 1e4 sources 175 -> 169).
-// What such a kernel reads of its
-// predecessors' output goes through plain pointers: the compiler may move loads through
-// const __restrict__ parameters above the wait.
+// 1206 -> 1175 us, 1 yr, 1e4 sources 175 -> 169).  What it reads of its predecessors' output
+// goes through plain pointers: the compiler may move loads through const __restrict__ parameters
+// above the wait.
 // chain_next lets the next kernel's CTAs in once every CTA of this one has called it or ended.
 // A kernel calls it at once when no CTA has more than one item of work, which hides the next
 // launch behind it (a run over 3e7 sources 1257 -> 1232 us, over 1e7 with the mean 481 -> 473).
@@ -71,6 +69,8 @@ static void launch_after(void (*kern)(P...), int bl, int th, size_t smem, cudaSt
   cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
+
+// ============================================================================ tables
 
 __global__ void k_tables(Grid g, int tdi2, double* __restrict__ S, double* __restrict__ R,
                          double* __restrict__ gq, float* __restrict__ Gf,
