@@ -768,7 +768,7 @@ def prior_record(args, est, draws=12, T_obs=4 * synth.YEAR):
                         "model drawn on the device" % (draws, ntot),
             "note": "the time of a draw grows with the bins its sources sweep: the Gamma prior of "
                     "log10 fdot puts some sources at fdot > 1e-12 Hz/s, whose sweeps of 1e4 bins "
-                    "and more are deposited by the FP64 path",
+                    "and more are held by nodes over many bins",
             "api": "sub_load_population(fused) + sub_run + sub_coarse_grain(100 bins) -> host",
             "ms_per_simulation": 1e3 * sum(times) / len(times),
             "ms_per_simulation_median": 1e3 * float(np.median(times)),

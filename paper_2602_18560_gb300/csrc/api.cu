@@ -945,8 +945,8 @@ extern "C" int sub_coarse_grain(sub_ctx* c, const double* x, int32_t add_instr, 
     CU(cudaMemcpyAsync(c->estimate_in, x, (size_t)n * 8, cudaMemcpyHostToDevice, st), c);
     in = c->estimate_in;
   }
-  launch_coarse_grain(in, add_instr ? c->S : nullptr, de, nbins, c->grid.k_lo, c->p.T_obs, dS, df,
-                      dc, st);
+  launch_coarse_grain(in, add_instr ? c->S : nullptr, de, nbins, n, c->grid.k_lo, c->p.T_obs, dS,
+                      df, dc, st);
   CU(cudaGetLastError(), c);
   const cudaMemcpyKind k = where == SUB_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
   if (S_out) CU(cudaMemcpyAsync(S_out, dS, (size_t)nbins * 8, k, st), c);

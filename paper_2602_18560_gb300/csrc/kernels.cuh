@@ -295,8 +295,9 @@ void launch_generate(const CatalogRef* ref, long long start, long long n, double
 
 // Coarse graining: for every bin k of [edge[k], edge[k+1]) (nbins + 1 edges on the device),
 // the mean of x (of S + x when S is given), the mean frequency (k_lo + i) / T and the count.
+// n: values in all.
 void launch_coarse_grain(const double* x, const double* S, const long long* edge, int nbins,
-                         long long k_lo, double T, double* S_out, double* f_out,
+                         long long n, long long k_lo, double T, double* S_out, double* f_out,
                          long long* cnt_out, cudaStream_t st);
 
 // P[j] = S_j Q_j 2^-64 for every bin.
