@@ -1847,6 +1847,9 @@ __global__ void __launch_bounds__(1024, E == 2 ? 2 : 1) k_chunk_sort(SpecIn in, 
           posof[i] = (uint16_t)pos;
           c[a] = (keys[pos] & ~low) | (u64)i;
         }
+        // the next sort begins with the buffer that this one's last exchange read (an odd number
+        // of exchanges: 64, 128 and 1024 threads)
+        __syncthreads();
       } else {
         __syncthreads();
 #pragma unroll

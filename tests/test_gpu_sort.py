@@ -44,3 +44,20 @@ def test_values_that_differ_in_the_lowest_bits(W):
                 except gbsub.SubError:
                     continue  # not a width this window allows
                 np.testing.assert_array_equal(s.estimate(P), ref)
+
+
+@pytest.mark.parametrize("W", [100, 200, 500, 1100, 2000])
+def test_passes_of_the_second_order_do_not_overlap(W):
+    # every chunk of a band of many takes the second order (three sorts on the same two exchange
+    # buffers), several CTAs to an SM: 64, 128, 256 and twice 1024 threads, that is 1, 3, 6 and 15
+    # exchanges a sort, odd numbers but for the third
+    L, reps = 8 * W, 40  # L values over and over, so that the oracle does three times as many
+    n = reps * L
+    k_lo = int(np.ceil(1e-4 * T))
+    f_max = (k_lo + n - 1 + 0.25) / T
+    low = spectra(L)[0]
+    r = oracle.smooth(gbsub.MEDIAN, W, np.tile(low, 3))
+    ref = np.concatenate([r[:L], np.tile(r[L:2 * L], reps - 2), r[2 * L:]])
+    with gbsub.Subtraction(T_obs=T, window=W, estimator=gbsub.MEDIAN, f_max=f_max) as s:
+        for _ in range(3):
+            np.testing.assert_array_equal(s.estimate(np.tile(low, reps)), ref)
