@@ -498,10 +498,13 @@ constexpr size_t kPrepassSmem =
 // f T comes from the 53-bit mantissa of f, split in 21 + 32 bits, times T's in 32 + 21: three
 // 32-bit products, exact but for two units of their 2^53 (2^-32 of a bin in the band; the
 // dropped part of T's low bits).  With at most 30 integer bits, the product is shifted to 23
-// fraction bits.  The certificate is FP32: the start's offset from the bin's centre plus
-// du = fdot T^2 (off by less than 4e-7 |du|) must stay 2^-20 inside the cell, which covers the
-// truncation of the fraction and the FP64 rounding of f T in the reference.  A value that is
-// not finite fails it (f: no exponent in range; fdot: du is not a number or too large).
+// fraction bits.  The certificate is FP32: the start's offset from the bin's centre, and that plus
+// du = fdot T^2 (off by less than 4e-7 |du|), must both stay 2^-20 inside the cell, which covers
+// the truncation of the fraction and the FP64 rounding of f T in the reference.  (Both ends: a
+// start on an upper edge that is truncated into the cell below and moves down ends well inside
+// it, and the removal, which goes by the FP64 sweep, would take power from a bin that got none.)
+// A value that is not finite fails it (f: no exponent in range; fdot: du is not a number or too
+// large).
 //
 // T's mantissa is used with its top bit set: with its trailing zeros dropped instead (20 bits
 // left for 4 years) the product kept too few bits for f above 1 mHz, and every such source,
@@ -524,7 +527,7 @@ __device__ __forceinline__ bool source_bin(double fs, double fds, const Grid& g,
   const float fd = da >= (897u << 20) ? __uint_as_float(fb) : 0.0f;
   const float du = __fmul_rn(fd, g.T2f);
   const float edge = __fmaf_rn(-4e-7f, fabsf(du), 0.5f - 9.5367431640625e-7f);
-  return n <= 39u && da < (1151u << 20) && fabsf(__fadd_rn(off, du)) < edge;
+  return n <= 39u && da < (1151u << 20) && fabsf(off) < edge && fabsf(__fadd_rn(off, du)) < edge;
 }
 
 // Arguments of the catalog pass, one block so that the out-of-line parts take one pointer.

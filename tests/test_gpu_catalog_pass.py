@@ -7,7 +7,7 @@ import pytest
 
 import oracle
 from paper_2602_18560_gb300 import gbsub, synth
-from test_gpu_parity import compare_run
+from test_gpu_parity import RTOL, compare_run, rel_err
 
 pytestmark = pytest.mark.gpu
 
@@ -59,3 +59,38 @@ def test_first_bins_in_shared_memory(N):
     f = (k_lo + j + rng.uniform(-0.4, 0.4, N)) / T
     st, _, res, _ = compare_run(A, f, np.zeros(N), T, gbsub.MEDIAN_MEAN, 200, f_max=f_max)
     assert res[j < 4096].sum() > 20 and res[j >= 4096].sum() > 20
+
+
+@pytest.mark.parametrize("T", [synth.YEAR, 1.87654321 * synth.YEAR, 1e8 / 3.0,
+                               np.nextafter(2.0**25, 0.0)])
+@pytest.mark.parametrize("est", [gbsub.MEAN, gbsub.MEDIAN])
+def test_sweeps_down_from_an_edge_are_removed_whole(T, est):
+    # loud sources that start on the upper edge of their bin, or a few doubles beside it, and move
+    # down: FP64 gives the bin above a share of the sweep (none, on the edge), whatever a product
+    # of fewer bits says.  They are resolved, and what is taken away is what was deposited, in
+    # bins that nothing else is in.
+    f_max = 1.5e-3
+    k_lo, n = oracle.grid(T, 1e-4, f_max)
+    rng = np.random.default_rng(12)
+    j = np.arange(20, n - 40, 64)
+    f = (k_lo + j + 0.5) / T
+    ulps = rng.integers(-2, 3, j.size)
+    for step in range(2):
+        f = np.where(ulps > step, np.nextafter(f, np.inf), f)
+        f = np.where(ulps < -step, np.nextafter(f, 0.0), f)
+    fdot = -10 ** rng.uniform(-5.0, np.log10(0.5), j.size) / T**2
+    A = amplitude(T, k_lo, n, j, np.full(j.size, 1e4))
+    jb = np.arange(8, n, 16)  # a faint background beside them
+    jb = jb[(jb - 20) % 64 > 1]
+    A = np.append(A, amplitude(T, k_lo, n, jb, 0.05 * rng.gamma(2.0, size=jb.size)))
+    f, fdot = np.append(f, (k_lo + jb) / T), np.append(fdot, np.zeros(jb.size))
+    _, _, res, _ = compare_run(A, f, fdot, T, est, 101, f_max=f_max)
+    assert res[:j.size].all() and not res[j.size:].any()
+    with gbsub.Subtraction(T_obs=T, window=101, estimator=est, f_max=f_max) as s:
+        s.load(A, f, fdot)
+        s.run()
+        P = s.power()
+    S, R = oracle.tables(T, k_lo, n, True)
+    keep = ~res
+    ref = oracle.power(T, R, oracle.deposit(T, k_lo, n, A[keep], f[keep], fdot[keep]))
+    assert rel_err(P, ref) <= RTOL
