@@ -170,7 +170,10 @@ extern "C" int sub_create(const sub_params* p, void* stream, sub_ctx** out) {
     c->grid.tq = (unsigned)(mT >> 21);
     c->grid.tr = (unsigned)(mT << 11);
     c->grid.ebin = 1020 - (ex - 32);  // T = (tq + tr 2^-32) 2^(ex - 32)
-    if (c->grid.ebin - 39 < 1 || c->grid.ebin > 0x7FE) c->grid.ebin = -(1 << 20);
+    // the FP32 certificate works on 32-bit bin numbers below 2^30: a T_obs too extreme for it, or
+    // a band that begins higher, leaves every source to the FP64 path
+    if (c->grid.ebin - 39 < 1 || c->grid.ebin > 0x7FE || k_lo >= ((int64_t)1 << 30))
+      c->grid.ebin = -(1 << 20);
     c->grid.T2f = (float)(p->T_obs * p->T_obs);
   }
   c->plan = make_plan(p->window, n);

@@ -94,3 +94,22 @@ def test_sweeps_down_from_an_edge_are_removed_whole(T, est):
     keep = ~res
     ref = oracle.power(T, R, oracle.deposit(T, k_lo, n, A[keep], f[keep], fdot[keep]))
     assert rel_err(P, ref) <= RTOL
+
+
+@pytest.mark.parametrize("turns", [1, 2, 5])
+def test_bands_beyond_32_bit_bins(turns):
+    # a band that begins at bin 2^32 turns + 3000: a source of bin 3500 is far below it
+    T = 2.0**33 * turns
+    k0, n = 2**32 * turns + 3000, 2000
+    f_min, f_max = k0 / T, (k0 + n - 1) / T
+    k_lo, nb = oracle.grid(T, f_min, f_max)
+    assert (k_lo, nb) == (k0, n)
+    j = np.append(np.arange(0, n, 3), [700, 701])
+    p = np.append(np.full(j.size - 2, 0.1), [1e4, 1e4])
+    A = amplitude(T, k0, n, j, p)
+    f = (k0 + j + 0.125) / T
+    low = np.array([2900.0, 3500.0, 4000.25, 4999.0])  # bins a 32-bit difference puts in the band
+    A, f = np.append(A, np.full(low.size, 30.0 * A.max())), np.append(f, low / T)
+    for est in (gbsub.MEAN, gbsub.MEDIAN):
+        _, _, res, _ = compare_run(A, f, np.zeros(f.size), T, est, 51, f_max=f_max, f_min=f_min)
+        assert res.sum() == 2 and not res[j.size:].any()
