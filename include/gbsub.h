@@ -298,7 +298,8 @@ int sub_profile(sub_ctx* ctx, float ms[SUB_K_COUNT], int32_t launches[SUB_K_COUN
  *                    of the last estimate, in FP32), summed bin by bin on one thread
  *   rho2_exact[i]  : rho^2 in FP64, summed in the oracle's order (the value SUB_FP64 decides
  *                    on when the screen cannot; for a sweep of more than 4 bins the run sums
- *                    it across a warp, which differs by rounding only)
+ *                    it across a warp, of more than 4096 across a thread block, which
+ *                    differs by the order of the roundings only)
  *   nbins[i]       : bins of the band the screen summed (the error bound of this one-thread
  *                    sum grows with them)
  * All four are host arrays of cap entries; *n_out (may be null) receives the count.  The

@@ -2712,25 +2712,13 @@ __device__ double rho2_exact_warp(const Grid& g, const Tables& tb, const double*
   return __dmul_rn(4.0, acc);
 }
 
-// 1 / x for x > 0 within about 2^-43: the FP32 reciprocal of the mantissa and one FP64 Newton step,
-// two FP64 instructions where a division takes some twenty.
-__device__ __forceinline__ double rcp_newton(double x) {
-  const u64 b = (u64)__double_as_longlong(x);
-  const int e = (int)(b >> 52) & 0x7FF;
-  if (e == 0 || e > 2040) return __drcp_rn(x);
-  const float m = __uint_as_float(0x3F800000u | (unsigned)((b >> 29) & 0x7FFFFFu));
-  const unsigned r = __float_as_uint(__fdividef(1.0f, m));  // in (1/2, 1]
-  const int er = 2046 - e + ((int)(r >> 23) - 127);
-  if (er < 1) return __drcp_rn(x);
-  const double y = __longlong_as_double((i64)(((u64)er << 52) | ((u64)(r & 0x7FFFFFu) << 29)));
-  return __fma_rn(__fma_rn(-x, y, 1.0), y, y);
-}
-
 // rho^2 of a sweep of very many bins by the whole CTA, for a decision that its screen left open:
-// the terms of rho2_exact with the common factors outside the sum and the reciprocals of S_n
-// within 2^-43, so within 1e-12 of it, far inside the near-threshold band.  The value is in every
-// thread.  (One warp with a division per bin took some 30 ms for a sweep of the whole 4-year
-// band, and held the launch: a simulation that met one 9.7 ms on average over three seeds, now 3.0.)
+// the terms of rho2_exact with the common factors outside the sum, which differs from it by the
+// order of the roundings.  The value is in every thread.
+// Bound by the FP64 pipe (a division per bin).  One warp took some 30 ms for a sweep of the whole
+// 4-year band and held the launch; over twelve draws of 1e7 sources from the paper's priors, two
+// of which meet such sweeps, a simulation now takes 2.95 ms on average.  (With reciprocals of
+// 43 bits in place of the divisions it took 3.00, and rho^2 came out 3e-15 too small.)
 __device__ double rho2_cta(const Grid& g, const Tables& tb, const double* __restrict__ Sg,
                            double a2, double lo, double hi) {
   __shared__ double part[32];
@@ -2745,9 +2733,8 @@ __device__ double rho2_cta(const Grid& g, const Tables& tb, const double* __rest
 #pragma unroll 4
   for (long long k = k0 + threadIdx.x; k <= k1; k += blockDim.x) {
     const long long j = k - g.k_lo;
-    const double y = rcp_newton(__dadd_rn(tb.S[j], Sg[j]));
     const bool inner = k > sw.ka && k < sw.kb;
-    acc = __fma_rn(tb.R[j], inner ? y : 0.0, acc);
+    acc = __dadd_rn(acc, inner ? __ddiv_rn(tb.R[j], __dadd_rn(tb.S[j], Sg[j])) : 0.0);
   }
   acc = __dmul_rn(acc, sweep_inv_len(sw));
   if (threadIdx.x < 2) {  // the sweep's first and last cells, with their own weights

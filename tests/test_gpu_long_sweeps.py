@@ -123,3 +123,44 @@ def test_decisions_left_open_by_the_screen(first, length, delta):
         res = s.resolved().astype(bool)
     assert st.n_exact > 0
     assert np.array_equal(res, ref["resolved"])
+
+
+@pytest.mark.parametrize("first, length", [(-20.3, 75_838.7), (3000.2, 5000.4), (70_000.4, -66_000.1)])
+@pytest.mark.parametrize("side", [-1.0, 1.0])
+def test_open_decisions_have_the_precision_of_fp64(first, length, side):
+    # rho_th^2 at 1.5e-15 on either side of the rho^2 that the run's own tables and S_gal give in
+    # more than 64 bits.  A sum of correctly rounded quotients in 256 parts of at most 300 is off by
+    # some 3e-16 (one rounding of the mean of the parts' errors, the last sums and products, and
+    # rho_th^2); quotients of 43 bits, always too small, by 3e-15.
+    k_lo, n = oracle.grid(T, 1e-4, F_MAX)
+    S, R = oracle.tables(T, k_lo, n, True)
+    j = np.arange(n)
+    f = np.append((k_lo + j + 0.1) / T, (k_lo + first) / T)
+    fdot = np.append(np.zeros(n), length / T**2)
+    lo, hi = sorted((first, first + length))
+    A = np.append(np.sqrt(5.0 * 0.1 * S / (T * R)),
+                  10.0 / np.sqrt(0.8 * T * (R / S)[max(0, int(lo)):int(hi)].sum() / (hi - lo)))
+    kw = dict(T_obs=T, estimator=gbsub.MEAN, window=1001, f_max=F_MAX)
+    with gbsub.Subtraction(rho_th=9.99, **kw) as s:  # rho is below rho_0 = 10: not resolved
+        s.load(A, f, fdot)
+        s.run()
+        assert not s.resolved().any()
+        Sg = s.spectrum()
+        S, R = s.tables()
+    # the oracle's sweep and weights, the sum in long doubles
+    u0 = f[-1] * T
+    u1 = u0 + fdot[-1] * (T * T)
+    lo, hi = min(u0, u1), max(u0, u1)
+    k = np.arange(max(k_lo, int(np.floor(lo + 0.5))),
+                  min(k_lo + n - 1, int(np.floor(hi + 0.5))) + 1)
+    w = ((np.minimum(hi, k + 0.5) - np.maximum(lo, k - 0.5)) / (hi - lo)).clip(0.0)
+    X = np.longdouble
+    terms = R[k - k_lo].astype(X) * w.astype(X) / (S[k - k_lo] + Sg[k - k_lo]).astype(X)
+    rho2 = X(4.0) * X(T / 5.0) * X(A[-1]) * X(A[-1]) * terms.sum()
+    rho_th = float(np.sqrt(rho2 * (X(1.0) + X(side * 1.5e-15))))
+    with gbsub.Subtraction(rho_th=rho_th, **kw) as s:
+        s.load(A, f, fdot)
+        st = s.run()
+        res = s.resolved().astype(bool)
+    assert st.n_exact > 0 and st.n_near > 0
+    assert res[-1] == (side < 0) and not res[:-1].any()
