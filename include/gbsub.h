@@ -294,14 +294,18 @@ int sub_profile(sub_ctx* ctx, float ms[SUB_K_COUNT], int32_t launches[SUB_K_COUN
  * candidate (rho_0 > rho_th, see sub_stats.n_live) against the S_gal of the last run, for
  * measuring the FP32 screen that SUB_FP64 decides on first:
  *   src[i]         : the candidate's index in the catalog
- *   rho2_screen[i] : rho^2 in FP32 as the screen evaluates it (through 1 / (1 + S_gal/S_instr)
- *                    of the last estimate, in FP32), summed bin by bin on one thread
+ *   rho2_screen[i] : rho^2 in FP32 as the run's screen evaluates it (through 1 / (1 +
+ *                    S_gal/S_instr) of the last estimate, in FP32): bin by bin for a sweep of
+ *                    at most 4 bins, across a warp for a longer one, from the sums over nodes
+ *                    of 32, 1024 and 32768 bins for one of more than 512
  *   rho2_exact[i]  : rho^2 in FP64, summed in the oracle's order (the value SUB_FP64 decides
  *                    on when the screen cannot; for a sweep of more than 4 bins the run sums
  *                    it across a warp, of more than 4096 across a thread block, which
  *                    differs by the order of the roundings only)
- *   nbins[i]       : bins of the band the screen summed (the error bound of this one-thread
- *                    sum grows with them)
+ *   nbins[i]       : bins of the band in the sweep.  A term of the screen's sum passes through at
+ *                    most nbins roundings (an error of 2.2e-6 + 2e-7 for each of them); a warp's
+ *                    through nbins / 32 + 5, a sum over nodes through 26 and one for every 2^20
+ *                    bins of the band
  * All four are host arrays of cap entries; *n_out (may be null) receives the count.  The
  * call allocates and frees a temporary device buffer of 24 bytes per candidate and
  * synchronises.  Errors: SUB_EINVAL (cap below the count, null output), SUB_ESTATE (no run

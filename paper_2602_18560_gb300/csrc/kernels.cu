@@ -2858,6 +2858,27 @@ __device__ __forceinline__ bool screen_tree(const Cands& cd, long long c, const 
   return true;
 }
 
+// The FP32 value of a sweep of more than kSnrLaneBins bins by a whole warp, the same in every
+// lane: true when it came from the tree.  kcount: the roundings that a term passes through.
+__device__ __forceinline__ bool screen_wide(const Cands& cd, long long c, const int4 pk,
+                                            const Grid& g, const Tables& tb,
+                                            const float* __restrict__ inv_f, float* r2out,
+                                            int* kcount) {
+  if (screen_tree(cd, c, pk, g, tb, inv_f, r2out, kcount)) return true;
+  // butterfly sums.  The sum's longest sequential chain is the largest lane count, and the
+  // butterfly adds five roundings: the screen's bound takes that many terms, not every bin of
+  // the sweep
+  int kchain;
+  float r2 = screen_part(cd, c, pk, g, tb, inv_f, threadIdx.x & 31, 32, kchain);
+  for (int o = 16; o > 0; o >>= 1) {
+    r2 = __fadd_rn(r2, __shfl_xor_sync(0xFFFFFFFFu, r2, o));
+    kchain = max(kchain, __shfl_xor_sync(0xFFFFFFFFu, kchain, o));
+  }
+  *r2out = r2;
+  *kcount = kchain + 5;
+  return false;
+}
+
 // Decision from the FP32 value: 1 resolve, 0 keep, -1 too close to rho_th to tell (the
 // caller then computes rho^2 exactly).
 __device__ __forceinline__ int screen_decide(float r2, int kcount, float th2f, int mode) {
@@ -3092,31 +3113,18 @@ __global__ void __launch_bounds__(256) k_snr_resolve(
     if (!__any_sync(0xFFFFFFFFu, t)) continue;
     int kcount;
     float r2;
-    if (screen_tree(cd, cw, pkw, g, tb, inv_f, &r2, &kcount)) {
-      if (mode == 0 && pkw.y > kOpenBins && screen_decide(r2, kcount, th2f, mode) < 0) {
-        int at = 0;
-        if (lane == 0) at = atomicAdd(&open_n, 1);
-        at = __shfl_sync(0xFFFFFFFFu, at, 0);
-        if (at < kOpenMax) {
-          if (lane == 0) open_c[at] = cw;
-          continue;
-        }
+    if (screen_wide(cd, cw, pkw, g, tb, inv_f, &r2, &kcount) && mode == 0 && pkw.y > kOpenBins &&
+        screen_decide(r2, kcount, th2f, mode) < 0) {
+      int at = 0;
+      if (lane == 0) at = atomicAdd(&open_n, 1);
+      at = __shfl_sync(0xFFFFFFFFu, at, 0);
+      if (at < kOpenMax) {
+        if (lane == 0) open_c[at] = cw;
+        continue;
       }
-      snr_wide_decide(cd, cw, g, tb, Sg, th2, th2f, mode, r2, kcount, resolved, acc, di, Kc,
-                      local_new, local_exact, local_near, local_unc);
-    } else {
-      r2 = screen_part(cd, cw, pkw, g, tb, inv_f, lane, 32, kcount);
-      // butterfly sums: every lane ends with the same values.  The sum's longest sequential
-      // chain is the largest lane count, and the butterfly adds five roundings: the screen's
-      // bound takes that many terms, not every bin of the sweep
-      int kchain = kcount;
-      for (int o = 16; o > 0; o >>= 1) {
-        r2 = __fadd_rn(r2, __shfl_xor_sync(0xFFFFFFFFu, r2, o));
-        kchain = max(kchain, __shfl_xor_sync(0xFFFFFFFFu, kchain, o));
-      }
-      snr_wide_decide(cd, cw, g, tb, Sg, th2, th2f, mode, r2, kchain + 5, resolved, acc, di, Kc,
-                      local_new, local_exact, local_near, local_unc);
     }
+    snr_wide_decide(cd, cw, g, tb, Sg, th2, th2f, mode, r2, kcount, resolved, acc, di, Kc,
+                    local_new, local_exact, local_near, local_unc);
   }
   __syncthreads();
   for (int i = 0; i < min(open_n, kOpenMax); ++i) {
@@ -3150,8 +3158,9 @@ __global__ void __launch_bounds__(256) k_snr_resolve(
 }
 
 // Both evaluations of rho^2 for every kept candidate against the current S_gal: the FP32
-// screen (what the loop decides on first) and the FP64 value in the oracle's order of
-// summation, with the bins the screen summed.  A measurement of the screen's error.
+// screen as the loop evaluates it (a short sweep on one lane, a longer one by the warp) and the
+// FP64 value in the oracle's order of summation, with the bins of the band in the sweep.  A
+// measurement of the screen's error.
 __global__ void __launch_bounds__(256) k_snr_check(Cands cd, Grid g, Tables tb,
                                                    const double* __restrict__ Sg,
                                                    const float* __restrict__ inv_f,
@@ -3159,25 +3168,46 @@ __global__ void __launch_bounds__(256) k_snr_check(Cands cd, Grid g, Tables tb,
                                                    long long* __restrict__ src,
                                                    float* __restrict__ screen,
                                                    double* __restrict__ exact,
-                                                   int* __restrict__ kcount_out) {
+                                                   int* __restrict__ nbins) {
   const long long nlive = (long long)rs->nlive;
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < nlive;
-       c += (long long)gridDim.x * blockDim.x) {
-    const int4 pk = cd.pk[c];
-    int kcount = 0;
-    screen[c] = screen_part(cd, c, pk, g, tb, inv_f, 0, 1, kcount);
-    exact[c] = rho2_exact(g, tb, Sg, cd.a2[c], cd.lo[c], cd.hi[c]);
-    src[c] = cd.src[c];
-    kcount_out[c] = kcount;
+  const int lane = threadIdx.x & 31;
+  for (long long c0 = ((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5) << 5; c0 < nlive;
+       c0 += (long long)gridDim.x * blockDim.x) {
+    const long long c = c0 + lane;
+    const bool valid = c < nlive;
+    int4 pk = make_int4(0, 0, 0, 0);
+    if (valid) pk = cd.pk[c];
+    const bool wide = valid && pk.y > kSnrLaneBins;
+    int count = 0, chain;
+    float r2 = 0.0f;
+    if (valid && !wide) r2 = screen_part(cd, c, pk, g, tb, inv_f, 0, 1, count);
+    for (unsigned m = __ballot_sync(0xFFFFFFFFu, wide); m; m &= m - 1) {
+      const int l = __ffs(m) - 1;
+      const int4 pl = make_int4(__shfl_sync(0xFFFFFFFFu, pk.x, l), __shfl_sync(0xFFFFFFFFu, pk.y, l),
+                                __shfl_sync(0xFFFFFFFFu, pk.z, l), __shfl_sync(0xFFFFFFFFu, pk.w, l));
+      float v;
+      screen_wide(cd, c0 + l, pl, g, tb, inv_f, &v, &chain);
+      if (lane == l) {
+        const long long a = pl.x < 0 ? 0 : pl.x, b = min((long long)pl.x + pl.y, g.nb);
+        r2 = v;
+        count = b > a ? (int)(b - a) : 0;
+      }
+    }
+    if (valid) {
+      screen[c] = r2;
+      exact[c] = rho2_exact(g, tb, Sg, cd.a2[c], cd.lo[c], cd.hi[c]);
+      src[c] = cd.src[c];
+      nbins[c] = count;
+    }
   }
 }
 
 void launch_snr_check(Cands cd, long long ncap, const Grid& g, const Tables& tb, const double* Sg,
                       const float* inv_f, const RunState* rs, long long* src, float* screen,
-                      double* exact, int* kcount, cudaStream_t st) {
+                      double* exact, int* nbins, cudaStream_t st) {
   long long want = (ncap + 255) / 256;
   int bl = (int)(want < 4096 ? (want < 1 ? 1 : want) : 4096);
-  k_snr_check<<<bl, 256, 0, st>>>(cd, g, tb, Sg, inv_f, rs, src, screen, exact, kcount);
+  k_snr_check<<<bl, 256, 0, st>>>(cd, g, tb, Sg, inv_f, rs, src, screen, exact, nbins);
 }
 
 void launch_snr_resolve(Cands cd, long long ncap, const Grid& g, const Tables& tb,

@@ -340,11 +340,11 @@ void launch_snr_resolve(Cands cd, long long ncap, const Grid& g, const Tables& t
                         Dirty d, int Kc, int sg_radius, int nsm, cudaStream_t st);
 
 // For each kept candidate c < rs->nlive (ncap: capacity): its catalog index, its rho^2 as the
-// FP32 screen evaluates it against the current S_gal (through inv_f) with the count of bins
-// summed, and its rho^2 in FP64 in the oracle's order of summation.
+// FP32 screen evaluates it against the current S_gal (through inv_f) with the count of the
+// sweep's bins in the band, and its rho^2 in FP64 in the oracle's order of summation.
 void launch_snr_check(Cands cd, long long ncap, const Grid& g, const Tables& tb, const double* Sg,
                       const float* inv_f, const RunState* rs, long long* src, float* screen,
-                      double* exact, int* kcount, cudaStream_t st);
+                      double* exact, int* nbins, cudaStream_t st);
 
 // The state a run begins with (nb bins, a mask of cap sources in a buffer of whole 16 bytes).
 void launch_begin(unsigned long long* acc, long long nb, AccReplicas rep, unsigned char* resolved,

@@ -164,3 +164,44 @@ def test_open_decisions_have_the_precision_of_fp64(first, length, side):
         res = s.resolved().astype(bool)
     assert st.n_exact > 0 and st.n_near > 0
     assert res[-1] == (side < 0) and not res[:-1].any()
+
+
+@pytest.mark.parametrize("precision", [gbsub.FP64, gbsub.MIXED])
+def test_the_check_measures_the_screen_that_decides(precision):
+    # sweeps of 4 to 240 000 bins about the threshold (rho from 6.9999 to 7.0001 on the first
+    # estimate).  The check's FP32 value is the one the run decides on, within the bound of its own
+    # roundings of the FP64 one: a lane's chain and five levels for a sweep summed by a warp, 26
+    # (and one for every 32 nodes of the highest level) for one of more than 512 bins
+    f_max = 2e-3
+    k_lo, n = oracle.grid(T, 1e-4, f_max)
+    S, R = oracle.tables(T, k_lo, n, True)
+    rng = np.random.default_rng(3)
+    ln = np.append(10 ** rng.uniform(0.6, 5.2, 300), [n + 50.0, n - 3.0])
+    first = np.append(rng.uniform(0, 1, 300) * np.maximum(n - ln[:300] - 2, 1.0), [-20.0, 1.2])
+    A = np.empty(ln.size)
+    for i in range(ln.size):
+        lo, hi = max(0, int(first[i])), min(n, int(first[i] + ln[i]) + 1)
+        A[i] = 1e-3 / np.sqrt(0.8 * T * (R / S)[lo:hi].sum() / ln[i])
+    j = np.arange(n)
+    bg = np.sqrt(5.0 * 0.3 * rng.gamma(2.0, size=n) * S / (T * R))
+    f = np.append((k_lo + first) / T, (k_lo + j + 0.1) / T)
+    fdot = np.append(ln / T**2, np.zeros(n))
+    kw = dict(T_obs=T, estimator=gbsub.MEAN, window=400, f_max=f_max)
+    m = ln.size
+    for _ in range(4):
+        P = oracle.power(T, R, oracle.deposit(T, k_lo, n, np.append(A, bg), f, fdot))
+        rho2 = oracle.snr2(T, k_lo, n, S, R, oracle.smooth(gbsub.MEAN, 400, P), A, f[:m], fdot[:m])
+        A *= 7.0 * (1.0 + rng.uniform(-1e-5, 1e-5, m)) / np.sqrt(rho2)
+    with gbsub.Subtraction(precision=precision, **kw) as s:
+        s.load(np.append(A, bg), f, fdot)
+        s.run()
+        chk, res = s.snr_check(), s.resolved().astype(bool)
+    src = chk["src"]
+    assert src.size >= m // 2
+    ex, sc, nb = chk["exact"], chk["screen"].astype(np.float64), chk["nbins"]
+    steps = np.where(nb > 512, 26 + (n >> 15) // 32,
+                     np.where(nb > 4, np.ceil(nb / 32.0) + 5, nb))
+    assert np.all(np.abs(sc / ex - 1.0) <= 2.2e-6 + 2e-7 * steps)
+    assert res[:m].any() and not res[:m].all()  # (a removal lifts the others over the threshold)
+    if precision == gbsub.MIXED:
+        assert np.all(sc[~res[src]] <= np.float64(np.float32(49.0)))
