@@ -3325,7 +3325,7 @@ __device__ void build_lists_cta(const unsigned char* __restrict__ cur, int nch,
 // seven clears and a one-CTA list kernel the launches made it 12-18 us more of every run (1 yr, 1e4
 // sources 187 -> 173 us; 24 served requests 4.03 -> 3.69 ms).
 __global__ void __launch_bounds__(256) k_begin(ulonglong2* acc, long long n_acc, ulonglong2* rep,
-                                               long long n_rep, ulonglong2* resolved,
+                                               long long n_rep, unsigned char* resolved,
                                                long long n_resolved, unsigned char* dirty, int nch,
                                                int* lists, int* counts, int* new_hist,
                                                int max_iter, RunState* rs) {
@@ -3335,7 +3335,9 @@ __global__ void __launch_bounds__(256) k_begin(ulonglong2* acc, long long n_acc,
   const ulonglong2 z = make_ulonglong2(0ull, 0ull);
   for (long long i = t0; i < n_acc; i += step) acc[i] = z;
   for (long long i = t0; i < n_rep; i += step) rep[i] = z;
-  for (long long i = t0; i < n_resolved; i += step) resolved[i] = z;
+  const long long whole = n_resolved / 16;
+  for (long long i = t0; i < whole; i += step) reinterpret_cast<ulonglong2*>(resolved)[i] = z;
+  for (long long i = 16 * whole + t0; i < n_resolved; i += step) resolved[i] = 0;
   for (long long i = t0; i < max_iter; i += step) new_hist[i] = 0;
   for (long long i = t0; i <= nch; i += step) {
     if (i < nch) {
@@ -3360,12 +3362,11 @@ void launch_begin(unsigned long long* acc, long long nb, AccReplicas rep, unsign
                   long long cap, unsigned char* dirty, int nch, int* lists, int* counts,
                   int* new_hist, int max_iter, RunState* rs, int nsm, cudaStream_t st) {
   const long long n_acc = nb * 2, n_rep = (long long)kAccReplicas * rep.nbins;
-  const long long n_res = (cap + 15) / 16;  // the mask's allocation is a multiple of 256 bytes
-  const long long most = n_acc > n_res ? n_acc : n_res;
+  const long long most = n_acc > cap / 16 ? n_acc : cap / 16;
   const long long want = (most + 255) / 256, lim = (long long)nsm * 8;
   k_begin<<<(unsigned)(want < lim ? want : lim), 256, 0, st>>>(
-      (ulonglong2*)acc, n_acc, (ulonglong2*)rep.w, n_rep, (ulonglong2*)resolved, n_res, dirty, nch,
-      lists, counts, new_hist, max_iter, rs);
+      (ulonglong2*)acc, n_acc, (ulonglong2*)rep.w, n_rep, resolved, cap, dirty, nch, lists, counts,
+      new_hist, max_iter, rs);
 }
 
 __global__ void k_control(RunState* rs, int max_iter, double rtol, int* new_hist,

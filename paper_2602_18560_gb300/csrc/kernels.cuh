@@ -346,7 +346,7 @@ void launch_snr_check(Cands cd, long long ncap, const Grid& g, const Tables& tb,
                       const float* inv_f, const RunState* rs, long long* src, float* screen,
                       double* exact, int* nbins, cudaStream_t st);
 
-// The state a run begins with (nb bins, a mask of cap sources in a buffer of whole 16 bytes).
+// The state a run begins with (nb bins, a mask of cap sources that begins on 16 bytes).
 void launch_begin(unsigned long long* acc, long long nb, AccReplicas rep, unsigned char* resolved,
                   long long cap, unsigned char* dirty, int nch, int* lists, int* counts,
                   int* new_hist, int max_iter, RunState* rs, int nsm, cudaStream_t st);

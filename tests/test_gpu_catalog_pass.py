@@ -113,3 +113,17 @@ def test_bands_beyond_32_bit_bins(turns):
     for est in (gbsub.MEAN, gbsub.MEDIAN):
         _, _, res, _ = compare_run(A, f, np.zeros(f.size), T, est, 51, f_max=f_max, f_min=f_min)
         assert res.sum() == 2 and not res[j.size:].any()
+
+
+@pytest.mark.parametrize("N", [1, 15, 16, 17, 47])
+def test_the_mask_is_cleared_to_its_last_byte(N):
+    # one context: every source resolved, then none, in a mask that does not end on 16 bytes
+    T = synth.YEAR
+    k_lo, n = oracle.grid(T, 1e-4, 1e-3)
+    j = 100 + 200 * np.arange(N)
+    f = (k_lo + j) / T
+    with gbsub.Subtraction(T_obs=T, window=101, estimator=gbsub.MEDIAN, f_max=1e-3) as s:
+        for p, want in ((1e4, 1), (1e-2, 0), (1e4, 1), (1e-2, 0)):
+            s.load(amplitude(T, k_lo, n, j, p), f, np.zeros(N))
+            s.run()
+            assert np.array_equal(s.resolved(), np.full(N, want, np.uint8))
