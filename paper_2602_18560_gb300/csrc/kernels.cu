@@ -854,10 +854,6 @@ __device__ __forceinline__ void deposit_source(const PlacedSource p, SourceParts
   }
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
-}
-
 __device__ __forceinline__ bool mbar_try(uint32_t bar, unsigned parity) {
   uint32_t ok;
   asm volatile(

@@ -150,22 +150,6 @@ struct Dirty {
   const RunState* rs;
   const int* lists;   // [kNumLists][nch + 1], null when base is null
   const int* counts;  // [kNumLists]
-  __device__ __forceinline__ bool any(long long c, int radius) const {
-    return any_between(c - radius, c + radius);
-  }
-  // any chunk of [a, b] (clipped to the chunks that exist)
-  __device__ __forceinline__ bool any_between(long long a, long long b) const {
-    if (!base) return true;
-    const unsigned char* cur = base + (size_t)(rs->iter & 1) * nch;
-    if (a < 0) a = 0;
-    if (b > nch - 1) b = nch - 1;
-    for (long long i = a; i <= b; ++i)
-      if (cur[i]) return true;
-    return false;
-  }
-  __device__ __forceinline__ void mark_next(long long c) const {
-    if (base) base[(size_t)((rs->iter + 1) & 1) * nch + c] = 1;
-  }
   // items of work list `which` (all `all` of them when nothing is tracked)
   __device__ __forceinline__ int count(int which, int all) const {
     return lists ? counts[which] : all;
