@@ -8,13 +8,13 @@
 //              into an exact fixed-point spectrum, rho_0 against S_instr, the paper's
 //              candidates (rho_0 >= kappa rho_th) counted and the ones that can still be
 //              resolved (rho_0 > rho_th) kept.                                [per run]
-//   loop     : S_gal = estimator of P_k = S_k Q_k 2^-96 (running mean / running median /
+//   loop     : S_gal = estimator of P_k = S_k Q_k 2^-64 (running mean / running median /
 //              median then mean, Eqs. running mean, running median); rho of each kept
 //              candidate against S_instr + S_gal (Eqs. SNR inner product, inner product);
 //              sources with rho > rho_th removed from the spectrum exactly; loop control
 //              on the device.
 //
-// No floating-point atomics: the spectrum is an integer (units of 2^-96 S_instr,k per bin),
+// No floating-point atomics: the spectrum is an integer (units of 2^-64 S_instr,k per bin),
 // so deposits and removals commute and every run gives the same bits.  GB300 runs FP64 at
 // 1/58 of the FP32 rate, so per-iteration work avoids FP64: medians select on the integer
 // bits of the doubles, window sums are integer, and the SNR test is screened in FP32 with
@@ -48,7 +48,8 @@ namespace gbsub {
 // launch behind it (a run over 3e7 sources 1257 -> 1232 us, over 1e7 with the mean 481 -> 473).
 // With more items the waiting CTAs would hold room that other contexts' kernels could use: 64
 // runs at once took 12.7 ms with this rule and without it, 14.7 ms when every kernel called it
-// first.
+// first.  Two kernels call it at once whatever their work: k_begin, whose successor is one CTA per
+// SM at the most, and k_snr_resolve, whose successor is one CTA.
 __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -183,8 +184,9 @@ __device__ __noinline__ U128 tree_units(const unsigned long long* __restrict__ a
   return r;
 }
 
-// Estimator input of bin j: P_j = S_j Q_j 2^-64 (kSpec; flags: RunState::spec), or x[j].  The kernels that read it are built for each kind of input: an
-// estimate of a plain array keeps none of the spectrum's registers.
+// Estimator input of bin j: P_j = S_j Q_j 2^-64 (kSpec; flags: RunState::spec), or x[j].  The
+// kernels that read it are built for each kind of input: an estimate of a plain array keeps none of
+// the spectrum's registers.
 template <bool kSpec>
 __device__ __forceinline__ double spec_value(const SpecIn& in, long long j, int flags) {
   if (kSpec) {
@@ -469,14 +471,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity) {
 // stage takes the step after the next.  No barrier between warps runs in the steady state, so a
 // warp that meets a slow source delays no other.
 //
-// Bound: before, the requests from the SMs to L2 (two 64-bit atomics and most of a table gather
-// per source, one request a cycle and SM: 0.3 of 0.47 ms for 3e7 sources), and instruction issue.
-// Measured, catalog pass with its memsets and fold, start -> now: 3e7 sources 470 -> 343 us, 1e7
-// 170 -> 127, 1e6 45 -> 43.  What was tried on the way (3e7): steps in runs from a global counter
-// 376 (the counter gives out a number every 1.7 ns, and long runs lose the locality of the
-// stream: 450 at two runs a warp); 24 warps 351, 28 391, 16 with four sources a lane 371; the
-// table entries of the first bins in shared memory too, no gain; gathers issued a step ahead, no
-// gain.
+// Bound: latency.  With 20 warps on an SM (issue active 56%, L1 and L2 57 and 60% of their rates)
+// the warps wait for their gathers and for the results of dependent instructions.  Two reductions
+// and most of a table gather per source go to L2 beyond the first bins, and their number counts:
+// 3e7 sources took 470 us with all of them in L2, 268 with none.  With the rings and the first bins
+// in shared memory, set-up and fold included: 3e7 sources 470 -> 343 us, 1e7 170 -> 127, 1e6 45 ->
+// 43.  Other layouts at 3e7: steps in runs from a global counter 376 (it gives out a number every
+// 1.7 ns, and long runs lose the locality of the stream: 450 at two runs a warp); 24 warps 351, 28
+// 391, 16 with four sources a lane 371.
 constexpr int kPreWarps = 20;
 constexpr int kPrepassThreads = kPreWarps * 32;
 constexpr int kPrePer = 2;                                    // sources per lane per step
@@ -749,8 +751,9 @@ __device__ __forceinline__ void hot_add(const HotBins& h, int j, unsigned c0, un
 // One source of the catalog pass in two steps, so that the table gathers of a lane's sources
 // are under way together.
 //
-// Bound: instruction issue.  The pass reads 24 bytes a source (0.1 ms for 3e7 at the measured
-// HBM rate) and used to issue 301 instructions per 32 sources.  What is left out here: tests
+// 247 instructions per 32 sources (301 before; in the pass over a generated catalog they add to the
+// generator's, which is bound by instruction issue; the pass over a stored one waits more than it
+// issues).  What is left out here: tests
 // that the rare paths repeat (finite inputs, the range of q, both thresholds: a source is
 // handed to q_single only when its exponent and top 20 bits say that it may pass the lower
 // one, or when it reaches the third word), 64-bit shifts by zero-extended halves, and the
@@ -1045,8 +1048,8 @@ __global__ void __launch_bounds__(kPrepassThreads, 1)
 //
 // Bound: instruction issue.  An attempt at a source's Gamma variate is refused one time in four;
 // with a loop per lane a warp went on until its last lane was done, 3.5 attempts and half its
-// lanes idle (1 377 instructions per 32 sources; 1 034 now, 3e7 sources 1 340 -> 940 us).  So a warp keeps refused sources in a queue and
-// tries 32 of them at a time, and sources with their variate in another (for the paper's
+// lanes idle (1 377 instructions per 32 sources, 1 034 with the queues; 3e7 sources 1 340 -> 940
+// us).  So a warp keeps refused sources in a queue and tries 32 of them at a time, and sources with their variate in another (for the paper's
 // population one for each way through the incomplete gamma function), from which it computes
 // the rest 32 at a time.  The order of the sources changes nothing: deposits are integers.
 constexpr int kGenThreads = 256;
@@ -1979,8 +1982,8 @@ __device__ __forceinline__ void sts_u16(uint32_t addr, unsigned v) {
 
 // Wavelet matrix of the permutation seq0 (M elements, every warp owning exactly WPW words of a
 // level; the caller fills the last words up with ranks beyond the span's): each level loads the
-// warp's elements once, all of them before the first ballot, and the ballots serve both the count and the stable partition into the other buffer.
-// Level l stores its words in rk[l ws ..] (bits in the low half, ones of the earlier words
+// warp's elements once, all of them before the first ballot, and the ballots serve both the count
+// and the stable partition into the other buffer.  Level l stores its words in rk[l ws ..] (bits in the low half, ones of the earlier words
 // in the high half) and its number of zeros in zeros[l].  seq0 and seq1 are both
 // overwritten.
 template <int WPW>
@@ -2317,8 +2320,8 @@ __global__ void __launch_bounds__(512, 2) k_median_wm(
 
 // Two outputs per thread: a few tiles' latency is what a late iteration waits for.  At most 512
 // threads, so that two CTAs share an SM (W = 2000, every tile: 212 us, 228 with 1024).
-// Where tiles are many (all: every one of them; shared: other contexts' tiles too) their rate
-// counts, and four CTAs of 256 threads cover each other's barriers better than two of 512, as long
+// Where tiles are many (all: every one of them; shared: a grid divisor above 1 says that other
+// contexts run beside) their rate counts, and four CTAs of 256 threads cover each other's barriers better than two of 512, as long
 // as the build stays unrolled (eight words per warp: chunks of up to 1024).  W = 1000, 1.25e6 bins:
 // an estimate of every tile 213 us (220.5 with 512 threads), 64 runs at once 11.95 ms (12.2); a
 // run by itself over 3e7 sources, with its late iterations, 1262 us (1209), so it keeps 512.
@@ -2372,7 +2375,7 @@ __device__ __forceinline__ int sigma_from_max(u64 maxbits) {
 //
 // Bound: latency of one chunk (a maximum, a scan, two barriers each), so what counts is how
 // many chunks an SM works on at once.  With one value per thread a chunk of 1024 bins took the
-// SM alone (1024 threads of 56 registers).  1.25e6 bins, W = 1000, start -> now: 31 -> 13 us from
+// SM alone (1024 threads of 56 registers).  1.25e6 bins, W = 1000: 31 -> 13 us from
 // an array, 33 -> 28 us from the spectrum (W = 2000); running mean of 312 422 bins with its
 // window means 29.7 -> 18.4 us.
 template <bool kSpec, int kPer>
@@ -2580,7 +2583,7 @@ __device__ __forceinline__ double part_sum(const double* __restrict__ x, int a, 
 // Window means, a CTA per kMeanThreads outputs of a chunk and an output per thread: an output is
 // a dozen independent loads and a few dozen instructions, so small CTAs keep an SM's loads in
 // flight (with a chunk's 1024 outputs per CTA of 40 registers an SM held one, and waited for
-// each), and bins are 32-bit numbers.  1.25e6 bins, start -> now: 26 -> 19 us; a late
+// each), and bins are 32-bit numbers.  1.25e6 bins: 26 -> 19 us; a late
 // iteration's few chunks 8 -> 6 us.
 // kTree: the run's S_gal, whose node sums h are kept up to date.
 constexpr int kMeanThreads = 256;
@@ -2996,7 +2999,8 @@ constexpr int kOpenMax = 16;     // sweeps a CTA sets aside
 constexpr int kOpenBins = 4096;  // of more bins than this
 
 __global__ void __launch_bounds__(256) k_snr_resolve(
-    const __grid_constant__ Cands cd, const __grid_constant__ Grid g, const __grid_constant__ Tables tb, const double* Sg, const float* inv_f,
+    const __grid_constant__ Cands cd, const __grid_constant__ Grid g,
+    const __grid_constant__ Tables tb, const double* Sg, const float* inv_f,
     double th2, double rtol, int mode, unsigned char* __restrict__ resolved,
     unsigned long long* __restrict__ acc, RunState* rs, Dirty d, int Kc, int sg_radius) {
   // the loop state, read by one thread per CTA (every thread of the grid loading the same

@@ -86,9 +86,10 @@ struct Grid {
   double T, T2, t5;      // T_obs, T_obs^2, T_obs / 5
   long long k_lo;        // first DFT index in band
   long long nb;          // bins in band
-  // T_obs = (tq 2^32 + tr) 2^(etq - 32), tq in [2^31, 2^32) (source_bin); ebin - e is the count
+  // T_obs = (tq + tr 2^-32) 2^(ex - 32), tq in [2^31, 2^32) (source_bin); ebin - e is the count
   // of fraction bits beyond 23 of f tq for a mantissa exponent e of f (negative for every e
-  // when T_obs is so extreme that f's exponent could leave the normal range)
+  // when T_obs is so extreme that f's exponent could leave the normal range, and for a band from
+  // bin 2^30 on)
   unsigned tq, tr;
   int ebin;
   float T2f;             // T_obs^2 in FP32
@@ -115,13 +116,13 @@ struct SmoothPlan {
   double key_scale;  // power of two the values are scaled by before rounding to FP32
   // CTAs resident at once (plan_grids); res_median_all: where every tile is computed
   int res_sort, res_median, res_median_all, res_prefix, res_mean;
-  int shared;     // 1: the GPU is shared with other contexts' runs (SUB_TUNE_GRID_DIV)
+  int shared;     // 1: a grid divisor above 1 (sub_set_grid_div, SUB_TUNE_GRID_DIV)
   int sort_e;     // elements per sorting thread (2, 4, 8), 0: chosen from kpad
   int median_th;  // threads per median tile (multiple of 32, <= 512), 0: chosen from Kc
   int median_mp;  // positions of a median tile filled up to whole words per warp (at launch)
 };
 
-// Source of an estimator's input: the run's fixed-point spectrum (P_k = S_k Q_k 2^-96) or
+// Source of an estimator's input: the run's fixed-point spectrum (P_k = S_k Q_k 2^-64) or
 // a plain array of doubles.
 struct SpecIn {
   const unsigned long long* acc;  // 4 words per bin (three used), or null
