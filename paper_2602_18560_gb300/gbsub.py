@@ -436,7 +436,7 @@ def sub_device_bytes(ctx) -> int:
 
 def sub_snr_check(ctx):
     """rho^2 of every kept candidate against the last run's S_gal, two ways: the FP32 screen
-    and FP64 in the oracle's order.  Returns dict of numpy arrays src, screen, exact, nbins."""
+    as the run evaluates it and FP64 in the oracle's order.  Returns dict of numpy arrays src, screen, exact, nbins."""
     n = ctypes.c_int64()
     _check(ctx, lib().sub_snr_check(ctx, None, None, None, None, 0, ctypes.byref(n)),
            allow=(EINVAL,))
