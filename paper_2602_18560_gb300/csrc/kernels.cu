@@ -751,7 +751,7 @@ __device__ __forceinline__ void hot_add(const HotBins& h, int j, unsigned c0, un
 // One source of the catalog pass in two steps, so that the table gathers of a lane's sources
 // are under way together.
 //
-// 247 instructions per 32 sources (301 before; in the pass over a generated catalog they add to the
+// Some 240 instructions per 32 sources (301 before; in the pass over a generated catalog they add to the
 // generator's, which is bound by instruction issue; the pass over a stored one waits more than it
 // issues).  What is left out here: tests
 // that the rare paths repeat (finite inputs, the range of q, both thresholds: a source is
